@@ -25,7 +25,10 @@
 // index sits in device memory, so one captured graph serves every step.
 #include <climits>
 
+#include <cooperative_groups.h>
+
 #include "fcd_adjoint.cuh"
+#include "fcd_cross.cuh"
 
 namespace fcd {
 
@@ -375,7 +378,7 @@ __global__ void set_slot_kernel(int *slot, int v) { *slot = v; }
 __global__ void dec_slot_kernel(int *slot) { *slot -= 1; }
 
 // ---------------------------------------------------------------- seeds
-constexpr int SOB = 1024;
+constexpr int SOB = 256;
 
 struct Cross {
     int first, last;
@@ -383,19 +386,20 @@ struct Cross {
     double alo, blo, ahi, bhi;  // the values either side of each crossing
 };
 
-__device__ __forceinline__ void cross_step(Cross &c, int i, double a, double b) {
-    if (a < 0.5 && b >= 0.5 && c.first == -2) {
-        c.first = i;
-        c.lo = double(i) + (0.5 - a) / (b - a);
-        c.alo = a;
-        c.blo = b;
-    }
-    if (a >= 0.5 && b < 0.5) {
-        c.last = i;
-        c.hi = double(i) + (a - 0.5) / (a - b);
-        c.ahi = a;
-        c.bhi = b;
-    }
+// the crossing pair at steps first, last of the n values at(i), 0 beyond them
+template <typename F>
+__device__ __forceinline__ Cross cross_at(int first, int last, int n, F at) {
+    auto v = [&](int i) { return i < 0 || i >= n ? 0.0 : at(i); };
+    Cross c;
+    c.first = first;
+    c.last = last;
+    c.alo = v(first);
+    c.blo = v(first + 1);
+    c.ahi = v(last);
+    c.bhi = v(last + 1);
+    c.lo = double(first) + (0.5 - c.alo) / (c.blo - c.alo);
+    c.hi = double(last) + (c.ahi - 0.5) / (c.ahi - c.bhi);
+    return c;
 }
 
 // d lo / d(a, b) and d hi / d(a, b) of a crossing pair
@@ -411,90 +415,122 @@ __device__ __forceinline__ double indicator(const double *phi1, const double *ph
     return cl01(phi1[n]) + cl01(phi2[n]);
 }
 
+// Per column: the vertical extent of the shell indicator, its centre-line value
+// and the column's part of the overlap; a cluster per 32 columns, a run of rows
+// a warp (see obs_columns; one block over all columns took about 500 us on
+// 800 x 100).
+constexpr int ARUNS = 8;
+__global__ void __launch_bounds__(32 * ARUNS) adj_seed_columns(int nx, int ny, int pitch, const double *phi1,
+                                                               const double *phi2, double *ext, double *cl,
+                                                               double *ovl) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ double part[ARUNS][32], bsum[32];
+    __shared__ RunCross cross[ARUNS][32], bcross[32];
+    const int lane = threadIdx.x, run = threadIdx.y, x = blockIdx.x * 32 + lane, CH = (int)cluster.num_blocks();
+    const int rows = (ny + CH * ARUNS - 1) / (CH * ARUNS);
+    const int y0 = (blockIdx.y * ARUNS + run) * rows, y1 = min(ny, y0 + rows);
+    double o = 0.0;
+    RunCross cr;
+    cr.clear();
+    if (x < nx)
+        for (int y = y0; y < y1; y++) {
+            const long long n = (long long)y * pitch + x;
+            const double p1 = phi1[n], p2 = phi2[n];
+            o += p1 * (1.0 - p1 - p2);
+            cr.add(y, cl01(p1) + cl01(p2));
+        }
+    part[run][lane] = o;
+    cross[run][lane] = cr;
+    __syncthreads();
+    if (run == 0) {  // the block's runs in row order, then (below) the cluster's blocks
+        RunCross all;
+        all.clear();
+        for (int r = 0; r < ARUNS; r++) all.join((blockIdx.y * ARUNS + r) * rows, cross[r][lane]);
+        bcross[lane] = all;
+    } else if (run == 1) {
+        double s = 0.0;
+        for (int r = 0; r < ARUNS; r++) s += part[r][lane];
+        bsum[lane] = s;
+    }
+    cluster.sync();
+    if (cluster.block_rank() == 0 && x < nx) {
+        auto at = [&](int y) { return indicator(phi1, phi2, (long long)y * pitch + x); };
+        if (run == 0) {
+            RunCross all;
+            all.clear();
+            for (int q = 0; q < CH; q++) all.join(q * ARUNS * rows, *cluster.map_shared_rank(&bcross[lane], q));
+            all.close(ny);
+            ext[x] = all.found() ? cross_extent<double>(all.first, all.last, ny, at) : 0.0;
+        } else if (run == 1) {
+            cl[x] = (ny & 1) ? at(ny / 2) : 0.5 * (at(ny / 2 - 1) + at(ny / 2));
+        } else if (run == 2) {
+            double s = 0.0;
+            for (int q = 0; q < CH; q++) s += *cluster.map_shared_rank(&bsum[lane], q);
+            ovl[x] = s;
+        }
+    }
+    cluster.sync();  // the other blocks' shared memory is read until here
+}
+
 // Adjoint of J = wT T_o + wO sum_nodes phi_1 phi_3 (unclamped) at the current
 // state: T_o (Eq. 42) as the plain observables measure it (l_y the largest
 // vertical 1/2-extent of phi^_1 + phi^_2, first column among equal maxima; l_x
 // from the centre-line crossings in the frame that starts at column xcut).
 // Writes the T_o part into pb (zeroed before); the overlap part is added by
-// adj_seed_bcast.
+// adj_seed_bcast. One block over the columns.
 __global__ void __launch_bounds__(SOB) adj_seed_obs_kernel(int nx, int ny, int pitch, long long ps,
                                                            const double *phi1, const double *phi2,
-                                                           const ObsOut *prim, double wT, double *ext,
-                                                           double *cl, double *pb, AdjOut *out) {
-    __shared__ double sv[SOB];
-    __shared__ int si[SOB];
-    __shared__ double sred[SOB / 32];
-    const int t = threadIdx.x;
-    double ovl = 0.0;
-    for (int x = t; x < nx; x += SOB) {
-        Cross c{-2, -2, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        double a = 0.0, mid = 0.0;
-        for (int i = -1; i < ny; i++) {
-            double b = 0.0;
-            if (i + 1 < ny) {
-                const long long n = (long long)(i + 1) * pitch + x;
-                b = indicator(phi1, phi2, n);
-                const double p1 = phi1[n], p2 = phi2[n];
-                ovl += p1 * (1.0 - p1 - p2);
-                const int yy = i + 1;
-                if ((ny & 1) ? yy == ny / 2 : (yy == ny / 2 - 1 || yy == ny / 2)) mid += b;
-            }
-            cross_step(c, i, a, b);
-            a = b;
-        }
-        ext[x] = (c.first != -2 && c.last != -2) ? c.hi - c.lo : 0.0;
-        cl[x] = (ny & 1) ? mid : 0.5 * mid;
-    }
-    __syncthreads();
-    {
-        double best = -1.0;
-        int bi = INT_MAX;
-        for (int x = t; x < nx; x += SOB)
-            if (ext[x] > best) { best = ext[x]; bi = x; }
-        sv[t] = best;
-        si[t] = bi;
-        __syncthreads();
-        for (int s = SOB / 2; s > 0; s >>= 1) {
-            if (t < s && (sv[t + s] > sv[t] || (sv[t + s] == sv[t] && si[t + s] < si[t]))) {
-                sv[t] = sv[t + s];
-                si[t] = si[t + s];
-            }
-            __syncthreads();
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) ovl += __shfl_down_sync(0xffffffffu, ovl, o);
-    if ((t & 31) == 0) sred[t / 32] = ovl;
-    __syncthreads();
-    if (t != 0) return;
-    double tot = 0.0;
-    for (int w = 0; w < SOB / 32; w++) tot += sred[w];
-    // l_y again at the chosen column, keeping the crossing rows
-    const int xs = si[0];
-    Cross cy_{-2, -2, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    if (xs < nx) {
-        double a = 0.0;
-        for (int i = -1; i < ny; i++) {
-            const double b = i + 1 < ny ? indicator(phi1, phi2, (long long)(i + 1) * pitch + xs) : 0.0;
-            cross_step(cy_, i, a, b);
-            a = b;
-        }
-    }
-    const bool hy = xs < nx && cy_.first != -2 && cy_.last != -2;
-    const double ly = hy ? cy_.hi - cy_.lo : 0.0;
-    // l_x along the centre line, unwrapped from column xcut
-    const int xcut = prim->xcut;
+                                                           const ObsOut *prim, double wT, const double *ext,
+                                                           const double *cl, const double *ovl, double *pb,
+                                                           AdjOut *out) {
+    const int t = threadIdx.x, xcut = prim->xcut;
     auto colx = [&](int j) { int xx = xcut + j; return xx >= nx ? xx - nx : xx; };
-    Cross cx_{-2, -2, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int i = -1; i < nx; i++) {
-        const double a = i < 0 ? 0.0 : cl[colx(i)], b = i + 1 < nx ? cl[colx(i + 1)] : 0.0;
-        cross_step(cx_, i, a, b);
+    auto clv = [&](int j) { return cl[colx(j)]; };
+    long long best[1] = {-1};  // extents are >= 0
+    double tot[1] = {0.0};
+    for (int x = t; x < nx; x += SOB) {
+        if (ext[x] >= 0.0) best[0] = max(best[0], order_bits(ext[x]));
+        tot[0] += ovl[x];
     }
-    const bool hx = cx_.first != -2 && cx_.last != -2;
-    const double lx = hx ? cx_.hi - cx_.lo : 0.0;
+    block_reduce<SOB>(best, [](long long a, long long b) { return max(a, b); });
+    block_reduce<SOB>(tot, [](double a, double b) { return a + b; });
+    // first column of the largest extent; rising step along the centre line
+    int fi[2] = {INT_MAX, INT_MAX}, la[1] = {-3};
+    for (int x = t; x < nx; x += SOB)
+        if (order_bits(ext[x]) == best[0]) fi[0] = min(fi[0], x);
+    for (int i = t - 1; i < nx; i += SOB) {
+        const double a = i < 0 ? 0.0 : clv(i), b = i + 1 < nx ? clv(i + 1) : 0.0;
+        if (a < 0.5 && b >= 0.5) fi[1] = min(fi[1], i);
+        if (a >= 0.5 && b < 0.5) la[0] = max(la[0], i);
+    }
+    auto least = [](int a, int b) { return min(a, b); };
+    auto most = [](int a, int b) { return max(a, b); };
+    block_reduce<SOB>(fi, least);
+    block_reduce<SOB>(la, most);
+    // the crossing rows of that column
+    const int xs = fi[0];
+    int fy[1] = {INT_MAX}, ly_[1] = {-3};
+    if (xs < nx)
+        for (int i = t - 1; i < ny; i += SOB) {
+            const double a = i < 0 ? 0.0 : indicator(phi1, phi2, (long long)i * pitch + xs);
+            const double b = i + 1 < ny ? indicator(phi1, phi2, (long long)(i + 1) * pitch + xs) : 0.0;
+            if (a < 0.5 && b >= 0.5) fy[0] = min(fy[0], i);
+            if (a >= 0.5 && b < 0.5) ly_[0] = max(ly_[0], i);
+        }
+    block_reduce<SOB>(fy, least);
+    block_reduce<SOB>(ly_, most);
+    if (t != 0) return;
+    const bool hy = fy[0] != INT_MAX && ly_[0] != -3, hx = fi[1] != INT_MAX && la[0] != -3;
+    Cross cy_{}, cx_{};
+    if (hy)
+        cy_ = cross_at(fy[0], ly_[0], ny, [&](int i) { return indicator(phi1, phi2, (long long)i * pitch + xs); });
+    if (hx) cx_ = cross_at(fi[1], la[0], nx, clv);
+    const double ly = hy ? cy_.hi - cy_.lo : 0.0, lx = hx ? cx_.hi - cx_.lo : 0.0;
     const double sum = lx + ly;
     const double To = sum > 0.0 ? (ly - lx) / sum : 0.0;
     out->T_o = To;
-    out->overlap = tot;
+    out->overlap = tot[0];
     out->lx = lx;
     out->ly = ly;
     if (!(sum > 0.0) || wT == 0.0) return;
@@ -556,7 +592,7 @@ inline dim3 grid2(int nx, int ny, dim3 b) { return dim3((nx + b.x - 1) / b.x, (n
 
 int adj_collide_blocks(int nx, int ny) { return ((nx + TX - 1) / TX) * ((ny + ATY - 1) / ATY); }
 int adj_kbar_blocks(int nx, int ny) { return ((nx + 31) / 32) * ((ny + 7) / 8); }
-size_t adj_seed_scratch_bytes(int nx) { return 2ull * nx * sizeof(double); }
+size_t adj_seed_scratch_bytes(int nx) { return 3ull * nx * sizeof(double); }
 
 void launch_adj_phase(const Phys<double> &P, const double *seg, const int *slot, long long stride,
                       double *phi1, double *phi2, double *k, cudaStream_t s) {
@@ -597,9 +633,10 @@ void launch_dec_slot(int *slot, cudaStream_t s) { dec_slot_kernel<<<1, 1, 0, s>>
 void launch_adj_seed(const Phys<double> &P, const double *phi1, const double *phi2, const ObsOut *prim,
                      double wT, double wO, void *scratch, double *pb, double *ab, AdjOut *out,
                      cudaStream_t s) {
-    double *ext = static_cast<double *>(scratch), *cl = ext + P.nx;
+    double *ext = static_cast<double *>(scratch), *cl = ext + P.nx, *ovl = cl + P.nx;
     cudaMemsetAsync(pb, 0, 2 * P.ps * sizeof(double), s);
-    adj_seed_obs_kernel<<<1, SOB, 0, s>>>(P.nx, P.ny, P.pitch, P.ps, phi1, phi2, prim, wT, ext, cl, pb, out);
+    launch_columns(adj_seed_columns, ARUNS, P.nx, P.ny, s, P.nx, P.ny, P.pitch, phi1, phi2, ext, cl, ovl);
+    adj_seed_obs_kernel<<<1, SOB, 0, s>>>(P.nx, P.ny, P.pitch, P.ps, phi1, phi2, prim, wT, ext, cl, ovl, pb, out);
     dim3 b(32, 8);
     adj_seed_bcast_kernel<<<grid2(P.nx, P.ny, b), b, 0, s>>>(P, phi1, phi2, pb, wO, ab);
 }

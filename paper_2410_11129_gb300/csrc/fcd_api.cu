@@ -232,7 +232,7 @@ struct Engine : fcd_ctx {
     double *obs_scratch = nullptr;
     ObsOut *obs_out = nullptr;
     MgCtl *h_ctl = nullptr;
-    ObsOut *h_obs = nullptr;
+    ObsPack *h_obs = nullptr;  // pinned; the last kernel of an observation writes it
     SnapHeader *h_snap = nullptr;  // pinned staging of snapshot headers
     unsigned long long *h_brk = nullptr;
     unsigned long long *h_unst = nullptr;
@@ -314,7 +314,7 @@ struct Engine : fcd_ctx {
                         (void *)obs_scratch, (void *)obs_out})
             if (!p) return fail(FCD_ENOMEM, "device allocation failed");
         CK(cudaMallocHost(&h_ctl, sizeof(MgCtl)));
-        CK(cudaMallocHost(&h_obs, sizeof(ObsOut)));
+        CK(cudaMallocHost(&h_obs, sizeof(ObsPack)));
         CK(cudaMallocHost(&h_snap, sizeof(SnapHeader)));
         CK(cudaMallocHost(&h_brk, sizeof(unsigned long long)));
         CK(cudaMallocHost(&h_unst, sizeof(unsigned long long)));
@@ -749,15 +749,14 @@ struct Engine : fcd_ctx {
 
     fcd_status observe(fcd_obs *o) override {
         cudaStream_t s = stream;
-        launch_observe<T>(mode, P, g[cur], obs_scratch, obs_out, s, prm.open_x);
-        host_kernels += 4;
+        launch_observe<T>(mode, P, g[cur], obs_scratch, obs_out, s, prm.open_x, ObsTail{h_obs, brk, unst, ctl});
+        host_kernels += 3;
         CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(h_obs, obs_out, sizeof(ObsOut), cudaMemcpyDeviceToHost, s));
-        CK(cudaMemcpyAsync(h_brk, brk, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-        CK(cudaMemcpyAsync(h_unst, unst, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-        CK(cudaMemcpyAsync(h_ctl, ctl, sizeof(MgCtl), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        const ObsOut &r = *h_obs;
+        const ObsOut &r = h_obs->o;
+        *h_brk = h_obs->brk;
+        *h_unst = h_obs->unst;
+        *h_ctl = h_obs->ctl;
         std::memset(o, 0, sizeof *o);
         o->step = step;
         o->t_star = step * D.u_avg / (2.0 * prm.r2);  // Eq. 38
@@ -1297,17 +1296,14 @@ struct TangentEngine : Engine<double> {
         const fcd_status st = observe(&po);  // primal observables (and the seam column)
         if (st != FCD_OK && st != FCD_ENOCONV) return st;
         cudaStream_t s = stream;
-        launch_tangent_obs(P, static_cast<const double *>(g[cur]), obs_out, tobs, tan_out, s);
-        host_kernels += 1;
+        TanCtls ctls;
+        for (int c = 0; c < NT; c++) ctls.c[c] = mgt[c] ? ctlt[c] : nullptr;
+        launch_tangent_obs(P, static_cast<const double *>(g[cur]), obs_out, tobs, tan_out, ctls, s);
+        host_kernels += 2;
         CK(cudaGetLastError());
         CK(cudaMemcpyAsync(h_tan, tan_out, sizeof(TanOut), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        int nonconv = 0;
-        for (int c = 0; c < NT; c++) {
-            if (!mgt[c]) continue;
-            CK(cudaMemcpy(h_ctl, ctlt[c], sizeof(MgCtl), cudaMemcpyDeviceToHost));
-            nonconv += h_ctl->nonconv_count;
-        }
+        const int nonconv = h_tan->nonconv;
         std::memset(o, 0, sizeof *o);
         o->step = step;
         o->T_o = h_tan->T_o;
@@ -1645,7 +1641,7 @@ struct AdjointEngine : Engine<double> {
         launch_phase<double>(MODE_FP64, P, g[cur], phi1, phi2, nullptr,
                              PhaseCtl{nullptr, 0, 0.0, 0, nullptr, 0, nullptr, nullptr, nullptr}, s);
         launch_adj_seed(P, phi1, phi2, obs_out, wT, wO, seed_scr, pb, ab[0], adj_out, s);
-        host_kernels += 3;
+        host_kernels += 4;
         CK(cudaMemcpyAsync(h_adj, adj_out, sizeof(AdjOut), cudaMemcpyDeviceToHost, s));
         if (state_seed) {  // the caller's dJ/d(f_N, g_N) replaces the seed's planes
             const size_t Nn = (size_t)prm.nx * prm.ny;

@@ -190,10 +190,27 @@ struct ObsOut {
     int nonfinite;
 };
 
+// What the host reads after an observation, gathered by its last kernel in one
+// block of pinned memory; tail.pack == nullptr: nothing is gathered.
+struct ObsPack {
+    ObsOut o;
+    unsigned long long brk, unst;
+    MgCtl ctl;
+};
+struct ObsTail {
+    ObsPack *pack = nullptr;
+    const unsigned long long *brk = nullptr, *unst = nullptr;
+    const MgCtl *ctl = nullptr;
+};
+
 // Tangent observables: values and derivatives along the NT directions.
 struct TanOut {
     double T_o, overlap, lx, ly;
     double dT_o[NT], doverlap[NT], dlx[NT], dly[NT];
+    int nonconv;  // capped tangent solves so far, all directions
+};
+struct TanCtls {
+    const MgCtl *c[NT];  // nullptr: that direction has not been solved
 };
 
 }  // namespace fcd
@@ -354,7 +371,7 @@ void launch_tangent_phase(const Phys<double> &P, const double *g, double *phi1, 
                           double *k, cudaStream_t s);
 size_t tangent_obs_scratch_bytes(int nx);
 void launch_tangent_obs(const Phys<double> &P, const double *g, const ObsOut *prim, void *scratch,
-                        TanOut *out, cudaStream_t s);
+                        TanOut *out, TanCtls ctls, cudaStream_t s);
 
 // adjoint step (FP64, periodic channel). A segment of forward states sits in
 // slots of `stride` doubles (f 9 planes, g 18 planes, psi' 1 plane); *slot is
@@ -440,6 +457,6 @@ constexpr size_t observe_scratch_doubles_of(long long nx, long long ny) {
 size_t observe_scratch_doubles(int nx, int ny);
 template <typename T>
 void launch_observe(int mode, const Phys<T> &P, const void *g, double *scratch, ObsOut *out,
-                    cudaStream_t s, int open_x = 0);
+                    cudaStream_t s, int open_x = 0, ObsTail tail = ObsTail());
 
 }  // namespace fcd

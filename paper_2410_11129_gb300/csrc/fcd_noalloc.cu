@@ -82,7 +82,7 @@ extern "C" fcd_status fcd_observe_populations_noalloc(const double *g, int nx, i
     P.ps = (long long)nx * ny;
     ObsOut *res = reinterpret_cast<ObsOut *>(scratch + observe_scratch_doubles_of(nx, ny));
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    // launch_observe clears the result block before its kernels run; open_x
+    // launch_observe writes the whole result block; open_x
     // selects the open channel's frame (no periodic seam, no wrap in x)
     launch_observe<double>(MODE_FP64, P, g, scratch, res, s, open_x);
     ObsOut r;

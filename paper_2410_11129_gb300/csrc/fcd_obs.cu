@@ -6,33 +6,19 @@
 // repeated calls give identical bits.
 #include <climits>
 
+#include <cooperative_groups.h>
+
+#include "fcd_cross.cuh"
 #include "fcd_internal.cuh"
 
 namespace fcd {
 
-constexpr int COLS = OBS_COLS;  // per-column record: see obs_columns
+constexpr int COLS = OBS_COLS;  // records per column (planes of nx values): see obs_columns
 
 template <int MODE>
 struct StoreO { using type = float; };
 template <>
 struct StoreO<MODE_FP64> { using type = double; };
-
-template <typename T, int MODE>
-__global__ void obs_phi(Phys<T> P, const void *gv, double *phi1, double *phi2, ObsOut *out) {
-    using S = typename StoreO<MODE>::type;
-    const S *g = static_cast<const S *>(gv);
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= P.nx || y >= P.ny) return;
-    const long long n = (long long)y * P.pitch + x, m = (long long)y * P.nx + x;
-    T p1 = T(0), p2 = T(0);
-    for (int a = 0; a < 9; a++) {
-        p1 += T(g[a * P.ps + n]) - g_off<MODE, T>(a);
-        p2 += T(g[(9 + a) * P.ps + n]) - g_off<MODE, T>(a);
-    }
-    phi1[m] = double(p1);
-    phi2[m] = double(p2);
-    if (!(fabs(double(p1)) < 1e300) || !(fabs(double(p2)) < 1e300)) out->nonfinite = 1;
-}
 
 __device__ __forceinline__ double c01(double v) { return v < 0.0 ? 0.0 : (v > 1.0 ? 1.0 : v); }
 
@@ -57,199 +43,243 @@ __global__ void obs_touch(int nx, int ny, const double *phi1, const double *phi2
     }
 }
 
-// First upward and last downward crossing of 1/2 along v[0..n-1] (zero outside).
-struct Cross {
-    int first, last;
-    double lo, hi;
-};
-template <typename F>
-__device__ __forceinline__ Cross crossings(F v, int n) {
-    Cross c{-2, -2, 0.0, 0.0};
-    for (int i = -1; i < n; i++) {
-        const double a = i < 0 ? 0.0 : v(i), b = i + 1 < n ? v(i + 1) : 0.0;
-        if (a < 0.5 && b >= 0.5 && c.first == -2) { c.first = i; c.lo = i + (0.5 - a) / (b - a); }
-        if (a >= 0.5 && b < 0.5) { c.last = i; c.hi = i + (a - 0.5) / (a - b); }
-    }
-    return c;
-}
+// Phase fields and per-column records in one pass: phi_1, phi_2 of every node
+// (for obs_touch), and per column masses (3), sum so, sum si, sum y*so,
+// sum y*si, vertical extents of so and si, centre-line values of so and si, and
+// whether a value is not finite.
+// A cluster takes 32 columns (lane = column, so the 18 population loads are
+// coalesced) and cuts them into CH blocks x RUNS warps of consecutive rows. Each
+// block joins its runs in row order, the first block then the blocks: the
+// result does not depend on scheduling. Bound by FP64 arithmetic, of which an SM does about 2.2
+// operations a clock: with one thread per column walking all the rows (13
+// blocks on 1600 columns) this was about 430 of the 536 us of an observation
+// of the 1600 x 200 FP32 channel, with one block per 32 columns 72 us, with the
+// clusters 29 us (cold caches); the whole call 85 us.
+constexpr int RUNS = 8;  // runs of rows per block (one warp each)
+template <typename T>
+__device__ __forceinline__ bool finite_value(T v) { return fabs(v) < T(1e300); }
+template <>
+__device__ __forceinline__ bool finite_value<float>(float v) { return fabsf(v) < INFINITY; }
 
-// Per column: masses (3), sum so, sum si, sum y*so, sum y*si, vertical extents
-// of so and si, centre-line values of so and si.
-__global__ void obs_columns(int nx, int ny, const double *phi1, const double *phi2, double *col) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= nx) return;
-    double m1 = 0, m2 = 0, m3 = 0, so = 0, si = 0, yso = 0, ysi = 0;
-    for (int y = 0; y < ny; y++) {
-        const double p1 = phi1[(long long)y * nx + x], p2 = phi2[(long long)y * nx + x];
-        m1 += p1;
-        m2 += p2;
-        m3 += 1.0 - p1 - p2;
-        const double i1 = c01(p1), o = i1 + c01(p2);
-        so += o;
-        si += i1;
-        yso += y * o;
-        ysi += y * i1;
-    }
-    auto vo = [&](int y) { return c01(phi1[(long long)y * nx + x]) + c01(phi2[(long long)y * nx + x]); };
-    auto vi = [&](int y) { return c01(phi1[(long long)y * nx + x]); };
-    const Cross co = crossings(vo, ny), ci = crossings(vi, ny);
-    double *c = col + (long long)x * COLS;
-    c[0] = m1; c[1] = m2; c[2] = m3; c[3] = so; c[4] = si; c[5] = yso; c[6] = ysi;
-    c[7] = (co.first != -2 && co.last != -2) ? co.hi - co.lo : 0.0;
-    c[8] = (ci.first != -2 && ci.last != -2) ? ci.hi - ci.lo : 0.0;
-    if (ny & 1) {
-        c[9] = vo(ny / 2);
-        c[10] = vi(ny / 2);
-    } else {
-        c[9] = 0.5 * (vo(ny / 2 - 1) + vo(ny / 2));
-        c[10] = 0.5 * (vi(ny / 2 - 1) + vi(ny / 2));
-    }
-}
-
-constexpr int FIN = 1024;
-
-// Fixed-order block sum of one value per thread.
-__device__ double block_sum(double v, double *sh) {
-    sh[threadIdx.x] = v;
+template <typename T, int MODE>
+__global__ void __launch_bounds__(32 * RUNS) obs_columns(Phys<T> P, const void *gv, double *phi1,
+                                                         double *phi2, double *col, ObsOut *out) {
+    using S = typename StoreO<MODE>::type;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ double part[6][RUNS][32], bsum[6][32];
+    __shared__ RunCross cross[2][RUNS][32], bcross[2][32];
+    __shared__ int bad[32];
+    const S *g = static_cast<const S *>(gv);
+    const int nx = P.nx, ny = P.ny, lane = threadIdx.x, run = threadIdx.y;
+    const int x = blockIdx.x * 32 + lane, CH = (int)cluster.num_blocks();
+    const int rows = (ny + CH * RUNS - 1) / (CH * RUNS);  // per run
+    const int y0 = (blockIdx.y * RUNS + run) * rows, y1 = min(ny, y0 + rows);
+    if (run == 0) bad[lane] = 0;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && run == 0 && lane == 0) out->brk_now = ~0ull;  // obs_touch follows
     __syncthreads();
-    for (int s = FIN / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
-    }
-    const double r = sh[0];
-    __syncthreads();
-    return r;
-}
-__device__ double block_max(double v, double *sh) {
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int s = FIN / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + s]);
-        __syncthreads();
-    }
-    const double r = sh[0];
-    __syncthreads();
-    return r;
-}
-
-// open: the frame starts at the inlet (no periodic seam to cut)
-__global__ void __launch_bounds__(FIN) obs_final(int nx, const double *col, ObsOut *out, int open) {
-    __shared__ double sh[FIN];
-    __shared__ int ish[FIN];
-    const int t = threadIdx.x;
-    const int chunk = (nx + FIN - 1) / FIN, lo = t * chunk, hi = min(nx, lo + chunk);
-    // masses
-    for (int q = 0; q < 3; q++) {
-        double s = 0;
-        for (int x = lo; x < hi; x++) s += col[(long long)x * COLS + q];
-        s = block_sum(s, sh);
-        if (t == 0) out->mass[q] = s;
-    }
-    // emptiest column (first of the minima): the seam for the periodic frame
-    {
-        double best = INFINITY;
-        int bi = nx;
-        for (int x = lo; x < hi; x++) {
-            const double v = col[(long long)x * COLS + 3];
-            if (v < best) { best = v; bi = x; }
-        }
-        sh[t] = best;
-        ish[t] = bi;
-        __syncthreads();
-        for (int s = FIN / 2; s > 0; s >>= 1) {
-            if (t < s) {
-                const double a = sh[t], b = sh[t + s];
-                if (b < a || (b == a && ish[t + s] < ish[t])) { sh[t] = b; ish[t] = ish[t + s]; }
+    double v[6] = {0, 0, 0, 0, 0, 0};
+    RunCross cr[2];
+    cr[0].clear();
+    cr[1].clear();
+    if (x < nx) {
+        for (int y = y0; y < y1; y++) {
+            const long long n = (long long)y * P.pitch + x, m = (long long)y * nx + x;
+            T p1 = T(0), p2 = T(0);
+#pragma unroll
+            for (int a = 0; a < 9; a++) {
+                p1 += T(g[a * P.ps + n]) - g_off<MODE, T>(a);
+                p2 += T(g[(9 + a) * P.ps + n]) - g_off<MODE, T>(a);
             }
-            __syncthreads();
+            const double d1 = double(p1), d2 = double(p2);
+            phi1[m] = d1;
+            phi2[m] = d2;
+            if (!finite_value(p1) || !finite_value(p2)) bad[lane] = 1;
+            const double i1 = double(clamp01(p1)), o = i1 + double(clamp01(p2));
+            v[0] += d1;
+            v[1] += d2;
+            v[2] += o;
+            v[3] += i1;
+            v[4] += y * o;
+            v[5] += y * i1;
+            cr[0].add(y, o);
+            cr[1].add(y, i1);
         }
     }
-    const int xcut = open ? 0 : ish[0];
+#pragma unroll
+    for (int q = 0; q < 6; q++) part[q][run][lane] = v[q];
+    cross[0][run][lane] = cr[0];
+    cross[1][run][lane] = cr[1];
     __syncthreads();
-    if (t == 0) out->xcut = xcut;
-    for (int w = 0; w < 2; w++) {  // 0: shell indicator, 1: core indicator
-        double m = 0, mx = 0, my = 0, ly = 0;
-        for (int x = lo; x < hi; x++) {
-            const double *c = col + (long long)x * COLS;
-            const double xu = x >= xcut ? x : x + nx;
-            m += c[3 + w];
-            mx += xu * c[3 + w];
-            my += c[5 + w];
-            ly = fmax(ly, c[7 + w]);
-        }
-        m = block_sum(m, sh);
-        mx = block_sum(mx, sh);
-        my = block_sum(my, sh);
-        ly = block_max(ly, sh);
-        // centre-line crossings in the unwrapped frame j = 0..nx-1 (x = xcut + j)
-        auto cl = [&](int j) {
-            int x = xcut + j;
-            x = x >= nx ? x - nx : x;
-            return col[(long long)x * COLS + 9 + w];
+    static_assert(RUNS == 8, "warps 0-5 take the sums, 6 and 7 the crossings");
+    if (run < 6) {
+        double s = 0;
+#pragma unroll
+        for (int r = 0; r < RUNS; r++) s += part[run][r][lane];
+        bsum[run][lane] = s;
+    } else {
+        RunCross all;
+        all.clear();
+#pragma unroll
+        for (int r = 0; r < RUNS; r++) all.join((blockIdx.y * RUNS + r) * rows, cross[run - 6][r][lane]);
+        bcross[run - 6][lane] = all;
+    }
+    __threadfence();  // the phase fields are read back by the first block below
+    cluster.sync();
+    if (cluster.block_rank() == 0 && x < nx) {
+        auto at = [&](int w, int y) {
+            const long long m = (long long)y * nx + x;
+            const double p1 = __ldcg(phi1 + m);
+            return w ? c01(p1) : c01(p1) + c01(__ldcg(phi2 + m));
         };
-        int first = INT_MAX, last = -3;
-        double flo = 0, lhi = 0;
-        const int jhi = min(nx, (t + 1) * chunk);
-        for (int i = (t == 0 ? -1 : t * chunk); i < jhi; i++) {
-            const double a = i < 0 ? 0.0 : cl(i), b = i + 1 < nx ? cl(i + 1) : 0.0;
-            if (a < 0.5 && b >= 0.5 && first == INT_MAX) { first = i; flo = i + (0.5 - a) / (b - a); }
-            if (a >= 0.5 && b < 0.5) { last = i; lhi = i + (a - 0.5) / (a - b); }
+        auto total = [&](int q) {
+            double s = 0;
+            for (int r = 0; r < CH; r++) s += *cluster.map_shared_rank(&bsum[q][lane], r);
+            return s;
+        };
+        for (int task = run; task < COLS; task += RUNS) {
+            double r = 0.0;
+            if (task < 2) {
+                r = total(task);
+            } else if (task == 2) {  // phi_3 = 1 - phi_1 - phi_2
+                r = ny - total(0) - total(1);
+            } else if (task < 7) {
+                r = total(task - 1);
+            } else if (task < 9) {
+                const int w = task - 7;
+                RunCross all;
+                all.clear();
+                for (int q = 0; q < CH; q++) all.join(q * RUNS * rows, *cluster.map_shared_rank(&bcross[w][lane], q));
+                all.close(ny);
+                if (all.found()) r = cross_extent<double>(all.first, all.last, ny, [&](int y) { return at(w, y); });
+            } else if (task < 11) {
+                const int w = task - 9;
+                r = (ny & 1) ? at(w, ny / 2) : 0.5 * (at(w, ny / 2 - 1) + at(w, ny / 2));
+            } else {
+                for (int q = 0; q < CH; q++)
+                    if (*cluster.map_shared_rank(&bad[lane], q)) r = 1.0;
+            }
+            col[(long long)task * nx + x] = r;
         }
-        // smallest first crossing and largest last crossing over the threads
-        ish[t] = first;
-        sh[t] = flo;
-        __syncthreads();
-        for (int s = FIN / 2; s > 0; s >>= 1) {
-            if (t < s && ish[t + s] < ish[t]) { ish[t] = ish[t + s]; sh[t] = sh[t + s]; }
-            __syncthreads();
+    }
+    cluster.sync();  // the other blocks' shared memory is read until here
+}
+
+constexpr int FIN = 512;
+
+// open: the frame starts at the inlet (no periodic seam to cut). pack: the
+// result and the context's records gathered for the host (nullptr: none).
+__global__ void __launch_bounds__(FIN) obs_final(int nx, const double *col, ObsOut *out, int open,
+                                                 ObsTail tail) {
+    const int t = threadIdx.x;
+    auto add = [](double a, double b) { return a + b; };
+    // masses, and whether any column holds a value that is not finite
+    double ms[3] = {0, 0, 0};
+    long long ends[1] = {LLONG_MAX};
+    int flag[1] = {0};
+    auto c = [&](int q, int x) { return col[(long long)q * nx + x]; };
+#pragma unroll 4
+    for (int x = t; x < nx; x += FIN) {
+        for (int q = 0; q < 3; q++) ms[q] += c(q, x);
+        const double so = c(3, x);
+        if (so == so) ends[0] = min(ends[0], order_bits(so));
+        flag[0] |= c(11, x) != 0.0;
+    }
+    auto least = [](auto a, auto b) { return min(a, b); };
+    auto most = [](auto a, auto b) { return max(a, b); };
+    block_reduce<FIN>(ms, add);
+    block_reduce<FIN>(flag, most);
+    // emptiest column (first of the minima): the seam for the periodic frame
+    block_reduce<FIN>(ends, least);
+    int xc[1] = {nx};
+    for (int x = t; x < nx; x += FIN)
+        if (order_bits(c(3, x)) == ends[0]) xc[0] = min(xc[0], x);
+    block_reduce<FIN>(xc, least);
+    const int xcut = open || xc[0] >= nx ? 0 : xc[0];
+    double mo[6] = {0, 0, 0, 0, 0, 0};  // mass, x and y moments of the two indicators
+    long long ly[2] = {0, 0};
+    int first[2] = {INT_MAX, INT_MAX}, last[2] = {-3, -3};
+#pragma unroll 4
+    for (int x = t; x < nx; x += FIN) {
+        const double xu = x >= xcut ? x : x + nx;
+        for (int w = 0; w < 2; w++) {
+            const double s = c(3 + w, x), l = c(7 + w, x);
+            mo[3 * w] += s;
+            mo[3 * w + 1] += xu * s;
+            mo[3 * w + 2] += c(5 + w, x);
+            if (l > 0.0) ly[w] = max(ly[w], order_bits(l));
         }
-        const int gfirst = ish[0];
-        const double glo = sh[0];
-        __syncthreads();
-        ish[t] = last;
-        sh[t] = lhi;
-        __syncthreads();
-        for (int s = FIN / 2; s > 0; s >>= 1) {
-            if (t < s && ish[t + s] > ish[t]) { ish[t] = ish[t + s]; sh[t] = sh[t + s]; }
-            __syncthreads();
+    }
+    block_reduce<FIN>(mo, add);
+    block_reduce<FIN>(ly, most);
+    // centre-line crossings in the unwrapped frame j = 0..nx-1 (x = xcut + j), 0 beyond it:
+    // the smallest upward and the largest downward one
+    auto cl = [&](int w, int j) {
+        if (j < 0 || j >= nx) return 0.0;
+        const int x = xcut + j;
+        return c(9 + w, x >= nx ? x - nx : x);
+    };
+#pragma unroll 4
+    for (int i = t - 1; i < nx; i += FIN)
+        for (int w = 0; w < 2; w++) {
+            const double a = cl(w, i), b = cl(w, i + 1);
+            if (a < 0.5 && b >= 0.5) first[w] = min(first[w], i);
+            if (a >= 0.5 && b < 0.5) last[w] = max(last[w], i);
         }
-        const int glast = ish[0];
-        const double ghi = sh[0];
-        __syncthreads();
-        if (t == 0) {
-            const double lx = (gfirst != INT_MAX && glast != -3) ? ghi - glo : 0.0;
-            const double cxv = m > 0.0 ? fmod(mx / m, (double)nx) : 0.0;
-            const double cyv = m > 0.0 ? my / m : 0.0;
-            if (w == 0) { out->xc_shell = cxv; out->yc_shell = cyv; out->lx_o = lx; out->ly_o = ly; }
-            else { out->xc_core = cxv; out->yc_core = cyv; out->lx_i = lx; out->ly_i = ly; }
-        }
+    block_reduce<FIN>(first, least);
+    block_reduce<FIN>(last, most);
+    if (t != 0) return;
+    ObsOut r;
+    for (int q = 0; q < 3; q++) r.mass[q] = ms[q];
+    double lx[2], xm[2], ym[2];
+    for (int w = 0; w < 2; w++) {
+        lx[w] = 0.0;
+        if (first[w] != INT_MAX && last[w] != -3)
+            lx[w] = cross_extent<double>(first[w], last[w], nx, [&](int j) { return cl(w, j); });
+        xm[w] = mo[3 * w] > 0.0 ? fmod(mo[3 * w + 1] / mo[3 * w], (double)nx) : 0.0;
+        ym[w] = mo[3 * w] > 0.0 ? mo[3 * w + 2] / mo[3 * w] : 0.0;
+    }
+    r.xc_shell = xm[0];
+    r.yc_shell = ym[0];
+    r.lx_o = lx[0];
+    r.ly_o = __longlong_as_double(ly[0]);
+    r.xc_core = xm[1];
+    r.yc_core = ym[1];
+    r.lx_i = lx[1];
+    r.ly_i = __longlong_as_double(ly[1]);
+    r.brk_now = out->brk_now;
+    r.xcut = xcut;
+    r.nonfinite = flag[0];
+    *out = r;
+    if (tail.pack) {
+        tail.pack->o = r;
+        tail.pack->brk = *tail.brk;
+        tail.pack->unst = *tail.unst;
+        tail.pack->ctl = *tail.ctl;
     }
 }
 
 template <typename T>
 void launch_observe(int mode, const Phys<T> &P, const void *g, double *scratch, ObsOut *out,
-                    cudaStream_t s, int open_x) {
+                    cudaStream_t s, int open_x, ObsTail tail) {
     const long long N = (long long)P.nx * P.ny;
     double *phi1 = scratch, *phi2 = scratch + N, *col = scratch + 2 * N;
-    cudaMemsetAsync(out, 0, sizeof(ObsOut), s);
-    cudaMemsetAsync(&out->brk_now, 0xff, sizeof(unsigned long long), s);
-    dim3 b(32, 8), gr((P.nx + 31) / 32, (P.ny + 7) / 8);
     if constexpr (sizeof(T) == 8) {
-        obs_phi<T, MODE_FP64><<<gr, b, 0, s>>>(P, g, phi1, phi2, out);
+        launch_columns(obs_columns<T, MODE_FP64>, RUNS, P.nx, P.ny, s, P, g, phi1, phi2, col, out);
     } else {
-        if (mode == MODE_FP32) obs_phi<T, MODE_FP32><<<gr, b, 0, s>>>(P, g, phi1, phi2, out);
-        else obs_phi<T, MODE_FP32_OFFSET><<<gr, b, 0, s>>>(P, g, phi1, phi2, out);
+        if (mode == MODE_FP32) launch_columns(obs_columns<T, MODE_FP32>, RUNS, P.nx, P.ny, s, P, g, phi1, phi2, col, out);
+        else launch_columns(obs_columns<T, MODE_FP32_OFFSET>, RUNS, P.nx, P.ny, s, P, g, phi1, phi2, col, out);
     }
+    dim3 b(32, 8), gr((P.nx + 31) / 32, (P.ny + 7) / 8);
     obs_touch<<<gr, b, 0, s>>>(P.nx, P.ny, phi1, phi2, out, open_x);
-    obs_columns<<<(P.nx + 127) / 128, 128, 0, s>>>(P.nx, P.ny, phi1, phi2, col);
-    obs_final<<<1, FIN, 0, s>>>(P.nx, col, out, open_x);
+    obs_final<<<1, FIN, 0, s>>>(P.nx, col, out, open_x, tail);
 }
 
 size_t observe_scratch_doubles(int nx, int ny) { return observe_scratch_doubles_of(nx, ny); }
 
 template void launch_observe<float>(int, const Phys<float> &, const void *, double *, ObsOut *,
-                                    cudaStream_t, int);
+                                    cudaStream_t, int, ObsTail);
 template void launch_observe<double>(int, const Phys<double> &, const void *, double *,
-                                     ObsOut *, cudaStream_t, int);
+                                     ObsOut *, cudaStream_t, int, ObsTail);
 
 }  // namespace fcd

@@ -11,6 +11,9 @@
 // (np * c + q) planes from the base.
 #include <climits>
 
+#include <cooperative_groups.h>
+
+#include "fcd_cross.cuh"
 #include "fcd_internal.cuh"
 
 namespace fcd {
@@ -48,120 +51,125 @@ __global__ void __launch_bounds__(256) tangent_phase_kernel(Phys<double> P, cons
     }
 }
 
-constexpr int TOB = 1024;
-
-// First upward and last downward crossing of 1/2 (zero outside the range),
-// with derivatives: lo = i + (1/2 - a)/(b - a), hi = i + (a - 1/2)/(a - b).
-struct DCross {
-    int first, last;
-    DualT lo, hi;
-};
-
-__device__ __forceinline__ void cross_step(DCross &c, int i, const DualT &a, const DualT &b) {
-    if (a < 0.5 && b >= 0.5 && c.first == -2) {
-        c.first = i;
-        c.lo = double(i) + (0.5 - a) / (b - a);
-    }
-    if (a >= 0.5 && b < 0.5) {
-        c.last = i;
-        c.hi = double(i) + (a - 0.5) / (a - b);
-    }
-}
-
 __device__ __forceinline__ DualT node_phi(const double *g, int base, long long ps, long long n) {
     DualT p(0.0);
+#pragma unroll
     for (int a = 0; a < 9; a++) p += ld_copies(g, base + a, 18, ps, n);
     return p;
 }
 
-// One block. Per column: the vertical 1/2-extent of the shell indicator
-// phi^_1 + phi^_2 and its centre-line value; then l_y = the largest extent
-// (first column among equal maxima), l_x from the centre-line crossings in the
-// frame that starts at the emptiest column found by the plain observables, and
-// T_o = (l_y - l_x) / (l_y + l_x).
-__global__ void __launch_bounds__(TOB) tangent_obs_kernel(int nx, int ny, int pitch, long long ps,
-                                                          const double *g, const ObsOut *prim,
-                                                          DualT *ext, DualT *cl, TanOut *out) {
-    __shared__ double sv[TOB];
-    __shared__ int si[TOB];
-    __shared__ DualT sred[TOB / 32];
-    const int t = threadIdx.x;
-    DualT ovl(0.0);
-    for (int x = t; x < nx; x += TOB) {
-        DCross c{-2, -2, DualT(0.0), DualT(0.0)};
-        DualT a(0.0), mid(0.0);
-        for (int i = -1; i < ny; i++) {
-            DualT b(0.0);
-            if (i + 1 < ny) {
-                const long long n = (long long)(i + 1) * pitch + x;
-                const DualT p1 = node_phi(g, 0, ps, n), p2 = node_phi(g, 9, ps, n);
-                b = clamp01(p1) + clamp01(p2);
-                ovl += p1 * (DualT(1.0) - p1 - p2);
-                const int y = i + 1;
-                if ((ny & 1) ? y == ny / 2 : (y == ny / 2 - 1 || y == ny / 2)) mid += b;
-            }
-            cross_step(c, i, a, b);
-            a = b;
+// Per column: the vertical 1/2-extent of the shell indicator phi^_1 + phi^_2,
+// its centre-line value, and the column's part of the overlap; a cluster per 32
+// columns, a run of rows per warp (see obs_columns). Bound by FP64 arithmetic
+// (about 115 operations a node for the 90 planes of g): one block walking the
+// columns of the 800 x 100 channel took 3.4 of the 3.5 ms of a tangent
+// observation, one block per 32 columns 138 us, the clusters 63 us (cold caches).
+constexpr int TRUNS = 8;
+__global__ void __launch_bounds__(32 * TRUNS) tangent_obs_columns(int nx, int ny, int pitch, long long ps,
+                                                                  const double *g, DualT *ext, DualT *cl,
+                                                                  DualT *ovl) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ DualT part[TRUNS][32], bsum[32];
+    __shared__ RunCross cross[TRUNS][32], bcross[32];
+    const int lane = threadIdx.x, run = threadIdx.y, x = blockIdx.x * 32 + lane, CH = (int)cluster.num_blocks();
+    const int rows = (ny + CH * TRUNS - 1) / (CH * TRUNS);
+    const int y0 = (blockIdx.y * TRUNS + run) * rows, y1 = min(ny, y0 + rows);
+    DualT o(0.0);
+    RunCross cr;
+    cr.clear();
+    if (x < nx)
+        for (int y = y0; y < y1; y++) {
+            const long long n = (long long)y * pitch + x;
+            const DualT p1 = node_phi(g, 0, ps, n), p2 = node_phi(g, 9, ps, n);
+            o += p1 * (DualT(1.0) - p1 - p2);
+            cr.add(y, clamp01(p1.v) + clamp01(p2.v));
         }
-        ext[x] = (c.first != -2 && c.last != -2) ? c.hi - c.lo : DualT(0.0);
-        cl[x] = (ny & 1) ? mid : 0.5 * mid;
-    }
+    part[run][lane] = o;
+    cross[run][lane] = cr;
     __syncthreads();
-    // l_y: argmax over the columns
-    {
-        double best = -1.0;
-        int bi = INT_MAX;
-        for (int x = t; x < nx; x += TOB)
-            if (ext[x].v > best) { best = ext[x].v; bi = x; }
-        sv[t] = best;
-        si[t] = bi;
-        __syncthreads();
-        for (int s = TOB / 2; s > 0; s >>= 1) {
-            if (t < s && (sv[t + s] > sv[t] || (sv[t + s] == sv[t] && si[t + s] < si[t]))) {
-                sv[t] = sv[t + s];
-                si[t] = si[t + s];
-            }
-            __syncthreads();
-        }
+    if (run == 0) {  // the block's runs in row order, then (below) the cluster's blocks
+        RunCross all;
+        all.clear();
+        for (int r = 0; r < TRUNS; r++) all.join((blockIdx.y * TRUNS + r) * rows, cross[r][lane]);
+        bcross[lane] = all;
+    } else if (run == 1) {
+        DualT s(0.0);
+        for (int r = 0; r < TRUNS; r++) s += part[r][lane];
+        bsum[lane] = s;
     }
-    // overlap: fixed-order reduction (warp, then the warps in order)
-    for (int o = 16; o > 0; o >>= 1) {
-        DualT other;
-        other.v = __shfl_down_sync(0xffffffffu, ovl.v, o);
-#pragma unroll
-        for (int c = 0; c < NT; c++) other.d[c] = __shfl_down_sync(0xffffffffu, ovl.d[c], o);
-        ovl += other;
-    }
-    if ((t & 31) == 0) sred[t / 32] = ovl;
-    __syncthreads();
-    if (t == 0) {
-        DualT tot(0.0);
-        for (int w = 0; w < TOB / 32; w++) tot += sred[w];
-        const DualT ly = si[0] < nx ? ext[si[0]] : DualT(0.0);
-        // l_x along the centre line, unwrapped from the emptiest column
-        const int xcut = prim->xcut;
-        auto clv = [&](int j) {
-            int x = xcut + j;
-            x = x >= nx ? x - nx : x;
-            return cl[x];
+    cluster.sync();
+    if (cluster.block_rank() == 0 && x < nx) {
+        auto at = [&](int y) {
+            const long long n = (long long)y * pitch + x;
+            return clamp01(node_phi(g, 0, ps, n)) + clamp01(node_phi(g, 9, ps, n));
         };
-        DCross c{-2, -2, DualT(0.0), DualT(0.0)};
-        for (int i = -1; i < nx; i++) {
-            const DualT a = i < 0 ? DualT(0.0) : clv(i), b = i + 1 < nx ? clv(i + 1) : DualT(0.0);
-            cross_step(c, i, a, b);
+        if (run == 0) {
+            RunCross all;
+            all.clear();
+            for (int q = 0; q < CH; q++) all.join(q * TRUNS * rows, *cluster.map_shared_rank(&bcross[lane], q));
+            all.close(ny);
+            ext[x] = all.found() ? cross_extent<DualT>(all.first, all.last, ny, at) : DualT(0.0);
+        } else if (run == 1) {
+            cl[x] = (ny & 1) ? at(ny / 2) : 0.5 * (at(ny / 2 - 1) + at(ny / 2));
+        } else if (run == 2) {
+            DualT s(0.0);
+            for (int q = 0; q < CH; q++) s += *cluster.map_shared_rank(&bsum[lane], q);
+            ovl[x] = s;
         }
-        const DualT lx = (c.first != -2 && c.last != -2) ? c.hi - c.lo : DualT(0.0);
-        const DualT To = (lx.v + ly.v) > 0.0 ? (ly - lx) / (ly + lx) : DualT(0.0);
-        out->T_o = To.v;
-        out->overlap = tot.v;
-        out->lx = lx.v;
-        out->ly = ly.v;
-        for (int q = 0; q < NT; q++) {
-            out->dT_o[q] = To.d[q];
-            out->doverlap[q] = tot.d[q];
-            out->dlx[q] = lx.d[q];
-            out->dly[q] = ly.d[q];
-        }
+    }
+    cluster.sync();  // the other blocks' shared memory is read until here
+}
+
+// One block over the columns: l_y = the largest extent (first column among
+// equal maxima), l_x from the centre-line crossings in the frame that starts at
+// the emptiest column found by the plain observables, the overlap, and
+// T_o = (l_y - l_x) / (l_y + l_x).
+constexpr int TOB = 256;
+__global__ void __launch_bounds__(TOB) tangent_obs_final(int nx, const DualT *ext, const DualT *cl,
+                                                         const DualT *ovl, const ObsOut *prim, TanOut *out,
+                                                         TanCtls ctls) {
+    const int t = threadIdx.x, xcut = prim->xcut;
+    auto clv = [&](int j) {
+        const int x = xcut + j;
+        return cl[x >= nx ? x - nx : x];
+    };
+    long long best[1] = {-1};  // extents are >= 0
+    double tot[1 + NT] = {};
+    int ij[2] = {INT_MAX, INT_MAX}, last[1] = {-3};  // first column of the maximum, rising step
+    for (int x = t; x < nx; x += TOB) {
+        if (ext[x].v >= 0.0) best[0] = max(best[0], order_bits(ext[x].v));
+        tot[0] += ovl[x].v;
+#pragma unroll
+        for (int c = 0; c < NT; c++) tot[1 + c] += ovl[x].d[c];
+    }
+    auto least = [](int a, int b) { return min(a, b); };
+    block_reduce<TOB>(best, [](long long a, long long b) { return max(a, b); });
+    block_reduce<TOB>(tot, [](double a, double b) { return a + b; });
+    for (int x = t; x < nx; x += TOB)
+        if (order_bits(ext[x].v) == best[0]) ij[0] = min(ij[0], x);
+    for (int i = t - 1; i < nx; i += TOB) {
+        const double a = i < 0 ? 0.0 : clv(i).v, b = i + 1 < nx ? clv(i + 1).v : 0.0;
+        if (a < 0.5 && b >= 0.5) ij[1] = min(ij[1], i);
+        if (a >= 0.5 && b < 0.5) last[0] = max(last[0], i);
+    }
+    block_reduce<TOB>(ij, least);
+    block_reduce<TOB>(last, [](int a, int b) { return max(a, b); });
+    if (t != 0) return;
+    const DualT ly = ij[0] < nx ? ext[ij[0]] : DualT(0.0);
+    const DualT lx = ij[1] != INT_MAX && last[0] != -3 ? cross_extent<DualT>(ij[1], last[0], nx, clv) : DualT(0.0);
+    const DualT To = (lx.v + ly.v) > 0.0 ? (ly - lx) / (ly + lx) : DualT(0.0);
+    out->T_o = To.v;
+    out->overlap = tot[0];
+    out->lx = lx.v;
+    out->ly = ly.v;
+    out->nonconv = 0;
+    for (int q = 0; q < NT; q++) {
+        out->dT_o[q] = To.d[q];
+        out->doverlap[q] = tot[1 + q];
+        out->dlx[q] = lx.d[q];
+        out->dly[q] = ly.d[q];
+        if (ctls.c[q]) out->nonconv += ctls.c[q]->nonconv_count;
     }
 }
 
@@ -173,12 +181,13 @@ void launch_tangent_phase(const Phys<double> &P, const double *g, double *phi1, 
     tangent_phase_kernel<<<gr, b, 0, s>>>(P, g, phi1, phi2, k);
 }
 
-size_t tangent_obs_scratch_bytes(int nx) { return 2ull * nx * sizeof(DualT); }
+size_t tangent_obs_scratch_bytes(int nx) { return 3ull * nx * sizeof(DualT); }
 
 void launch_tangent_obs(const Phys<double> &P, const double *g, const ObsOut *prim, void *scratch,
-                        TanOut *out, cudaStream_t s) {
-    DualT *ext = static_cast<DualT *>(scratch), *cl = ext + P.nx;
-    tangent_obs_kernel<<<1, TOB, 0, s>>>(P.nx, P.ny, P.pitch, P.ps, g, prim, ext, cl, out);
+                        TanOut *out, TanCtls ctls, cudaStream_t s) {
+    DualT *ext = static_cast<DualT *>(scratch), *cl = ext + P.nx, *ovl = cl + P.nx;
+    launch_columns(tangent_obs_columns, TRUNS, P.nx, P.ny, s, P.nx, P.ny, P.pitch, P.ps, g, ext, cl, ovl);
+    tangent_obs_final<<<1, TOB, 0, s>>>(P.nx, ext, cl, ovl, prim, out, ctls);
 }
 
 }  // namespace fcd
