@@ -281,10 +281,10 @@ void fcd_batch_destroy(fcd_batch *b);
  * (primal values), fcd_get_field (primal fields), fcd_kernel_launches,
  * fcd_solver_stats, fcd_last_error and fcd_destroy; state snapshots and
  * population import return FCD_ESTATE. Each step runs as one captured CUDA
- * graph (the primal and the four tangent solves as conditional-node loops, as in
- * fcd_step), with no host synchronisation between steps; with the environment
- * variable FCD_NO_GRAPH=1 the solves are driven from the host instead, one
- * synchronisation per multigrid cycle. */
+ * graph (the primal solve one kernel, the four tangent solves one kernel each,
+ * side by side), with no host synchronisation between steps; with the environment
+ * variable FCD_NO_GRAPH=1 the kernels are launched from the host instead, one
+ * synchronisation per solve. */
 enum { FCD_DIR_BO_M = 0, FCD_DIR_CA = 1, FCD_DIR_ALPHA = 2, FCD_DIR_NU_R = 3, FCD_NDIR = 4 };
 typedef struct {
     long step;

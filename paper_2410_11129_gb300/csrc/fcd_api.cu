@@ -2,9 +2,10 @@
 // (arXiv 2410.11129): parameter mapping, state, CUDA-graph step loop.
 //
 // One step is captured once per (buffer parity, store-macro flag) into a CUDA
-// graph: phase recovery -> coarse permeabilities -> a while node running
-// multigrid V-cycles until the device-side control block reports convergence
-// or the cycle cap -> fused collide-stream -> step counter. fcd_step(n)
+// graph: phase recovery -> potential solve (one cooperative kernel, or an
+// opening sweep, a residual and an IF node with further multigrid cycles, until
+// the device-side control block reports convergence or the cycle cap) -> fused
+// collide-stream. fcd_step(n)
 // launches n such graphs; nothing synchronises with the host in between.
 #include <algorithm>
 #include <cmath>
@@ -437,9 +438,8 @@ struct Engine : fcd_ctx {
             launch_open_bc<T>(mode, P, f[c], g[c], f[c ^ 1], g[c ^ 1], prm.u_max, D.u_avg, s);
     }
     int post_kernels() const { return prm.open_x ? 2 : 1; }
-    // the phase kernel, and in FP64 contexts with a field the solve's
-    // coefficient kernel (the multigrid counts its own cycles)
-    int pre_kernels() const { return 1 + (magnetic() && sizeof(T) == 8 ? 1 : 0); }
+    // the phase kernel, and a one-kernel solve (the other form counts its cycles)
+    int pre_kernels() const { return 1 + (magnetic() && mg_one_kernel<T>(mg) ? 1 : 0); }
 
     // One solve with host checks between cycles (hierarchy m with control
     // block c; default: the context's own).
@@ -448,17 +448,26 @@ struct Engine : fcd_ctx {
             m = mg;
             c = ctl;
         }
-        mg_presmooth<T>(m, P.H0c, P.H0s, s);
-        for (int guard = 0; guard < 1000000; guard++) {
-            mg_cycle_head<T>(m, P.H0c, P.H0s, 0, 0, 0, s);
-            CK(cudaGetLastError());
+        if (mg_one_kernel<T>(m)) {
+            CK(mg_solve<T>(m, P.H0c, P.H0s, s));
             CK(cudaMemcpyAsync(h_ctl, c, sizeof(MgCtl), cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
-            if (!h_ctl->keep_going) break;
-            if (h_ctl->mode == 1) mg_cycle_smooth<T>(m, P.H0c, P.H0s, s);
-            else if (h_ctl->mode == 2) mg_cycle_twogrid<T>(m, P.H0c, P.H0s, s);
-            else mg_cycle_rest<T>(m, P.H0c, P.H0s, s);
-            CK(cudaGetLastError());
+            if (h_ctl->stuck) return fail(FCD_ECUDA, "a grid barrier of the potential solve timed out");
+            return FCD_OK;
+        }
+        if constexpr (sizeof(T) == 4) {
+            mg_presmooth(m, P.H0c, P.H0s, s);
+            for (int guard = 0; guard < 1000000; guard++) {
+                mg_cycle_head(m, P.H0c, P.H0s, 0, 0, 0, s);
+                CK(cudaGetLastError());
+                CK(cudaMemcpyAsync(h_ctl, c, sizeof(MgCtl), cudaMemcpyDeviceToHost, s));
+                CK(cudaStreamSynchronize(s));
+                if (!h_ctl->keep_going) break;
+                if (h_ctl->mode == 1) mg_cycle_smooth(m, P.H0c, P.H0s, s);
+                else if (h_ctl->mode == 2) mg_cycle_twogrid(m, P.H0c, P.H0s, s);
+                else mg_cycle_rest(m, P.H0c, P.H0s, s);
+                CK(cudaGetLastError());
+            }
         }
         return FCD_OK;
     }
@@ -479,97 +488,22 @@ struct Engine : fcd_ctx {
         return FCD_OK;
     }
 
-    // The cycle loop of one potential solve in the graph (stream s is capturing;
-    // the opening sweeps are already captured), in one of two shapes. Contexts
-    // solving to 1e-5 or looser, whose solves mostly stop at their first head
-    // (1.0-1.1 heads per step on the FP32 production channels), take the IF
-    // form; tighter tolerances (FP64 at 1e-10: about 11 heads per step) the
-    // while form. Measured: 1600 x 200 FP32 solve stage 33.9 -> 28.0 us with the
-    // IF form; 200 x 40 FP64 0.72 -> 0.78 ms per step with it (one dispatch
-    // kernel node more per cycle), hence the split.
-    static constexpr double IF_FORM_TOL = 1e-5;
+    // One potential solve in the graph (stream s is capturing): one kernel, or
+    // the opening sweep and the cycle loop.
     fcd_status capture_mg_loop(cudaStream_t s, MgHost<T> *m = nullptr) {
         if (!m) m = mg;
-        return prm.mag_tol >= IF_FORM_TOL ? capture_mg_if_loop(s, m) : capture_mg_while_loop(s, m);
-    }
-
-    // The while form: a while node whose body is the cycle head (the residual
-    // kernel, which sets both conditions) and a switch node holding the rest of
-    // the chosen cycle. One kernel node fewer per cycle than the IF form, for
-    // solves that run many cycles.
-    fcd_status capture_mg_while_loop(cudaStream_t s, MgHost<T> *m) {
-        cudaStreamCaptureStatus cs;
-        cudaGraph_t gcap;
-        const cudaGraphNode_t *deps = nullptr;
-        size_t nd = 0;
-        CK(cudaStreamGetCaptureInfo(s, &cs, nullptr, &gcap, &deps, nullptr, &nd));
-        cudaGraphConditionalHandle h;
-        CK(cudaGraphConditionalHandleCreate(&h, gcap, 1, cudaGraphCondAssignDefault));
-        cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};
-        cp.conditional.handle = h;
-        cp.conditional.type = cudaGraphCondTypeWhile;
-        cp.conditional.size = 1;
-        cudaGraphNode_t wnode;
-        CK(cudaGraphAddNode(&wnode, gcap, deps, nullptr, nd, &cp));
-        // while body: lattice residual, then a switch node holding the rest
-        // of the V-cycle (case 0), lattice sweeps only (case 1) or a
-        // two-grid cycle (case 2); both conditions are set by the residual
-        // kernel
-        cudaGraph_t body = cp.conditional.phGraph_out[0];
-        cudaGraphConditionalHandle hi;
-        CK(cudaGraphConditionalHandleCreate(&hi, body, 0, cudaGraphCondAssignDefault));
-        cudaStream_t bs;
-        CK(cudaStreamCreateWithFlags(&bs, cudaStreamNonBlocking));
-        cudaError_t e1 = cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0,
-                                                       cudaStreamCaptureModeThreadLocal);
-        cudaGraph_t out1 = nullptr, out2 = nullptr;
-        if (e1 == cudaSuccess) {
-            mg_cycle_head<T>(m, P.H0c, P.H0s, h, hi, 1, bs);
-            const cudaGraphNode_t *bd = nullptr;
-            size_t bn = 0;
-            cudaStreamCaptureStatus bcs;
-            cudaGraph_t bg;
-            e1 = cudaStreamGetCaptureInfo(bs, &bcs, nullptr, &bg, &bd, nullptr, &bn);
-            cudaGraphNodeParams ip = {cudaGraphNodeTypeConditional};
-            ip.conditional.handle = hi;
-            ip.conditional.type = cudaGraphCondTypeSwitch;
-            ip.conditional.size = 3;
-            cudaGraphNode_t inode;
-            if (e1 == cudaSuccess) e1 = cudaGraphAddNode(&inode, body, bd, nullptr, bn, &ip);
-            if (e1 == cudaSuccess)
-                e1 = cudaStreamUpdateCaptureDependencies(bs, &inode, nullptr, 1,
-                                                         cudaStreamSetCaptureDependencies);
-            cudaError_t e2 = cudaStreamEndCapture(bs, &out1);
-            if (e1 == cudaSuccess) e1 = e2;
-            if (e1 == cudaSuccess)
-                e1 = cudaStreamBeginCaptureToGraph(bs, ip.conditional.phGraph_out[0], nullptr,
-                                                   nullptr, 0, cudaStreamCaptureModeThreadLocal);
-            if (e1 == cudaSuccess) {
-                mg_cycle_rest<T>(m, P.H0c, P.H0s, bs);
-                e1 = cudaStreamEndCapture(bs, &out2);
-            }
-            if (e1 == cudaSuccess)
-                e1 = cudaStreamBeginCaptureToGraph(bs, ip.conditional.phGraph_out[1], nullptr,
-                                                   nullptr, 0, cudaStreamCaptureModeThreadLocal);
-            if (e1 == cudaSuccess) {
-                mg_cycle_smooth<T>(m, P.H0c, P.H0s, bs);
-                e1 = cudaStreamEndCapture(bs, &out2);
-            }
-            if (e1 == cudaSuccess)
-                e1 = cudaStreamBeginCaptureToGraph(bs, ip.conditional.phGraph_out[2], nullptr,
-                                                   nullptr, 0, cudaStreamCaptureModeThreadLocal);
-            if (e1 == cudaSuccess) {
-                mg_cycle_twogrid<T>(m, P.H0c, P.H0s, bs);
-                e1 = cudaStreamEndCapture(bs, &out2);
-            }
+        if (mg_one_kernel<T>(m)) {
+            CK(mg_solve<T>(m, P.H0c, P.H0s, s));
+            return FCD_OK;
         }
-        cudaStreamDestroy(bs);
-        CK(e1);
-        CK(cudaStreamUpdateCaptureDependencies(s, &wnode, nullptr, 1, cudaStreamSetCaptureDependencies));
+        if constexpr (sizeof(T) == 4) {
+            mg_presmooth(m, P.H0c, P.H0s, s);
+            return capture_mg_if_loop(s, m);
+        }
         return FCD_OK;
     }
 
-    // The IF form: the first cycle head as a plain
+    // The cycle loop: the first cycle head as a plain
     // kernel node, then an IF node, entered only when that head chose another
     // cycle, around a while node (condition 1 on entry) whose body dispatches
     // the chosen cycle through a switch node (0 the rest of a V-cycle, 1 lattice
@@ -578,7 +512,7 @@ struct Engine : fcd_ctx {
     // body or not (measured on this GPU); a solve that stops at its first head,
     // the common case, pays for the IF node only, not for a while node entered
     // once with a switch node inside (about 14 us).
-    fcd_status capture_mg_if_loop(cudaStream_t s, MgHost<T> *m) {
+    fcd_status capture_mg_if_loop(cudaStream_t s, MgHost<float> *m) {
         cudaStreamCaptureStatus cs;
         cudaGraph_t gcap;
         const cudaGraphNode_t *deps = nullptr;
@@ -586,7 +520,7 @@ struct Engine : fcd_ctx {
         CK(cudaStreamGetCaptureInfo(s, &cs, nullptr, &gcap, nullptr, nullptr, nullptr));
         cudaGraphConditionalHandle hif;
         CK(cudaGraphConditionalHandleCreate(&hif, gcap, 0, cudaGraphCondAssignDefault));
-        mg_cycle_head<T>(m, P.H0c, P.H0s, hif, 0, 3, s);
+        mg_cycle_head(m, P.H0c, P.H0s, hif, 0, 3, s);
         CK(cudaGetLastError());
         CK(cudaStreamGetCaptureInfo(s, &cs, nullptr, &gcap, &deps, nullptr, &nd));
         cudaGraphNodeParams ip = {cudaGraphNodeTypeConditional};
@@ -619,7 +553,7 @@ struct Engine : fcd_ctx {
         cudaError_t e = cudaStreamBeginCaptureToGraph(bs, body, nullptr, nullptr, 0,
                                                       cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            mg_cycle_dispatch<T>(m, hs, bs);
+            mg_cycle_dispatch(m, hs, bs);
             const cudaGraphNode_t *bd = nullptr;
             size_t bn = 0;
             cudaStreamCaptureStatus bcs;
@@ -630,7 +564,7 @@ struct Engine : fcd_ctx {
             if (e == cudaSuccess)
                 e = cudaStreamUpdateCaptureDependencies(bs, &snode, nullptr, 1,
                                                         cudaStreamSetCaptureDependencies);
-            if (e == cudaSuccess) mg_cycle_head<T>(m, P.H0c, P.H0s, hw, 0, 3, bs);
+            if (e == cudaSuccess) mg_cycle_head(m, P.H0c, P.H0s, hw, 0, 3, bs);
             const cudaError_t e2 = cudaStreamEndCapture(bs, &out);
             if (e == cudaSuccess) e = e2;
         }
@@ -639,9 +573,9 @@ struct Engine : fcd_ctx {
             e = cudaStreamBeginCaptureToGraph(bs, sp.conditional.phGraph_out[c], nullptr, nullptr, 0,
                                               cudaStreamCaptureModeThreadLocal);
             if (e != cudaSuccess) break;
-            if (c == 0) mg_cycle_rest<T>(m, P.H0c, P.H0s, bs);
-            else if (c == 1) mg_cycle_smooth<T>(m, P.H0c, P.H0s, bs);
-            else mg_cycle_twogrid<T>(m, P.H0c, P.H0s, bs);
+            if (c == 0) mg_cycle_rest(m, P.H0c, P.H0s, bs);
+            else if (c == 1) mg_cycle_smooth(m, P.H0c, P.H0s, bs);
+            else mg_cycle_twogrid(m, P.H0c, P.H0s, bs);
             e = cudaStreamEndCapture(bs, &out);
         }
         cudaStreamDestroy(bs);
@@ -656,7 +590,6 @@ struct Engine : fcd_ctx {
         enqueue_pre(c, s);
         if (profiling) CK(cudaEventRecordWithFlags(ev[1], s, cudaEventRecordExternal));
         if (magnetic()) {
-            mg_presmooth<T>(mg, P.H0c, P.H0s, s);
             const fcd_status st = capture_mg_loop(s);
             if (st != FCD_OK) return st;
         }
@@ -785,6 +718,7 @@ struct Engine : fcd_ctx {
         }
         o->mag_iters = magnetic() ? h_ctl->last_iters : 0;
         o->mag_resid = magnetic() ? h_ctl->last_resid : 0.0;
+        if (h_ctl->stuck) return fail(FCD_ECUDA, "a grid barrier of the potential solve timed out");
         if (unstable_status() != FCD_OK) return FCD_EUNSTABLE;
         if (r.nonfinite) return fail(FCD_EUNSTABLE, "non-finite phase field at step %ld", step);
         if (h_ctl->nonconv_count > reported_nonconv) {
@@ -1011,10 +945,13 @@ struct Engine : fcd_ctx {
     }
 
     long launches() const override {
+        if (mg_one_kernel<T>(mg)) return host_kernels;  // solves included
         MgCtl c;
         if (cudaMemcpy(&c, ctl, sizeof c, cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
-        return host_kernels + (long)c.cycles_launched + (long)c.total_cycles * mg_kernels_per_cycle(mg) +
-               (long)c.smooth_cycles + 2 * (long)c.twogrid_cycles + (long)c.dispatches;
+        int per_cycle = 0;
+        if constexpr (sizeof(T) == 4) per_cycle = mg_kernels_per_cycle(mg);
+        return host_kernels + (long)c.cycles_launched + (long)c.total_cycles * per_cycle + (long)c.smooth_cycles +
+               2 * (long)c.twogrid_cycles + (long)c.dispatches;
     }
 };
 
@@ -1153,6 +1090,7 @@ struct TangentEngine : Engine<double> {
                                        release, user, err, sizeof err, 0, mg);
             if (!mgt[c]) return FCD_ENOMEM;
             mg_set_rhs<double>(mgt[c], rhst[c]);
+            mg_set_share<double>(mgt[c], NT);  // the NT solves of a step run side by side
         }
         return FCD_OK;
     }
@@ -1178,7 +1116,6 @@ struct TangentEngine : Engine<double> {
             mg_reset_scaled(ctlt[c], rmax + c, tol, max_iter, sc);
             fcd_status st;
             if (capture) {
-                mg_presmooth<double>(mgt[c], P.H0c, P.H0s, sc);
                 st = capture_mg_loop(sc, mgt[c]);
             } else {
                 st = host_mg_loop(sc, mgt[c], ctlt[c]);
@@ -1194,24 +1131,11 @@ struct TangentEngine : Engine<double> {
         return FCD_OK;
     }
 
-    // kernels of one step outside the multigrid cycles (those are counted on
-    // the device): two phase kernels, the primal solve's coefficient kernel and
-    // per direction the right-hand side, two copies and the reset, the
-    // potential copy and the collision
+    // kernels of one step: two phase kernels, the primal solve and per direction
+    // the right-hand side, two copies, the reset and the solve, the potential
+    // copy and the collision
     long step_kernels() const {
-        return 2 + (magnetic() ? 4 * NT + 1 : 0) + 2 + (prm.open_x ? 1 : 0);
-    }
-
-    long launches() const override {
-        long n = Engine<double>::launches();
-        for (int c = 0; c < NT; c++) {
-            if (!mgt[c]) continue;
-            MgCtl q;
-            if (cudaMemcpy(&q, ctlt[c], sizeof q, cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
-            n += (long)q.cycles_launched + (long)q.total_cycles * mg_kernels_per_cycle(mgt[c]) +
-                 (long)q.smooth_cycles + 2 * (long)q.twogrid_cycles + (long)q.dispatches;
-        }
-        return n;
+        return 2 + (magnetic() ? 5 * NT + 1 : 0) + 2 + (prm.open_x ? 1 : 0);
     }
 
     fcd_status solve(double tol, int max_iter, int *iters, double *resid) override {
@@ -1220,7 +1144,7 @@ struct TangentEngine : Engine<double> {
         const fcd_status st = Engine<double>::solve(tol, max_iter, iters, resid);
         if (st != FCD_OK && st != FCD_ENOCONV) return st;
         launch_tangent_phase(P, static_cast<const double *>(g[cur]), phi1, phi2, k, stream);
-        host_kernels += 1 + (magnetic() ? 4 * NT : 0);  // the tangent phase; per direction 4
+        host_kernels += 1 + (magnetic() ? 5 * NT : 0);  // the tangent phase; per direction 5
         const fcd_status st2 = tangent_solves(false, tol, max_iter, stream, false);
         return st2 != FCD_OK ? st2 : st;
     }
@@ -1232,7 +1156,6 @@ struct TangentEngine : Engine<double> {
         if (magnetic()) {
             fcd_status st;
             if (capture) {
-                mg_presmooth<double>(mg, P.H0c, P.H0s, s);
                 st = capture_mg_loop(s);
             } else {
                 st = host_mg_loop(s);
@@ -1529,7 +1452,6 @@ struct AdjointEngine : Engine<double> {
             // initial guess 2 lam(n+1) - lam(n+2), as the plain solve extrapolates psi'
             mg_psi_io(mga, 2, lamS, lamP, s);
             mg_reset_scaled(ctla, rmax, prm.mag_tol, prm.mag_max_iter, s);
-            mg_presmooth<double>(mga, P.H0c, P.H0s, s);
             const fcd_status st = capture ? capture_mg_loop(s, mga) : host_mg_loop(s, mga, ctla);
             if (st != FCD_OK) return st;
             mg_psi_io(mga, 0, lamS, nullptr, s);
@@ -1553,8 +1475,8 @@ struct AdjointEngine : Engine<double> {
         CK(cudaGetLastError());
         return FCD_OK;
     }
-    // kernels of one adjoint step outside the multigrid cycles
-    long adj_step_kernels() const { return 6 + (magnetic() ? 5 : 0) + (prm.open_x ? 2 : 0); }
+    // kernels of one adjoint step (the solve with its guess, reset and copy: 4)
+    long adj_step_kernels() const { return 5 + (magnetic() ? 4 : 0) + (prm.open_x ? 2 : 0); }
 
     fcd_status adj_step(int c) {
         cudaStream_t s = stream;
@@ -1738,17 +1660,6 @@ struct AdjointEngine : Engine<double> {
         return FCD_OK;
     }
 
-    long launches() const override {
-        long n = Engine<double>::launches();
-        if (mga) {
-            MgCtl q;
-            if (cudaMemcpy(&q, ctla, sizeof q, cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
-            n += (long)q.cycles_launched + (long)q.total_cycles * mg_kernels_per_cycle(mga) +
-                 (long)q.smooth_cycles + 2 * (long)q.twogrid_cycles + (long)q.dispatches;
-        }
-        return n;
-    }
-
     size_t state_bytes() const override { return 0; }
     fcd_status get_state(void *, size_t) override {
         return fail(FCD_ESTATE, "state snapshots are not available for adjoint contexts");
@@ -1790,6 +1701,11 @@ bool engine_view(fcd_ctx *c, EngineView *v) {
     v->max_iter = e->prm.mag_max_iter;
     v->comp = e->comp;
     return true;
+}
+
+void engine_share(fcd_ctx *c, int share) {
+    if (auto *e = dynamic_cast<Engine<float> *>(c)) mg_set_share<float>(e->mg, share);
+    else if (auto *d = dynamic_cast<Engine<double> *>(c)) mg_set_share<double>(d->mg, share);
 }
 
 fcd_status engine_step1(fcd_ctx *c, int store_macro) {

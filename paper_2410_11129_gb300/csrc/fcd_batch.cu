@@ -29,6 +29,8 @@ using namespace fcd;
 
 namespace {
 
+constexpr int SIDE_SOLVES = 8;  // one-kernel solves of a batch that run side by side
+
 struct Group {
     int mode = MODE_FP32;
     std::vector<int> idx;          // instances in the group
@@ -37,7 +39,13 @@ struct Group {
     int n_ptiles = 0, n_ctiles = 0;
     BatchTile *d_ptiles = nullptr, *d_ctiles = nullptr;
     BatchLbm<float> *d_tab[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // [parity][macro]
-    MgBatch *mg = nullptr;
+    MgBatch *mg = nullptr;         // batched solves (single-plane form)
+    // pair form: every instance's solve is one kernel, several side by side
+    std::vector<MgHost<float> *> one;
+    std::vector<float> one_c, one_s;
+    std::vector<cudaStream_t> side;
+    std::vector<cudaEvent_t> joined;
+    cudaEvent_t fork = nullptr;
     cudaStream_t stream = nullptr, cap = nullptr;
     cudaEvent_t done = nullptr, solved = nullptr;
     // per buffer parity: graph A = phase recovery + potential solves; graph B
@@ -73,6 +81,9 @@ void group_free(Group *g) {
     }
     if (g->mg) mg_batch_destroy(g->mg);
     for (void *p : g->mem) cudaFree(p);
+    for (auto e : g->joined) cudaEventDestroy(e);
+    for (auto t : g->side) cudaStreamDestroy(t);
+    if (g->fork) cudaEventDestroy(g->fork);
     if (g->done) cudaEventDestroy(g->done);
     if (g->solved) cudaEventDestroy(g->solved);
     if (g->stream) cudaStreamDestroy(g->stream);
@@ -188,7 +199,30 @@ fcd_status group_build(Group &g, const char **why) {
             hc.push_back(v.P.H0c);
             hs.push_back(v.P.H0s);
         }
-    if (!mgs.empty()) {
+    if (!mgs.empty() && mg_one_kernel<float>(mgs[0])) {
+        g.one = mgs;
+        g.one_c = hc;
+        g.one_s = hs;
+        const size_t n = std::min<size_t>(mgs.size(), SIDE_SOLVES);
+        if (cudaEventCreateWithFlags(&g.fork, cudaEventDisableTiming) != cudaSuccess) {
+            *why = "stream/event creation";
+            return FCD_ECUDA;
+        }
+        for (size_t i = 0; i < n; i++) {
+            cudaStream_t t;
+            cudaEvent_t e;
+            if (cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking) != cudaSuccess) {
+                *why = "stream/event creation";
+                return FCD_ECUDA;
+            }
+            g.side.push_back(t);
+            if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
+                *why = "stream/event creation";
+                return FCD_ECUDA;
+            }
+            g.joined.push_back(e);
+        }
+    } else if (!mgs.empty()) {
         static char mgerr[256];
         g.mg = mg_batch_create(mgs, hc, hs, [](size_t n, void *) -> void * {
                                    void *p = nullptr;
@@ -254,12 +288,30 @@ cudaError_t capture_solve_loop(Group &g, cudaStream_t s) {
     return cudaStreamUpdateCaptureDependencies(s, &wnode, nullptr, 1, cudaStreamSetCaptureDependencies);
 }
 
+// The one-kernel solves of a group at the capture point of s, as parallel
+// branches that s waits for.
+cudaError_t capture_one_kernel_solves(Group &g, cudaStream_t s) {
+    cudaError_t e = cudaEventRecord(g.fork, s);
+    for (size_t t = 0; t < g.side.size() && e == cudaSuccess; t++) e = cudaStreamWaitEvent(g.side[t], g.fork, 0);
+    for (size_t i = 0; i < g.one.size() && e == cudaSuccess; i++)
+        e = mg_solve<float>(g.one[i], g.one_c[i], g.one_s[i], g.side[i % g.side.size()]);
+    for (size_t t = 0; t < g.side.size() && e == cudaSuccess; t++) {
+        e = cudaEventRecord(g.joined[t], g.side[t]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, g.joined[t], 0);
+    }
+    return e;
+}
+
 // One step of the group launched from the host (FCD_NO_GRAPH=1: profilers that
 // do not follow conditional graph nodes see every kernel); the host reads the
 // loop condition after each pass of the body.
 cudaError_t group_host_step(Group &g, int c, int sm) {
     cudaStream_t s = g.stream;
     launch_phase_batch<float>(g.mode, g.d_tab[c][0], g.d_ptiles, g.n_ptiles, s);
+    for (size_t i = 0; i < g.one.size(); i++) {
+        const cudaError_t e = mg_solve<float>(g.one[i], g.one_c[i], g.one_s[i], s);
+        if (e != cudaSuccess) return e;
+    }
     if (g.mg) {
         mg_batch_presmooth(g.mg, s);
         for (int guard = 0; guard < 1000000; guard++) {
@@ -292,6 +344,7 @@ cudaError_t group_graph_a(Group &g, int c) {
     cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
     launch_phase_batch<float>(g.mode, g.d_tab[c][0], g.d_ptiles, g.n_ptiles, s);
+    if (!g.one.empty()) e = capture_one_kernel_solves(g, s);
     if (g.mg) {
         mg_batch_presmooth(g.mg, s);
         e = capture_solve_loop(g, s);
@@ -396,6 +449,7 @@ fcd_status fcd_batch_create(const fcd_params *params, int n, fcd_batch **out) {
         }
         b->inst.push_back(c);
         fcd_set_stream(c, s);
+        engine_share(c, std::min(n, SIDE_SOLVES));  // solves of several instances side by side
     }
     // group the periodic FP32 instances by storage form and level-0 form of the
     // potential (one FP32 plane or the hi + lo pair), and split each such set

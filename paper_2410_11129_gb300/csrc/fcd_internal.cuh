@@ -128,7 +128,7 @@ struct Level {
     const T *pwx, *pwy;
     const T *rhs;  // level 0: explicit right-hand side (nullptr: -L psi0 formed from k)
     // level 0 of FP64 hierarchies: the 9-point coefficients of every node, formed
-    // once per solve (planes c_1..c_8, diagonal, its reciprocal, -L psi0)
+    // once per solve (planes c_1..c_8, diagonal, -L psi0)
     T *coef;
     // level 0 of FP32 hierarchies: 1 when psi' is the hi + lo pair (the lo
     // plane one plane stride after each buffer) and the residual is formed in
@@ -163,7 +163,27 @@ struct MgCtl {
     long long twogrid_cycles;      // cumulative two-grid cycles (launch accounting)
     unsigned batch_visits;         // batched solves: blocks of the current residual launch seen
     long long dispatches;          // cumulative cycle dispatch launches of graph loops (accounting)
+    // solves that run as one cooperative kernel (fcd_mg_solve.cuh); reset with the solve
+    unsigned long long norm_slot[4];  // max |r| of the last heads (bits of doubles >= 0)
+    unsigned bar;                     // arrivals at the kernel's grid barriers
+    int stuck;                        // a barrier timed out: no solve runs any more
 };
+// start of a potential solve (one thread)
+__device__ __forceinline__ void mg_reset_ctl(MgCtl *c, double tolH0, int max_iter) {
+    c->norm_bits = 0ull;
+    c->iter = 0;
+    c->done = 0;
+    c->converged = 0;
+    c->tolH0 = tolH0;
+    c->max_iter = max_iter;
+    c->keep_going = 1;
+    c->blocks_done = 0u;
+    c->mode = 1;         // the opening sweeps count as a lattice-sweep cycle
+    c->smooth_left = 0;  // ... and use up the sweep allowance
+    c->twogrid_left = 2;
+    for (int q = 0; q < 4; q++) c->norm_slot[q] = 0ull;
+    c->bar = 0u;
+}
 
 // What the phase kernel does besides Eq. 32: reset the solve's control block
 // (reset != 0) and, when step != nullptr, record the step index in flight in
@@ -309,25 +329,28 @@ MgHost<T> *mg_create(int nx, int ny, int pitch, T *k0, T *psiA, T *psiB, MgCtl *
                      const MgHost<T> *share_coef = nullptr);  // FP64: use its coefficient planes
 template <typename T>
 void mg_destroy(MgHost<T> *m);
-// One V-cycle = head (lattice residual; decides whether the cycle runs) +
-// rest (launched only when the head said so: graph if node or host check).
-template <typename T>
-void mg_cycle_head(MgHost<T> *m, T H0c, T H0s, cudaGraphConditionalHandle hwhile,
+// Solves of several kernels (the single FP32 plane). One V-cycle = head (lattice
+// residual; decides whether the cycle runs) + rest (launched only when the head
+// said so: graph if node or host check).
+void mg_cycle_head(MgHost<float> *m, float H0c, float H0s, cudaGraphConditionalHandle hwhile,
                    cudaGraphConditionalHandle hif, int in_graph, cudaStream_t s);
+void mg_cycle_rest(MgHost<float> *m, float H0c, float H0s, cudaStream_t s);
+void mg_cycle_smooth(MgHost<float> *m, float H0c, float H0s, cudaStream_t s);
+void mg_cycle_twogrid(MgHost<float> *m, float H0c, float H0s, cudaStream_t s);
+void mg_presmooth(MgHost<float> *m, float H0c, float H0s, cudaStream_t s);  // opens every such solve
+int mg_kernels_per_cycle(const MgHost<float> *m);
+// Whole solve as one cooperative kernel (FP64 and the FP32 pair): whether the
+// hierarchy takes it, its launch, and the share of the GPU it may fill (1 /
+// share of the SMs: solves that run side by side).
 template <typename T>
-void mg_cycle_rest(MgHost<T> *m, T H0c, T H0s, cudaStream_t s);
+bool mg_one_kernel(const MgHost<T> *m);
 template <typename T>
-void mg_cycle_smooth(MgHost<T> *m, T H0c, T H0s, cudaStream_t s);
+cudaError_t mg_solve(MgHost<T> *m, T H0c, T H0s, cudaStream_t s);
 template <typename T>
-void mg_cycle_twogrid(MgHost<T> *m, T H0c, T H0s, cudaStream_t s);
-template <typename T>
-void mg_presmooth(MgHost<T> *m, T H0c, T H0s, cudaStream_t s);  // opens every solve
-template <typename T>
-int mg_kernels_per_cycle(const MgHost<T> *m);
+void mg_set_share(MgHost<T> *m, int share);
 // Graph form of the cycle loop: a one-thread kernel at the top of the loop body
 // that sets the body's switch node from the mode the last head chose.
-template <typename T>
-void mg_cycle_dispatch(MgHost<T> *m, cudaGraphConditionalHandle hswitch, cudaStream_t s);
+void mg_cycle_dispatch(MgHost<float> *m, cudaGraphConditionalHandle hswitch, cudaStream_t s);
 // Tangent solves (FP64): explicit right-hand side on level 0; reset of the
 // control block with tolerance tol * max|rhs|; right-hand side along one
 // direction, L(k) dpsi' = b(k, dH0) + b(dk, H0) - L(dk) psi'; copies between
@@ -345,6 +368,8 @@ int mg_levels(const MgHost<T> *m);
 // Batched solves of many FP32 hierarchies (one per instance; fields and
 // control blocks stay the instances' own): opening sweeps of every solve, and
 // the body of the loop that runs until every solve is done.
+// FP32 hierarchies of the single-plane form only (the pair's solves are one
+// kernel each).
 struct MgBatch;
 MgBatch *mg_batch_create(const std::vector<MgHost<float> *> &ms, const std::vector<float> &H0c,
                          const std::vector<float> &H0s, void *(*alloc)(size_t, void *),
@@ -443,6 +468,8 @@ struct EngineView {
 };
 // false (and v untouched) for any other context
 bool engine_view(fcd_ctx *c, EngineView *v);
+// the context's solves run beside those of other contexts (1 / share of the SMs)
+void engine_share(fcd_ctx *c, int share);
 // the host-side record of a context after `steps` steps run by the batch
 void engine_advance(fcd_ctx *c, long steps);
 // one step of a context on its own stream; store_macro: also store u and p*

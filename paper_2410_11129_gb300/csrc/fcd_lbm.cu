@@ -33,19 +33,7 @@ __device__ __forceinline__ void phase_tile(const Phys<T> &P, const void *gv, T *
     using S = typename StoreT<MODE>::type;
     if (pc.ctl && lead && threadIdx.x == 0 && threadIdx.y == 0) {
         MgCtl *c = pc.ctl;
-        if (pc.reset) {  // start of a potential solve
-            c->norm_bits = 0ull;
-            c->iter = 0;
-            c->done = 0;
-            c->converged = 0;
-            c->tolH0 = pc.tolH0;
-            c->max_iter = pc.max_iter;
-            c->keep_going = 1;
-            c->blocks_done = 0u;
-            c->mode = 1;         // the opening sweeps count as a lattice-sweep cycle
-            c->smooth_left = 0;  // ... and use up the sweep allowance
-            c->twogrid_left = 2;
-        }
+        if (pc.reset) mg_reset_ctl(c, pc.tolH0, pc.max_iter);  // start of a potential solve
         if (pc.step) {
             c->step_cur = *pc.step;
             *pc.step += 1;

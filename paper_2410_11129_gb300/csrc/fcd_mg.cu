@@ -14,9 +14,14 @@
 // type, forms the residual that is restricted and adds the interpolated
 // correction, so the coarse precision only perturbs each cycle's contraction,
 // not the converged potential; on this GPU FP64 arithmetic is 1/58 of FP32, and
-// the single-block coarse levels are bound by one SM's arithmetic. Cycles are V(0, 2) on level 0 and V(2, 2)
-// below; residuals are summed onto the coarse cells and corrections are
-// interpolated bilinearly between cell centres (zero on the walls).
+// the single-block coarse levels are bound by one SM's arithmetic. Residuals are
+// summed onto the coarse cells and corrections are interpolated bilinearly
+// between cell centres (zero on the walls).
+//
+// FP64 contexts and FP32 contexts with the hi + lo pair solve in one cooperative
+// kernel (fcd_mg_solve.cuh). The kernels of this file below it serve the single
+// FP32 plane, whose solves mostly end at their first residual, with cycles V(0, 2)
+// on level 0 and V(2, 2) below.
 //
 // Level 0 is smoothed by block Gauss-Seidel: each 32 x 8 tile loads its cells
 // with a one-cell frozen halo into shared memory, adds the interpolated coarse
@@ -61,6 +66,7 @@ constexpr double SMOOTH_RATIO = 2.5;
 constexpr int NU_SMOOTH_ONLY = 1, NU_TWOGRID = 2;
 constexpr size_t CTA_SMEM_MAX = 200 * 1024;  // shared memory of the single-block levels
 constexpr size_t CTA_CELLS = 2048;            // cells of the single-block levels
+constexpr size_t SOLVE_CELLS = 3072;          // the same in the one-kernel solve
 using TC = float;                             // type of the coarse levels (>= 1)
 
 __device__ __forceinline__ double norm_of(const MgCtl *c) {
@@ -257,42 +263,12 @@ __device__ __forceinline__ void comp_add(float &hi, float &lo, float v) {
 }
 
 // FP64 hierarchies keep the lattice level's node coefficients in COEF planes,
-// formed once per solve by coef0_kernel (k does not change within a solve):
-// the FP64 arithmetic of node9 and its division cost more than the loads on
-// this GPU (FP64 is 1/58 of FP32). FP32 hierarchies form them on the fly.
-constexpr int COEF = 11;  // c_1..c_8, diag, 1/diag, b
+// formed once per solve (k does not change within a solve): the FP64 arithmetic
+// of node9 costs more than the loads on this GPU (FP64 is 1/58 of FP32). FP32
+// hierarchies form them on the fly.
+constexpr int COEF = 10;  // c_1..c_8, diag, b
 template <typename T>
 __host__ __device__ constexpr bool keeps_coef() { return sizeof(T) == 8; }
-
-template <typename T>
-__device__ __forceinline__ void coef_load(const Level<T> &L0, long long n, Node9<T> &nd, T &inv) {
-    const long long ps = (long long)L0.pitch * L0.ny;
-#pragma unroll
-    for (int a = 1; a < 9; a++) nd.c[a] = L0.coef[(a - 1) * ps + n];
-    nd.diag = L0.coef[8 * ps + n];
-    inv = L0.coef[9 * ps + n];
-    nd.b = L0.coef[10 * ps + n];
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) coef0_kernel(Level<T> L0, T H0c, T H0s) {
-    const int nx = L0.nx, ny = L0.ny, pitch = L0.pitch;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= nx || y >= ny) return;
-    auto kat = [&](int dx, int dy) {
-        int xx = x + dx;
-        xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
-        const int yy = y + dy < 0 ? 0 : (y + dy >= ny ? ny - 1 : y + dy);  // mirrored ghost rows
-        return L0.k[(long long)yy * pitch + xx];
-    };
-    const Node9<T> nd = node9<T>(kat, y, ny, H0c, H0s);
-    const long long ps = (long long)pitch * ny, n = (long long)y * pitch + x;
-#pragma unroll
-    for (int a = 1; a < 9; a++) L0.coef[(a - 1) * ps + n] = nd.c[a];
-    L0.coef[8 * ps + n] = nd.diag;
-    L0.coef[9 * ps + n] = T(1) / nd.diag;
-    L0.coef[10 * ps + n] = nd.b;
-}
 
 // Interpolation weights of a tile's columns and rows, staged in shared memory.
 template <typename T, int NXT, int NYT>
@@ -350,9 +326,8 @@ __device__ void cycle_decide(MgCtl *ctl, cudaGraphConditionalHandle hw,
 constexpr int RX = 2 * 32 + 1 + 2, RY = 2 * 8 + 1 + 2;
 
 // One 32 x 8 block of level-1 cells (bx, by) of a grid of nblocks blocks;
-// grid_lead: the block that reports a solve that is already done. SPLIT as
-// for the smoothing tiles.
-template <typename T, bool COMP, bool SPLIT = true>
+// grid_lead: the block that reports a solve that is already done.
+template <typename T>
 __device__ __forceinline__ void resid0_tile(const Level<T> &L0, const Level<TC> &L1, T H0c, T H0s,
                                             MgCtl *ctl, cudaGraphConditionalHandle hw,
                                             cudaGraphConditionalHandle hi, int in_graph, int bx,
@@ -362,11 +337,8 @@ __device__ __forceinline__ void resid0_tile(const Level<T> &L0, const Level<TC> 
         if (lead && grid_lead) cycle_decide(ctl, hw, hi, in_graph);
         return;
     }
-    static_assert(!COMP || sizeof(T) == 4, "the hi + lo pair is an FP32 form");
     __shared__ T sk[RY][RX], sp[RY][RX];
-    __shared__ T sl[COMP ? RY : 1][COMP ? RX : 1];  // lo part of psi' (FP32 level 0)
     const int nx = L0.nx, ny = L0.ny, pitch = L0.pitch;
-    const long long lo_off = (long long)pitch * ny;
     const int I0 = bx * 32, J0 = by * 8;
     const int I1 = min(I0 + 32, L1.nx), J1 = min(J0 + 8, L1.ny);
     const int fx0 = L1.cx0[I0], fx1 = L1.cx0[I1], fy0 = L1.cy0[J0], fy1 = L1.cy0[J1];
@@ -384,7 +356,7 @@ __device__ __forceinline__ void resid0_tile(const Level<T> &L0, const Level<TC> 
             while (gx >= nx) gx -= nx;
             gxs[c] = gx;
         }
-        T kv[NR][NC], pv[NR][NC], lv[COMP ? NR : 1][COMP ? NC : 1];
+        T kv[NR][NC], pv[NR][NC];
 #pragma unroll
         for (int r = 0; r < NR; r++) {
             const int ly = warp + 8 * r, gy = fy0 - 1 + ly;
@@ -393,12 +365,10 @@ __device__ __forceinline__ void resid0_tile(const Level<T> &L0, const Level<TC> 
             for (int c = 0; c < NC; c++) {
                 kv[r][c] = T(0);
                 pv[r][c] = T(0);
-                if constexpr (COMP) lv[r][c] = T(0);
                 if (ly < wy && lane + 32 * c < wx) {
                     const long long m = (long long)my * pitch + gxs[c];
                     kv[r][c] = L0.k[m];  // mirrored ghost rows
                     pv[r][c] = psi[m];   // ghost rows never read
-                    if constexpr (COMP) lv[r][c] = psi[lo_off + m];
                 }
             }
         }
@@ -410,7 +380,6 @@ __device__ __forceinline__ void resid0_tile(const Level<T> &L0, const Level<TC> 
                 if (ly < wy && lx < wx) {
                     sk[ly][lx] = kv[r][c];
                     sp[ly][lx] = pv[r][c];
-                    if constexpr (COMP) sl[ly][lx] = lv[r][c];
                 }
             }
     }
@@ -426,24 +395,8 @@ __device__ __forceinline__ void resid0_tile(const Level<T> &L0, const Level<TC> 
             const int lx = i - fx0 + 1, ly = j - fy0 + 1;
             auto kat = [&](int dx, int dy) { return sk[ly + dy][lx + dx]; };
             auto pat = [&](int dx, int dy) { return sp[ly + dy][lx + dx]; };
-            T r;
-            if constexpr (COMP) {
-                auto lat = [&](int dx, int dy) { return sl[ly + dy][lx + dx]; };
-                Node9<float> nd = node9_pairs<W>(kat, j, ny, H0c, H0s);
-                if (L0.rhs) nd.b = L0.rhs[(long long)j * pitch + i];
-                r = resid_pairs<W>(nd, pat, lat, j, ny);
-            } else {
-                Node9<T> nd;
-                if constexpr (keeps_coef<T>()) {
-                    T inv;
-                    coef_load(L0, (long long)j * pitch + i, nd, inv);
-                    (void)kat;
-                } else {
-                    nd = node9<T, W>(kat, j, ny, H0c, H0s);
-                }
-                const T bb = L0.rhs ? L0.rhs[(long long)j * pitch + i] : nd.b;
-                r = bb - (off9<T, W>(nd, pat, j, ny) - nd.diag * sp[ly][lx]);
-            }
+            const Node9<T> nd = node9<T, W>(kat, j, ny, H0c, H0s);
+            const T r = nd.b - (off9<T, W>(nd, pat, j, ny) - nd.diag * sp[ly][lx]);
             sum += r;
             ksum += sk[ly][lx];
             const T ar = fabs(r);
@@ -462,7 +415,7 @@ __device__ __forceinline__ void resid0_tile(const Level<T> &L0, const Level<TC> 
         L1.b[(long long)J * L1.pitch + I] = TC(sum);
         L1.k[(long long)J * L1.pitch + I] = TC(ksum / (T(L1.wx[I]) * T(L1.wy[J])));  // unit lattice cells
     };
-    if (!SPLIT || fy0 == 0 || fy1 >= ny) cells(std::true_type{});
+    if (fy0 == 0 || fy1 >= ny) cells(std::true_type{});
     else cells(std::false_type{});
     for (int o = 16; o > 0; o >>= 1) mxt = fmax(mxt, __shfl_xor_sync(0xffffffffu, mxt, o));
     __shared__ T wmax[8];  // one per warp (blockDim 32 x 8)
@@ -479,11 +432,11 @@ __device__ __forceinline__ void resid0_tile(const Level<T> &L0, const Level<TC> 
     }
 }
 
-template <typename T, bool COMP>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 4) resid0_restrict(Level<T> L0, Level<TC> L1, T H0c, T H0s,
+template <typename T>
+__global__ void __launch_bounds__(256, 5) resid0_restrict(Level<T> L0, Level<TC> L1, T H0c, T H0s,
                                                        MgCtl *ctl, cudaGraphConditionalHandle hw,
                                                        cudaGraphConditionalHandle hi, int in_graph) {
-    resid0_tile<T, COMP>(L0, L1, H0c, H0s, ctl, hw, hi, in_graph, blockIdx.x, blockIdx.y,
+    resid0_tile<T>(L0, L1, H0c, H0s, ctl, hw, hi, in_graph, blockIdx.x, blockIdx.y,
                          gridDim.x * gridDim.y, blockIdx.x == 0 && blockIdx.y == 0);
 }
 
@@ -499,22 +452,19 @@ constexpr int QT = (SX / 2) * (SY / 2);  // threads of a smoothing tile
 static_assert(QT % 32 == 0 && 2 * (SY + 2) <= QT, "tile load layout");
 constexpr int TILE_ROWS = (SY + 2 + QT / 32 - 1) / (QT / 32);  // ring rows per warp
 
-// One 32 x 8 tile (bx, by) of a grid of nblocks tiles. SPLIT: tiles without a
-// wall row take a second copy of the sweeps that skips the ghost tests (fewer
-// instructions; the batched kernels keep one copy to bound their registers).
-template <typename T, bool COMP, bool SPLIT = true>
+// One 32 x 8 tile (bx, by) of a grid of nblocks tiles. Tiles without a wall row
+// take a second copy of the sweeps that skips the ghost tests (fewer
+// instructions).
+template <typename T>
 __device__ __forceinline__ void smooth0_tile(const Level<T> &L0, const Level<TC> &L1,
                                              int add_coarse, int sweeps, T H0c, T H0s, MgCtl *ctl,
                                              int first, int bx, int by, unsigned nblocks) {
     const int tid = threadIdx.x;
     // first: the sweeps that open a solve (no residual known yet)
     if (block_skip(ctl, first != 0)) return;
-    static_assert(!COMP || sizeof(T) == 4, "the hi + lo pair is an FP32 form");
     __shared__ T sp[SY + 2][SX + 2];
-    __shared__ T sl[COMP ? SY + 2 : 1][COMP ? SX + 2 : 1];  // lo part of psi' (FP32)
     __shared__ T sk[SY + 2][SX + 2];
     const int nx = L0.nx, ny = L0.ny, pitch = L0.pitch;
-    const long long lo_off = (long long)pitch * ny;
     const int x0 = bx * SX, y0 = by * SY;
     const T *src = ctl->cur ? L0.r : L0.e;
     T *dst = ctl->cur ? L0.e : L0.r;
@@ -532,7 +482,7 @@ __device__ __forceinline__ void smooth0_tile(const Level<T> &L0, const Level<TC>
         const int gxa = wrap(x0 - 1 + lane);
         const bool extra = tid < 2 * (SY + 2);
         const int ey = tid >> 1, ex = SX + (tid & 1), gxe = wrap(x0 - 1 + ex);
-        T kv[TILE_ROWS + 1], pv[TILE_ROWS + 1], lv[COMP ? TILE_ROWS + 1 : 1];
+        T kv[TILE_ROWS + 1], pv[TILE_ROWS + 1];
 #pragma unroll
         for (int q = 0; q <= TILE_ROWS; q++) {
             const int ly = q < TILE_ROWS ? warp + q * (QT / 32) : ey;
@@ -540,15 +490,11 @@ __device__ __forceinline__ void smooth0_tile(const Level<T> &L0, const Level<TC>
             const bool act = q < TILE_ROWS ? ly < SY + 2 : extra;
             kv[q] = T(0);
             pv[q] = T(0);
-            if constexpr (COMP) lv[q] = T(0);
             if (act) {
                 const int gy = y0 - 1 + ly;
                 const int my = gy < 0 ? 0 : (gy >= ny ? ny - 1 : gy);
                 kv[q] = L0.k[(long long)my * pitch + gx];
-                if (gy >= 0 && gy < ny) {
-                    pv[q] = src[(long long)gy * pitch + gx];
-                    if constexpr (COMP) lv[q] = src[lo_off + (long long)gy * pitch + gx];
-                }
+                if (gy >= 0 && gy < ny) pv[q] = src[(long long)gy * pitch + gx];
             }
         }
 #pragma unroll
@@ -558,7 +504,6 @@ __device__ __forceinline__ void smooth0_tile(const Level<T> &L0, const Level<TC>
             if (q < TILE_ROWS ? ly < SY + 2 : extra) {
                 sk[ly][lx] = kv[q];
                 sp[ly][lx] = pv[q];
-                if constexpr (COMP) sl[ly][lx] = lv[q];
             }
         }
     }
@@ -566,10 +511,7 @@ __device__ __forceinline__ void smooth0_tile(const Level<T> &L0, const Level<TC>
     if (add_coarse) {  // ghost rows are never read: the mirror is used instead
         for (int t = tid; t < (SX + 2) * (SY + 2); t += QT) {
             const int lx = t % (SX + 2), ly = t / (SX + 2), gy = y0 - 1 + ly;
-            if (gy >= 0 && gy < ny) {
-                if constexpr (COMP) comp_add(sp[ly][lx], sl[ly][lx], prolong_at(pt, L1, lx, ly));
-                else sp[ly][lx] += prolong_at(pt, L1, lx, ly);
-            }
+            if (gy >= 0 && gy < ny) sp[ly][lx] += prolong_at(pt, L1, lx, ly);
         }
         __syncthreads();
     }
@@ -587,15 +529,9 @@ __device__ __forceinline__ void smooth0_tile(const Level<T> &L0, const Level<TC>
             own[c] = x < nx && y < ny;
             inv_diag[c] = T(0);
             if (own[c]) {
-                if constexpr (keeps_coef<T>()) {
-                    coef_load(L0, (long long)y * pitch + x, nd[c], inv_diag[c]);
-                } else {
-                    auto kat = [&](int dx, int dy) { return sk[ly + dy][lx + dx]; };
-                    if constexpr (COMP) nd[c] = node9_pairs<W>(kat, y, ny, H0c, H0s);
-                    else nd[c] = node9<T, W>(kat, y, ny, H0c, H0s);
-                    inv_diag[c] = T(1) / nd[c].diag;
-                }
-                if (L0.rhs) nd[c].b = L0.rhs[(long long)y * pitch + x];
+                auto kat = [&](int dx, int dy) { return sk[ly + dy][lx + dx]; };
+                nd[c] = node9<T, W>(kat, y, ny, H0c, H0s);
+                inv_diag[c] = T(1) / nd[c].diag;
             }
         }
         for (int s = 0; s < sweeps; s++) {
@@ -603,15 +539,7 @@ __device__ __forceinline__ void smooth0_tile(const Level<T> &L0, const Level<TC>
             for (int c = 0; c < 4; c++) {
                 const int lx = qx + (c & 1) + 1, ly = qy + (c >> 1) + 1, y = y0 + ly - 1;
                 auto pat = [&](int dx, int dy) { return sp[ly + dy][lx + dx]; };
-                if (own[c]) {
-                    if constexpr (COMP) {  // correction form: dr/dpsi'_0 = diag, so psi'_0 -= r_0 / diag
-                        auto lat = [&](int dx, int dy) { return sl[ly + dy][lx + dx]; };
-                        const float r = resid_pairs<W>(nd[c], pat, lat, y, ny);
-                        comp_add(sp[ly][lx], sl[ly][lx], -r * inv_diag[c]);
-                    } else {
-                        sp[ly][lx] = (off9<T, W>(nd[c], pat, y, ny) - nd[c].b) * inv_diag[c];
-                    }
-                }
+                if (own[c]) sp[ly][lx] = (off9<T, W>(nd[c], pat, y, ny) - nd[c].b) * inv_diag[c];
                 __syncthreads();
             }
         }
@@ -621,11 +549,10 @@ __device__ __forceinline__ void smooth0_tile(const Level<T> &L0, const Level<TC>
             if (own[c]) {
                 const long long n = (long long)(y0 + ly - 1) * pitch + (x0 + lx - 1);
                 dst[n] = sp[ly][lx];
-                if constexpr (COMP) dst[lo_off + n] = sl[ly][lx];
             }
         }
     };
-    if (!SPLIT || y0 == 0 || y0 + SY >= ny) sweep_tile(std::true_type{});
+    if (y0 == 0 || y0 + SY >= ny) sweep_tile(std::true_type{});
     else sweep_tile(std::false_type{});
     __syncthreads();
     if (tid == 0) {
@@ -634,39 +561,24 @@ __device__ __forceinline__ void smooth0_tile(const Level<T> &L0, const Level<TC>
     }
 }
 
-template <typename T, bool COMP>
+template <typename T>
 __global__ void __launch_bounds__(QT) smooth0(Level<T> L0, Level<TC> L1, int add_coarse,
                                               int sweeps, T H0c, T H0s, MgCtl *ctl, int first) {
-    smooth0_tile<T, COMP>(L0, L1, add_coarse, sweeps, H0c, H0s, ctl, first, blockIdx.x, blockIdx.y,
+    smooth0_tile<T>(L0, L1, add_coarse, sweeps, H0c, H0s, ctl, first, blockIdx.x, blockIdx.y,
                           gridDim.x * gridDim.y);
 }
 
-// Host-side dispatch on the lattice level's form (FP32: one plane or the pair).
-template <typename T>
-static void launch_smooth0(const Level<T> &L0, const Level<TC> &L1, int add, int sweeps, T H0c,
-                           T H0s, MgCtl *ctl, int first, cudaStream_t s) {
+static void launch_smooth0(const Level<float> &L0, const Level<TC> &L1, int add, int sweeps, float H0c, float H0s,
+                           MgCtl *ctl, int first, cudaStream_t s) {
     const dim3 g((L0.nx + SX - 1) / SX, (L0.ny + SY - 1) / SY);
-    if constexpr (sizeof(T) == 4) {
-        if (L0.comp) {
-            smooth0<T, true><<<g, QT, 0, s>>>(L0, L1, add, sweeps, H0c, H0s, ctl, first);
-            return;
-        }
-    }
-    smooth0<T, false><<<g, QT, 0, s>>>(L0, L1, add, sweeps, H0c, H0s, ctl, first);
+    smooth0<float><<<g, QT, 0, s>>>(L0, L1, add, sweeps, H0c, H0s, ctl, first);
 }
 
-template <typename T>
-static void launch_resid0(const Level<T> &L0, const Level<TC> &L1, T H0c, T H0s, MgCtl *ctl,
+static void launch_resid0(const Level<float> &L0, const Level<TC> &L1, float H0c, float H0s, MgCtl *ctl,
                           cudaGraphConditionalHandle hw, cudaGraphConditionalHandle hi, int in_graph,
                           cudaStream_t s) {
     const dim3 b(32, 8), g((L1.nx + 31) / 32, (L1.ny + 7) / 8);
-    if constexpr (sizeof(T) == 4) {
-        if (L0.comp) {
-            resid0_restrict<T, true><<<g, b, 0, s>>>(L0, L1, H0c, H0s, ctl, hw, hi, in_graph);
-            return;
-        }
-    }
-    resid0_restrict<T, false><<<g, b, 0, s>>>(L0, L1, H0c, H0s, ctl, hw, hi, in_graph);
+    resid0_restrict<float><<<g, b, 0, s>>>(L0, L1, H0c, H0s, ctl, hw, hi, in_graph);
 }
 
 // ------------------------------------------------------------- coarse levels
@@ -845,6 +757,56 @@ __device__ __forceinline__ void cta_gs(const Level<T> &L, const CtaView<T> &V, i
         }
 }
 
+// V(1,1) over levels lc .. nl - 1, all in the block's shared memory.
+template <typename T>
+__device__ __forceinline__ void cta_vcycle(T *sm, const int *off, const Level<T> *L, int lc, int nl, int tid,
+                                           int nthr) {
+    // V-cycle: down
+    for (int l = lc; l < nl - 1; l++) {
+        const CtaView<T> F = cta_view(sm, off, L, l), V = cta_view(sm, off, L, l + 1);
+        cta_gs(L[l], F, NU_CTA, tid, nthr, false);
+        const Level<T> &C = L[l + 1];
+        const int fnx = L[l].nx, fny = L[l].ny;
+        for (int t = tid; t < C.nx * C.ny; t += nthr) {
+            const int I = t % C.nx, J = t / C.nx;
+            T s = T(0);
+            for (int j = C.cy0[J]; j < C.cy0[J + 1]; j++)
+                for (int i = C.cx0[I]; i < C.cx0[I + 1]; i++) {
+                    const int q = j * fnx + i;
+                    const int iw = i == 0 ? fnx - 1 : i - 1, ie = i + 1 == fnx ? 0 : i + 1;
+                    T v = F.te[q] * F.e[j * fnx + ie] + F.te[j * fnx + iw] * F.e[j * fnx + iw];
+                    if (j + 1 < fny) v += F.tn[q] * F.e[q + fnx];
+                    if (j > 0) v += F.tn[q - fnx] * F.e[q - fnx];
+                    s += F.b[q] - (v - F.e[q] / F.dg[q]);
+                }
+            V.b[t] = s;
+            V.e[t] = T(0);
+        }
+        __syncthreads();
+    }
+    {  // coarsest (<= 100 cells, walls at most a few cells away: GS converges fast)
+        const CtaView<T> V = cta_view(sm, off, L, nl - 1);
+        cta_gs(L[nl - 1], V, NU_COARSEST, tid, nthr, false);
+    }
+    // up
+    for (int l = nl - 2; l >= lc; l--) {
+        const CtaView<T> F = cta_view(sm, off, L, l), V = cta_view(sm, off, L, l + 1);
+        const Level<T> &Fl = L[l];
+        for (int t = tid; t < Fl.nx * Fl.ny; t += nthr) {
+            const int i = t % Fl.nx, j = t / Fl.nx;
+            const int x0 = Fl.px0[i], x1 = Fl.px1[i], y0 = Fl.py0[j], y1 = Fl.py1[j];
+            const T wx = Fl.pwx[i], wy = Fl.pwy[j];
+            const int cnx = L[l + 1].nx;
+            T a = T(0), b = T(0);
+            if (y0 >= 0) a = (T(1) - wx) * V.e[y0 * cnx + x0] + wx * V.e[y0 * cnx + x1];
+            if (y1 >= 0) b = (T(1) - wx) * V.e[y1 * cnx + x0] + wx * V.e[y1 * cnx + x1];
+            F.e[t] += (T(1) - wy) * a + wy * b;
+        }
+        __syncthreads();
+        cta_gs(L[l], F, NU_CTA, tid, nthr, false);
+    }
+}
+
 template <typename T>
 __device__ __forceinline__ void coarse_cta_block(const Level<T> *lv, int lc, int nl, MgCtl *ctl) {
     if (cycle_skip(ctl)) return;
@@ -902,50 +864,7 @@ __device__ __forceinline__ void coarse_cta_block(const Level<T> *lv, int lc, int
         }
     }
     __syncthreads();
-    // V-cycle: down
-    for (int l = lc; l < nl - 1; l++) {
-        const CtaView<T> F = cta_view(sm, off, L, l), V = cta_view(sm, off, L, l + 1);
-        cta_gs(L[l], F, NU_CTA, tid, nthr, false);
-        const Level<T> &C = L[l + 1];
-        const int fnx = L[l].nx, fny = L[l].ny;
-        for (int t = tid; t < C.nx * C.ny; t += nthr) {
-            const int I = t % C.nx, J = t / C.nx;
-            T s = T(0);
-            for (int j = C.cy0[J]; j < C.cy0[J + 1]; j++)
-                for (int i = C.cx0[I]; i < C.cx0[I + 1]; i++) {
-                    const int q = j * fnx + i;
-                    const int iw = i == 0 ? fnx - 1 : i - 1, ie = i + 1 == fnx ? 0 : i + 1;
-                    T v = F.te[q] * F.e[j * fnx + ie] + F.te[j * fnx + iw] * F.e[j * fnx + iw];
-                    if (j + 1 < fny) v += F.tn[q] * F.e[q + fnx];
-                    if (j > 0) v += F.tn[q - fnx] * F.e[q - fnx];
-                    s += F.b[q] - (v - F.e[q] / F.dg[q]);
-                }
-            V.b[t] = s;
-            V.e[t] = T(0);
-        }
-        __syncthreads();
-    }
-    {  // coarsest (<= 100 cells, walls at most a few cells away: GS converges fast)
-        const CtaView<T> V = cta_view(sm, off, L, nl - 1);
-        cta_gs(L[nl - 1], V, NU_COARSEST, tid, nthr, false);
-    }
-    // up
-    for (int l = nl - 2; l >= lc; l--) {
-        const CtaView<T> F = cta_view(sm, off, L, l), V = cta_view(sm, off, L, l + 1);
-        const Level<T> &Fl = L[l];
-        for (int t = tid; t < Fl.nx * Fl.ny; t += nthr) {
-            const int i = t % Fl.nx, j = t / Fl.nx;
-            const int x0 = Fl.px0[i], x1 = Fl.px1[i], y0 = Fl.py0[j], y1 = Fl.py1[j];
-            const T wx = Fl.pwx[i], wy = Fl.pwy[j];
-            const int cnx = L[l + 1].nx;
-            T a = T(0), b = T(0);
-            if (y0 >= 0) a = (T(1) - wx) * V.e[y0 * cnx + x0] + wx * V.e[y0 * cnx + x1];
-            if (y1 >= 0) b = (T(1) - wx) * V.e[y1 * cnx + x0] + wx * V.e[y1 * cnx + x1];
-            F.e[t] += (T(1) - wy) * a + wy * b;
-        }
-        __syncthreads();
-        cta_gs(L[l], F, NU_CTA, tid, nthr, false);
-    }
+    cta_vcycle(sm, off, L, lc, nl, tid, nthr);
     {
         const CtaView<T> V = cta_view(sm, off, L, lc);
         const int nx = L[lc].nx, n = nx * L[lc].ny;
@@ -1020,6 +939,12 @@ __device__ void cycle_close(MgCtl *ctl) {
     ctl->norm_bits = 0ull;
 }
 
+}  // namespace fcd
+
+#include "fcd_mg_solve.cuh"
+
+namespace fcd {
+
 // ------------------------------------------------------------------ host side
 template <typename T>
 struct MgHost {
@@ -1034,6 +959,10 @@ struct MgHost {
     void (*release)(void *, void *) = nullptr;
     void *user = nullptr;
     size_t cta_smem = 0;
+    // the one-kernel form: its first single-block level, shared memory, blocks
+    int solve_lc = 0, solve_blocks = 0, sms = 0;
+    TC *corr = nullptr;  // its lattice planes: residual, correction (two), k
+    size_t solve_smem = 0;
 };
 
 static std::vector<int> merge_faces(int n) {
@@ -1090,6 +1019,68 @@ static void interp_table(const std::vector<double> &fine, const std::vector<doub
 }
 
 template <typename T>
+bool mg_one_kernel(const MgHost<T> *m) { return keeps_coef<T>() || m->L0.comp; }
+
+template <typename T>
+static const void *solve_kernel(const MgHost<T> *m) {
+    if constexpr (sizeof(T) == 4) {
+        (void)m;
+        return reinterpret_cast<const void *>(&mg_solve_kernel<float, true>);
+    } else {
+        return reinterpret_cast<const void *>(&mg_solve_kernel<T, false>);
+    }
+}
+
+// Blocks: at most one per SM (all must be resident), at most one per tile.
+template <typename T>
+void mg_set_share(MgHost<T> *m, int share) {
+    const int tiles = ((m->L0.nx + SX - 1) / SX) * ((m->L0.ny + SY - 1) / SY);
+    m->solve_blocks = std::max(1, std::min(tiles, m->sms / std::max(1, share)));
+}
+
+template <typename T>
+static bool solve_setup(MgHost<T> *m) {
+    int dev = 0, coop = 0, fit = 0;
+    size_t bottom = 0;
+    for (int q = m->solve_lc; q < m->nl; q++)
+        bottom += (size_t)BOTTOM_ARRAYS * m->lv[q].nx * m->lv[q].ny * sizeof(TC);
+    m->solve_smem = bottom + (sizeof(T) == 4 ? solve_tiles_bytes<float, true>() : solve_tiles_bytes<double, false>());
+    const void *k = solve_kernel(m);
+    // the limit is the kernel's, shared by every context: the budget, not this need
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
+        cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        m->solve_smem > CTA_SMEM_MAX ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CTA_SMEM_MAX) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k, SOLVE_THREADS, m->solve_smem) != cudaSuccess ||
+        fit < 1)
+        return false;
+    mg_set_share(m, 1);
+    return true;
+}
+
+template <typename T>
+cudaError_t mg_solve(MgHost<T> *m, T H0c, T H0s, cudaStream_t s) {
+    SolveArgs<T> A;
+    A.L0 = m->L0;
+    A.lv = m->d_lv;
+    A.nl = m->nl;
+    A.lc = m->solve_lc;
+    A.H0c = H0c;
+    A.H0s = H0s;
+    A.ctl = m->ctl;
+    A.form_coef = m->coef_shared ? 0 : 1;
+    const size_t ps = (size_t)m->L0.pitch * m->L0.ny;
+    A.r0 = m->corr;
+    A.eA = m->corr + ps;
+    A.eB = m->corr + 2 * ps;
+    A.k0 = m->corr + 3 * ps;
+    void *args[] = {&A};
+    return cudaLaunchCooperativeKernel(solve_kernel(m), dim3(m->solve_blocks), dim3(SOLVE_THREADS), args,
+                                       m->solve_smem, s);
+}
+
+template <typename T>
 MgHost<T> *mg_create(int nx, int ny, int pitch, T *k0, T *psiA, T *psiB, MgCtl *ctl,
                      void *(*alloc)(size_t, void *), void (*release)(void *, void *), void *user,
                      char *err, size_t errlen, int comp, const MgHost<T> *share_coef) {
@@ -1140,6 +1131,13 @@ MgHost<T> *mg_create(int nx, int ny, int pitch, T *k0, T *psiA, T *psiB, MgCtl *
     }
     m->cta_smem = 0;
     for (int q = m->lc; q < m->nl; q++) m->cta_smem += (size_t)CTA_ARRAYS * xcs[q].size() * ycs[q].size() * sizeof(TC);
+    m->solve_lc = m->nl - 1;
+    for (int l = m->nl - 1; l >= 1; l--) {
+        size_t cells = 0;
+        for (int q = l; q < m->nl; q++) cells += xcs[q].size() * ycs[q].size();
+        if (cells > SOLVE_CELLS) break;
+        m->solve_lc = l;
+    }
     if (m->nl > MAX_LEVELS || m->cta_smem > CTA_SMEM_MAX) {
         snprintf(err, errlen, "multigrid: hierarchy too deep or coarse levels too large");
         mg_destroy(m);
@@ -1234,6 +1232,12 @@ MgHost<T> *mg_create(int nx, int ny, int pitch, T *k0, T *psiA, T *psiB, MgCtl *
         L.cy0 = up.put<int>(cy0[l].data(), cy0[l].size() * sizeof(int));
     }
     m->d_lv = up.put<Level<TC>>(m->lv.data(), m->lv.size() * sizeof(Level<TC>));
+    if (mg_one_kernel(m)) m->corr = up.put<TC>(nullptr, 4 * (size_t)pitch * ny * sizeof(TC));
+    if (up.ok && mg_one_kernel(m) && !solve_setup(m)) {
+        snprintf(err, errlen, "multigrid: the cooperative solve cannot be launched on this device");
+        mg_destroy(m);
+        return nullptr;
+    }
     if (!up.ok) {
         snprintf(err, errlen, "multigrid: device allocation or upload failed");
         mg_destroy(m);
@@ -1251,20 +1255,17 @@ void mg_destroy(MgHost<T> *m) {
 
 static dim3 g2(int nx, int ny, dim3 b) { return dim3((nx + b.x - 1) / b.x, (ny + b.y - 1) / b.y); }
 
-template <typename T>
-void mg_cycle_dispatch(MgHost<T> *m, cudaGraphConditionalHandle hs, cudaStream_t s) {
+void mg_cycle_dispatch(MgHost<float> *m, cudaGraphConditionalHandle hs, cudaStream_t s) {
     cycle_dispatch_kernel<<<1, 32, 0, s>>>(m->ctl, hs);
 }
 
-template <typename T>
-void mg_cycle_head(MgHost<T> *m, T H0c, T H0s, cudaGraphConditionalHandle hw,
+void mg_cycle_head(MgHost<float> *m, float H0c, float H0s, cudaGraphConditionalHandle hw,
                    cudaGraphConditionalHandle hi, int in_graph, cudaStream_t s) {
     const std::vector<Level<TC>> &lv = m->lv;
-    launch_resid0<T>(m->L0, lv[1], H0c, H0s, m->ctl, hw, hi, in_graph, s);
+    launch_resid0(m->L0, lv[1], H0c, H0s, m->ctl, hw, hi, in_graph, s);
 }
 
-template <typename T>
-void mg_cycle_rest(MgHost<T> *m, T H0c, T H0s, cudaStream_t s) {
+void mg_cycle_rest(MgHost<float> *m, float H0c, float H0s, cudaStream_t s) {
     dim3 b(32, 8), bs(SX, SY);
     const std::vector<Level<TC>> &lv = m->lv;
     for (int l = 1; l < m->lc; l++) {
@@ -1274,35 +1275,27 @@ void mg_cycle_rest(MgHost<T> *m, T H0c, T H0s, cudaStream_t s) {
     coarse_cta<TC><<<1, CTA_THREADS, m->cta_smem, s>>>(m->d_lv, m->lc, m->nl, m->ctl);
     for (int l = m->lc - 1; l >= 1; l--)
         fv_smooth<TC, 1><<<g2(lv[l].nx, lv[l].ny, bs), bs, 0, s>>>(lv[l], lv[l + 1], NU_POST, m->ctl);
-    launch_smooth0<T>(m->L0, lv[1], 1, NU_FINE, H0c, H0s, m->ctl, 0, s);
+    launch_smooth0(m->L0, lv[1], 1, NU_FINE, H0c, H0s, m->ctl, 0, s);
 }
 
-template <typename T>
-void mg_cycle_smooth(MgHost<T> *m, T H0c, T H0s, cudaStream_t s) {
+void mg_cycle_smooth(MgHost<float> *m, float H0c, float H0s, cudaStream_t s) {
     const std::vector<Level<TC>> &lv = m->lv;
-    launch_smooth0<T>(m->L0, lv[1], 0, NU_SMOOTH_ONLY, H0c, H0s, m->ctl, 0, s);
+    launch_smooth0(m->L0, lv[1], 0, NU_SMOOTH_ONLY, H0c, H0s, m->ctl, 0, s);
 }
 
-template <typename T>
-void mg_presmooth(MgHost<T> *m, T H0c, T H0s, cudaStream_t s) {
+void mg_presmooth(MgHost<float> *m, float H0c, float H0s, cudaStream_t s) {
     const std::vector<Level<TC>> &lv = m->lv;
-    if (keeps_coef<T>() && !m->coef_shared) {  // the solve's node coefficients, before its first sweep
-        dim3 b(32, 8);
-        coef0_kernel<T><<<g2(m->L0.nx, m->L0.ny, b), b, 0, s>>>(m->L0, H0c, H0s);
-    }
-    launch_smooth0<T>(m->L0, lv[1], 0, NU_SMOOTH_ONLY, H0c, H0s, m->ctl, 1, s);
+    launch_smooth0(m->L0, lv[1], 0, NU_SMOOTH_ONLY, H0c, H0s, m->ctl, 1, s);
 }
 
-template <typename T>
-void mg_cycle_twogrid(MgHost<T> *m, T H0c, T H0s, cudaStream_t s) {
+void mg_cycle_twogrid(MgHost<float> *m, float H0c, float H0s, cudaStream_t s) {
     dim3 bs(SX, SY);
     const std::vector<Level<TC>> &lv = m->lv;
     fv_smooth<TC, 2><<<g2(lv[1].nx, lv[1].ny, bs), bs, 0, s>>>(lv[1], lv[1], NU_TWOGRID, m->ctl);
-    launch_smooth0<T>(m->L0, lv[1], 1, NU_FINE, H0c, H0s, m->ctl, 0, s);
+    launch_smooth0(m->L0, lv[1], 1, NU_FINE, H0c, H0s, m->ctl, 0, s);
 }
 
-template <typename T>
-int mg_kernels_per_cycle(const MgHost<T> *m) { return 2 + 3 * (m->lc - 1); }  // after the head
+int mg_kernels_per_cycle(const MgHost<float> *m) { return 2 + 3 * (m->lc - 1); }  // after the head
 
 template <typename T>
 int mg_levels(const MgHost<T> *m) { return m->nl; }
@@ -1342,7 +1335,6 @@ struct MgBatchCtl {
 constexpr int BS_FIRST = 0;  // the sweeps that open every solve
 constexpr int BS_CYCLE = 1;  // the lattice part that ends every cycle
 
-template <bool COMP>
 __global__ void __launch_bounds__(QT) smooth0_batch(const MgBatchInst *tab, const MgBatchTile *tiles,
                                                     int kind) {
     const MgBatchTile t = tiles[blockIdx.x];
@@ -1356,13 +1348,12 @@ __global__ void __launch_bounds__(QT) smooth0_batch(const MgBatchInst *tab, cons
     }
     const int q0 = t.by * I.gx0 + t.bx;
     for (int q = q0; q < q0 + t.cnt; q++) {
-        smooth0_tile<float, COMP>(I.L0, I.lv[1], add, sweeps, I.H0c, I.H0s, I.ctl, kind == BS_FIRST,
+        smooth0_tile<float>(I.L0, I.lv[1], add, sweeps, I.H0c, I.H0s, I.ctl, kind == BS_FIRST,
                                   q % I.gx0, q / I.gx0, I.n0);
         __syncthreads();  // the tile's shared arrays are reused by the next one
     }
 }
 
-template <bool COMP>
 __global__ void __launch_bounds__(256) resid0_batch(const MgBatchInst *tab, const MgBatchTile *tiles,
                                                     MgBatchCtl *bc, int ninst,
                                                     cudaGraphConditionalHandle hw,
@@ -1373,7 +1364,7 @@ __global__ void __launch_bounds__(256) resid0_batch(const MgBatchInst *tab, cons
     if (!I.ctl->done) {  // uniform across the block
         const int q0 = t.by * I.gx1 + t.bx;
         for (int q = q0; q < q0 + t.cnt; q++) {
-            resid0_tile<float, COMP>(I.L0, I.lv[1], I.H0c, I.H0s, I.ctl, 0, 0, 0, q % I.gx1, q / I.gx1,
+            resid0_tile<float>(I.L0, I.lv[1], I.H0c, I.H0s, I.ctl, 0, 0, 0, q % I.gx1, q / I.gx1,
                                      I.n1, false);
             __syncthreads();  // the tile's shared arrays are reused by the next one
         }
@@ -1434,7 +1425,6 @@ __global__ void __launch_bounds__(CTA_THREADS) coarse_batch(const MgBatchInst *t
 
 struct MgBatch {
     int ninst = 0, maxlc = 1;
-    int comp = 0;  // the instances' level-0 form (one for the whole batch)
     MgBatchInst *d_tab = nullptr;
     MgBatchCtl *d_ctl = nullptr;
     int *d_inst = nullptr;                     // every instance (coarse blocks)
@@ -1455,13 +1445,6 @@ MgBatch *mg_batch_create(const std::vector<MgHost<float> *> &ms, const std::vect
     b->release = release;
     b->user = user;
     b->ninst = (int)ms.size();
-    b->comp = ms.empty() ? 0 : ms[0]->L0.comp;
-    for (const MgHost<float> *m : ms)
-        if (m->L0.comp != b->comp) {
-            snprintf(err, errlen, "multigrid batch: instances of both level-0 forms");
-            delete b;
-            return nullptr;
-        }
     Uploader up{alloc, user, &b->mem};
     std::vector<MgBatchInst> tab;
     std::vector<MgBatchTile> t0, t1, tl1;
@@ -1546,8 +1529,7 @@ void mg_batch_destroy(MgBatch *b) {
 }
 
 void mg_batch_presmooth(MgBatch *b, cudaStream_t s) {
-    if (b->comp) smooth0_batch<true><<<b->n_t0, QT, 0, s>>>(b->d_tab, b->d_t0, BS_FIRST);
-    else smooth0_batch<false><<<b->n_t0, QT, 0, s>>>(b->d_tab, b->d_t0, BS_FIRST);
+    smooth0_batch<<<b->n_t0, QT, 0, s>>>(b->d_tab, b->d_t0, BS_FIRST);
 }
 
 // One pass of the loop body, in three parts: every instance's cycle head
@@ -1559,12 +1541,7 @@ void mg_batch_presmooth(MgBatch *b, cudaStream_t s) {
 // their launches.
 void mg_batch_head(MgBatch *b, cudaGraphConditionalHandle hw, cudaGraphConditionalHandle hv,
                    cudaGraphConditionalHandle ht, int in_graph, cudaStream_t s) {
-    if (b->comp)
-        resid0_batch<true><<<b->n_t1, dim3(32, 8), 0, s>>>(b->d_tab, b->d_t1, b->d_ctl, b->ninst, hw,
-                                                           hv, ht, in_graph);
-    else
-        resid0_batch<false><<<b->n_t1, dim3(32, 8), 0, s>>>(b->d_tab, b->d_t1, b->d_ctl, b->ninst, hw,
-                                                            hv, ht, in_graph);
+    resid0_batch<<<b->n_t1, dim3(32, 8), 0, s>>>(b->d_tab, b->d_t1, b->d_ctl, b->ninst, hw, hv, ht, in_graph);
 }
 
 void mg_batch_vcycle(MgBatch *b, cudaStream_t s) {
@@ -1582,8 +1559,7 @@ void mg_batch_twogrid(MgBatch *b, cudaStream_t s) {
 }
 
 void mg_batch_close(MgBatch *b, cudaStream_t s) {
-    if (b->comp) smooth0_batch<true><<<b->n_t0, QT, 0, s>>>(b->d_tab, b->d_t0, BS_CYCLE);
-    else smooth0_batch<false><<<b->n_t0, QT, 0, s>>>(b->d_tab, b->d_t0, BS_CYCLE);
+    smooth0_batch<<<b->n_t0, QT, 0, s>>>(b->d_tab, b->d_t0, BS_CYCLE);
 }
 
 void mg_batch_body(MgBatch *b, cudaStream_t s) {
@@ -1612,19 +1588,9 @@ void mg_set_rhs(MgHost<T> *m, const T *rhs) { m->L0.rhs = rhs; }
 // residual check ends a solve whose right-hand side is zero).
 __global__ void mg_reset_kernel(MgCtl *c, const unsigned long long *scale_bits, double tol,
                                 int max_iter) {
-    c->norm_bits = 0ull;
-    c->iter = 0;
-    c->done = 0;
-    c->converged = 0;
     // a zero right-hand side: the solution is zero and the guess is kept
     const double scale = __longlong_as_double((long long)*scale_bits);
-    c->tolH0 = scale > 0.0 ? tol * scale : INFINITY;
-    c->max_iter = max_iter;
-    c->keep_going = 1;
-    c->blocks_done = 0u;
-    c->mode = 1;
-    c->smooth_left = 0;
-    c->twogrid_left = 2;
+    mg_reset_ctl(c, scale > 0.0 ? tol * scale : INFINITY, max_iter);
 }
 
 void mg_reset_scaled(MgCtl *ctl, const unsigned long long *scale_bits, double tol, int max_iter,
@@ -1704,16 +1670,11 @@ void mg_psi_io(MgHost<double> *m, int op, double *plane, double *prev, cudaStrea
                                      void *(*)(size_t, void *), void (*)(void *, void *), void *, \
                                      char *, size_t, int, const MgHost<T> *);                   \
     template void mg_destroy<T>(MgHost<T> *);                                                   \
-    template void mg_cycle_head<T>(MgHost<T> *, T, T, cudaGraphConditionalHandle,                \
-                                   cudaGraphConditionalHandle, int, cudaStream_t);              \
-    template void mg_cycle_rest<T>(MgHost<T> *, T, T, cudaStream_t);                             \
-    template void mg_cycle_smooth<T>(MgHost<T> *, T, T, cudaStream_t);                           \
-    template void mg_cycle_twogrid<T>(MgHost<T> *, T, T, cudaStream_t);                          \
-    template void mg_presmooth<T>(MgHost<T> *, T, T, cudaStream_t);                              \
-    template int mg_kernels_per_cycle<T>(const MgHost<T> *);                                    \
-    template void mg_cycle_dispatch<T>(MgHost<T> *, cudaGraphConditionalHandle, cudaStream_t);    \
     template int mg_levels<T>(const MgHost<T> *);                                               \
-    template void mg_set_rhs<T>(MgHost<T> *, const T *);
+    template void mg_set_rhs<T>(MgHost<T> *, const T *);                                        \
+    template bool mg_one_kernel<T>(const MgHost<T> *);                                          \
+    template cudaError_t mg_solve<T>(MgHost<T> *, T, T, cudaStream_t);                          \
+    template void mg_set_share<T>(MgHost<T> *, int);
 FCD_MG_INST(float)
 FCD_MG_INST(double)
 

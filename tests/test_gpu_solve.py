@@ -1,0 +1,70 @@
+"""The one-kernel potential solve at the edges of its tiling (needs a GB300):
+32 x 8 lattice tiles, rows merged in pairs with three in the last cell of an odd
+count, lattices of two and three rows (rows not merged), coarse levels inside one
+block and (402 x 123, 800 x 100) across the grid."""
+import numpy as np
+import pytest
+
+from paper_2410_11129_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [(4, 2), (6, 3), (34, 4), (32, 8), (34, 9), (66, 17), (100, 31), (402, 123), (800, 100)]
+
+
+def _cfg(nx, ny, **kw):
+    r2 = 0.3 * min(nx, ny) + 0.5
+    return W.small(nx=nx, ny=ny, r1=0.5 * r2, r2=r2, xc=0.93 * nx, yc=0.45 * ny, xi=3.0, Bo_m=2.0,
+                   alpha_deg=35.0, mag_max_iter=300, **kw)
+
+
+def _residual(orc, cfg, ch):
+    """max |L(psi0 + psi')| / H0 by the FP64 oracle, for the context's populations."""
+    _, g, psi = ch.populations()
+    k = orc.phase(cfg, g)[1]
+    H0 = ch.derived()["H0"]
+    return np.abs(orc.mag_apply(k, psi, 0.0, 0.0) - orc.mag_rhs(k, H0, cfg["alpha"])).max() / H0
+
+
+@pytest.mark.parametrize("nx,ny", SIZES)
+def test_fp64_solve_residual(orc, nx, ny):
+    """The residual that ends the solve is the oracle's: below the tolerance, up
+    to the rounding of nine terms of a potential of up to r2 H0 (1e-13 H0)."""
+    from paper_2410_11129_gb300 import fcd
+    cfg = _cfg(nx, ny, mag_tol=1e-11)
+    ch = fcd.Channel(dict(cfg, precision="fp64"))
+    ch.step(2)
+    it, res, st = ch.solve_magnetic(1e-11, 300)
+    assert st == fcd.FCD_OK and res <= 1e-11
+    assert _residual(orc, cfg, ch) <= 1e-11 + 2e-13
+    ch.close()
+
+
+@pytest.mark.parametrize("nx,ny", SIZES)
+def test_pair_solve_residual(orc, nx, ny):
+    """The hi + lo pair to 1e-6: the FP32 permeability (6e-8 of k, eight links,
+    gradients of up to a few H0) moves the oracle's residual by less than 1e-6."""
+    from paper_2410_11129_gb300 import fcd
+    cfg = _cfg(nx, ny, mag_tol=1e-6)
+    ch = fcd.Channel(dict(cfg, precision="fp32"))
+    ch.step(2)
+    it, res, st = ch.solve_magnetic(1e-6, 300)
+    assert st == fcd.FCD_OK and res <= 1e-6
+    assert _residual(orc, cfg, ch) <= 2e-6
+    ch.close()
+
+
+def test_share_of_the_gpu_does_not_change_bits(orc):
+    """An instance of a batch solves on fewer blocks than a lone context."""
+    from paper_2410_11129_gb300 import fcd
+    cfgs = [dict(_cfg(130, 33, mag_tol=1e-10), precision="fp64"), dict(_cfg(98, 41, mag_tol=1e-6), precision="fp32")]
+    b = fcd.Batch(cfgs * 4)
+    b.set_mode(0)
+    b.step(3)
+    for cfg, inst in zip(cfgs, b.instances):
+        ch = fcd.Channel(cfg)
+        ch.step(3)
+        for x, y in zip(ch.populations(), inst.populations()):
+            assert np.array_equal(x, y)
+        ch.close()
+    b.close()
