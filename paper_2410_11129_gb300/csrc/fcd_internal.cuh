@@ -163,6 +163,8 @@ struct MgCtl {
     long long twogrid_cycles;      // cumulative two-grid cycles (launch accounting)
     unsigned batch_visits;         // batched solves: blocks of the current residual launch seen
     long long dispatches;          // cumulative cycle dispatch launches of graph loops (accounting)
+    int solve_heads;               // cycle heads of this solve so far
+    int first_done;                // its first head ended it (written by that head only)
     // solves that run as one cooperative kernel (fcd_mg_solve.cuh); reset with the solve
     unsigned long long norm_slot[4];  // max |r| of the last heads (bits of doubles >= 0)
     unsigned bar;                     // arrivals at the kernel's grid barriers
@@ -181,6 +183,7 @@ __device__ __forceinline__ void mg_reset_ctl(MgCtl *c, double tolH0, int max_ite
     c->mode = 1;         // the opening sweeps count as a lattice-sweep cycle
     c->smooth_left = 0;  // ... and use up the sweep allowance
     c->twogrid_left = 2;
+    c->solve_heads = 0;
     for (int q = 0; q < 4; q++) c->norm_slot[q] = 0ull;
     c->bar = 0u;
 }
@@ -256,6 +259,7 @@ struct LbmArgs {
     // the step index; ~0ull while none; nullptr: no check)
     unsigned long long *unst = nullptr;
     int open_x = 0;              // open channel: no wrap in x (see launch_open_bc)
+    const int *gate = nullptr;   // nothing is done where it points to 0 (nullptr: no gate)
 };
 
 template <typename T>
@@ -295,7 +299,8 @@ void launch_open_bc_tangent(const Phys<double> &P, const void *f_src, const void
 // (f_dst, g_dst); one thread per row.
 template <typename T>
 void launch_open_bc(int mode, const Phys<T> &P, const void *f_src, const void *g_src,
-                    void *f_dst, void *g_dst, double u_max, double u_avg, cudaStream_t s);
+                    void *f_dst, void *g_dst, double u_max, double u_avg, cudaStream_t s,
+                    const int *gate = nullptr);
 template <typename T>
 void launch_init(int mode, const Phys<T> &P, double u_max, double r1, double r2, double xc,
                  double yc, double xi, void *f, void *g, T *macro, cudaStream_t s);

@@ -287,6 +287,7 @@ __device__ __forceinline__ void collide_tile(const LbmArgs<T, typename Compute<T
         }
     }
     const T *psi = A.ctl->cur ? A.psi1 : A.psi0;
+    if (A.gate && *A.gate == 0) return;
 
     for (int i = threadIdx.y * TX + threadIdx.x; i < (TX + 2) * (TYM + 2); i += TX * TYM) {
         int lx = i % (TX + 2), ly = i / (TX + 2);
@@ -578,13 +579,13 @@ __global__ void __launch_bounds__(TX *TYM, MINB) collide_batch_kernel(const Batc
 // p* = 0, and on g as it is.
 template <typename T, int MODE>
 __global__ void open_bc_kernel(Phys<T> P, const void *fsv, const void *gsv, void *fdv, void *gdv,
-                               T u_max, T u_avg) {
+                               T u_max, T u_avg, const int *gate) {
     using S = typename StoreT<MODE>::type;
     using R = typename Compute<T, MODE>::type;  // dual numbers in the tangent step
     using B = T;
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     const int nx = P.nx, ny = P.ny;
-    if (y >= ny) return;
+    if (y >= ny || (gate && *gate == 0)) return;
     const int ps = (int)P.ps, n = y * P.pitch, o = n + nx - 1, b = o - 1;
     const S *fs = static_cast<const S *>(fsv);
     const S *gs = static_cast<const S *>(gsv);
@@ -835,15 +836,15 @@ void launch_collide_tangent(const LbmArgs<double, DualT> &a, cudaStream_t s) {
 void launch_open_bc_tangent(const Phys<double> &P, const void *f_src, const void *g_src,
                             void *f_dst, void *g_dst, double u_max, double u_avg, cudaStream_t s) {
     const int b = 64, gr = (P.ny + b - 1) / b;
-    open_bc_kernel<double, MODE_TANGENT><<<gr, b, 0, s>>>(P, f_src, g_src, f_dst, g_dst, u_max, u_avg);
+    open_bc_kernel<double, MODE_TANGENT><<<gr, b, 0, s>>>(P, f_src, g_src, f_dst, g_dst, u_max, u_avg, nullptr);
 }
 
 template <typename T>
 void launch_open_bc(int mode, const Phys<T> &P, const void *f_src, const void *g_src,
-                    void *f_dst, void *g_dst, double u_max, double u_avg, cudaStream_t s) {
+                    void *f_dst, void *g_dst, double u_max, double u_avg, cudaStream_t s, const int *gate) {
     const int b = 64, gr = (P.ny + b - 1) / b;
     FCD_MODE_SWITCH(mode, T, (open_bc_kernel<T, M><<<gr, b, 0, s>>>(P, f_src, g_src, f_dst, g_dst,
-                                                                   T(u_max), T(u_avg))));
+                                                                   T(u_max), T(u_avg), gate)));
 }
 
 template <typename T>
@@ -909,7 +910,7 @@ void launch_phi3_to_f64(const T *p1, const T *p2, int nx, int ny, int pitch, dou
                                           int, cudaStream_t);                                  \
     template void launch_collide<T>(int, int, const LbmArgs<T> &, cudaStream_t);               \
     template void launch_open_bc<T>(int, const Phys<T> &, const void *, const void *, void *,    \
-                                    void *, double, double, cudaStream_t);                      \
+                                    void *, double, double, cudaStream_t, const int *);         \
     template void launch_init<T>(int, const Phys<T> &, double, double, double, double, double, \
                                  double, void *, void *, T *, cudaStream_t);                   \
     template void launch_export<T>(int, const Phys<T> &, const void *, const void *, double *, \

@@ -898,6 +898,7 @@ __device__ void cycle_decide(MgCtl *ctl, cudaGraphConditionalHandle hw,
         }
     }
     ctl->keep_going = !ctl->done;
+    if (ctl->solve_heads++ == 0) ctl->first_done = ctl->done;
     if (ctl->done) {
         ctl->mode = 3;
     } else if (ctl->smooth_left > 0 && norm_of(ctl) <= SMOOTH_RATIO * ctl->tolH0) {
