@@ -304,9 +304,12 @@ void launch_open_bc(int mode, const Phys<T> &P, const void *f_src, const void *g
 template <typename T>
 void launch_init(int mode, const Phys<T> &P, double u_max, double r1, double r2, double xc,
                  double yc, double xi, void *f, void *g, T *macro, cudaStream_t s);
+// Populations (fo 9 planes, go 18; nullptr: skipped) in the FP64 exchange
+// layout; unst: the instability record, copied to *unst_out (pinned host memory).
 template <typename T>
 void launch_export(int mode, const Phys<T> &P, const void *f, const void *g, double *fo,
-                   double *go, cudaStream_t s);
+                   double *go, cudaStream_t s, const unsigned long long *unst = nullptr,
+                   unsigned long long *unst_out = nullptr);
 template <typename T>
 void launch_import(int mode, const Phys<T> &P, const double *fi, const double *gi, void *f,
                    void *g, cudaStream_t s);
@@ -317,12 +320,15 @@ void launch_plane_from_f64(const double *src, int nx, int ny, int pitch, T *dst,
 template <typename T>
 void launch_phi3_to_f64(const T *p1, const T *p2, int nx, int ny, int pitch, double *dst,
                         cudaStream_t s);
-// psi' of a level-0 buffer (psi_planes<T>() planes) to and from FP64
+// psi' of the current level-0 buffer (ctl->cur picks A or B; psi_planes<T>()
+// planes) to FP64, and from FP64 into it and into the newest previous potential
+// prev (comp: keep the low part, else the low plane is 0)
 template <typename T>
-void launch_psi_to_f64(const T *src, int nx, int ny, int pitch, double *dst, cudaStream_t s);
+void launch_psi_to_f64(const MgCtl *ctl, const T *A, const T *B, int nx, int ny, int pitch, double *dst,
+                       cudaStream_t s);
 template <typename T>
-void launch_psi_from_f64(const double *src, int nx, int ny, int pitch, T *dst, int comp,
-                         cudaStream_t s);  // comp: keep the low part (else the low plane is 0)
+void launch_psi_from_f64(const double *src, const MgCtl *ctl, T *A, T *B, T *prev, int nx, int ny, int pitch,
+                         int comp, cudaStream_t s);
 
 // multigrid
 template <typename T>

@@ -673,23 +673,32 @@ __global__ void init_kernel(Phys<T> P, double u_max, double r1, double r2, doubl
 }
 
 // ---------------------------------------------------------------- exchange
+template <typename T>
+__device__ __forceinline__ T weight_of(int a) {
+    return a == 0 ? wgt<T>(0) : (a <= 4 ? wgt<T>(1) : wgt<T>(5));
+}
+
+// One plane per blockIdx.z: 27 independent streams of loads and stores.
 template <typename T, int MODE>
-__global__ void export_kernel(Phys<T> P, const void *fv, const void *gv, double *fo,
-                              double *go) {
+__global__ void __launch_bounds__(256) export_kernel(Phys<T> P, const void *fv, const void *gv, double *fo, double *go,
+                                                     const unsigned long long *unst,
+                                                     unsigned long long *unst_out) {
     using S = typename StoreT<MODE>::type;
-    int x = blockIdx.x * blockDim.x + threadIdx.x;
-    int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= P.nx || y >= P.ny) return;
-    long long n = (long long)y * P.pitch + x, m = (long long)y * P.nx + x;
-    long long N = (long long)P.nx * P.ny;
-    const S *f = static_cast<const S *>(fv);
-    const S *g = static_cast<const S *>(gv);
-    for (int a = 0; a < 9; a++) {
-        if (fo) fo[a * N + m] = double(T(f[a * P.ps + n]) - f_off<MODE, T>(a));
-        if (go) {
-            go[a * N + m] = double(T(g[a * P.ps + n]) - g_off<MODE, T>(a));
-            go[(9 + a) * N + m] = double(T(g[(9 + a) * P.ps + n]) - g_off<MODE, T>(a));
-        }
+    const int q = blockIdx.z;
+    if (unst_out && blockIdx.x == 0 && blockIdx.y == 0 && q == 0 && threadIdx.x == 0 && threadIdx.y == 0)
+        *unst_out = *unst;
+    double *out = q < 9 ? fo : go;
+    if (!out) return;
+    out += (long long)(q < 9 ? q : q - 9) * P.nx * P.ny;
+    const S *src = static_cast<const S *>(q < 9 ? fv : gv) + (q < 9 ? q : q - 9) * P.ps;
+    const int a = q < 9 ? q : (q - 9) % 9;
+    const T off = q < 9 ? (MODE == MODE_FP32 ? weight_of<T>(a) : T(0))
+                        : (MODE == MODE_FP32_OFFSET ? -weight_of<T>(a) / T(2) : T(0));
+    const int x = blockIdx.x * 32 + threadIdx.x;
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        const int y = blockIdx.y * 32 + threadIdx.y + 8 * r;
+        if (x < P.nx && y < P.ny) out[(long long)y * P.nx + x] = double(T(src[(long long)y * P.pitch + x]) - off);
     }
 }
 
@@ -732,10 +741,11 @@ __global__ void plane_from_f64(const double *src, int nx, int ny, int pitch, T *
 // psi' of a level-0 buffer in the FP64 exchange layout, and back (FP32: the
 // hi + lo pair of planes; FP64: one plane).
 template <typename T>
-__global__ void psi_to_f64(const T *src, int nx, int ny, int pitch, double *dst) {
+__global__ void psi_to_f64(const MgCtl *ctl, const T *A, const T *B, int nx, int ny, int pitch, double *dst) {
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= nx || y >= ny) return;
+    const T *src = ctl->cur ? B : A;
     const long long n = (long long)y * pitch + x;
     double v = double(src[n]);
     if constexpr (psi_planes<T>() == 2) v += double(src[(long long)pitch * ny + n]);
@@ -743,14 +753,16 @@ __global__ void psi_to_f64(const T *src, int nx, int ny, int pitch, double *dst)
 }
 
 template <typename T>
-__global__ void psi_from_f64(const double *src, int nx, int ny, int pitch, T *dst, int comp) {
+__global__ void psi_from_f64(const double *src, const MgCtl *ctl, T *A, T *B, T *prev, int nx, int ny, int pitch,
+                             int comp) {
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= nx || y >= ny) return;
-    const long long n = (long long)y * pitch + x;
+    T *dst = ctl->cur ? B : A;
+    const long long n = (long long)y * pitch + x, lo = (long long)pitch * ny + n;
     const double v = src[(long long)y * nx + x];
-    dst[n] = T(v);
-    if constexpr (psi_planes<T>() == 2) dst[(long long)pitch * ny + n] = comp ? T(v - double(T(v))) : T(0);
+    dst[n] = prev[n] = T(v);
+    if constexpr (psi_planes<T>() == 2) dst[lo] = prev[lo] = comp ? T(v - double(T(v))) : T(0);
 }
 
 template <typename T>
@@ -856,10 +868,10 @@ void launch_init(int mode, const Phys<T> &P, double u_max, double r1, double r2,
 }
 
 template <typename T>
-void launch_export(int mode, const Phys<T> &P, const void *f, const void *g, double *fo,
-                   double *go, cudaStream_t s) {
-    dim3 b(32, 8), gr = grid2(P.nx, P.ny, b);
-    FCD_MODE_SWITCH(mode, T, (export_kernel<T, M><<<gr, b, 0, s>>>(P, f, g, fo, go)));
+void launch_export(int mode, const Phys<T> &P, const void *f, const void *g, double *fo, double *go,
+                   cudaStream_t s, const unsigned long long *unst, unsigned long long *unst_out) {
+    const dim3 b(32, 8), gr((P.nx + 31) / 32, (P.ny + 31) / 32, 27);
+    FCD_MODE_SWITCH(mode, T, (export_kernel<T, M><<<gr, b, 0, s>>>(P, f, g, fo, go, unst, unst_out)));
 }
 
 template <typename T>
@@ -882,16 +894,17 @@ void launch_plane_from_f64(const double *src, int nx, int ny, int pitch, T *dst,
 }
 
 template <typename T>
-void launch_psi_to_f64(const T *src, int nx, int ny, int pitch, double *dst, cudaStream_t s) {
+void launch_psi_to_f64(const MgCtl *ctl, const T *A, const T *B, int nx, int ny, int pitch, double *dst,
+                       cudaStream_t s) {
     dim3 b(32, 8);
-    psi_to_f64<T><<<grid2(nx, ny, b), b, 0, s>>>(src, nx, ny, pitch, dst);
+    psi_to_f64<T><<<grid2(nx, ny, b), b, 0, s>>>(ctl, A, B, nx, ny, pitch, dst);
 }
 
 template <typename T>
-void launch_psi_from_f64(const double *src, int nx, int ny, int pitch, T *dst, int comp,
-                         cudaStream_t s) {
+void launch_psi_from_f64(const double *src, const MgCtl *ctl, T *A, T *B, T *prev, int nx, int ny, int pitch,
+                         int comp, cudaStream_t s) {
     dim3 b(32, 8);
-    psi_from_f64<T><<<grid2(nx, ny, b), b, 0, s>>>(src, nx, ny, pitch, dst, comp);
+    psi_from_f64<T><<<grid2(nx, ny, b), b, 0, s>>>(src, ctl, A, B, prev, nx, ny, pitch, comp);
 }
 
 template <typename T>
@@ -914,15 +927,18 @@ void launch_phi3_to_f64(const T *p1, const T *p2, int nx, int ny, int pitch, dou
     template void launch_init<T>(int, const Phys<T> &, double, double, double, double, double, \
                                  double, void *, void *, T *, cudaStream_t);                   \
     template void launch_export<T>(int, const Phys<T> &, const void *, const void *, double *, \
-                                   double *, cudaStream_t);                                    \
+                                   double *, cudaStream_t, const unsigned long long *,         \
+                                   unsigned long long *);                                      \
     template void launch_import<T>(int, const Phys<T> &, const double *, const double *,       \
                                    void *, void *, cudaStream_t);                              \
     template void launch_plane_to_f64<T>(const T *, int, int, int, double *, cudaStream_t);    \
     template void launch_plane_from_f64<T>(const double *, int, int, int, T *, cudaStream_t);  \
     template void launch_phi3_to_f64<T>(const T *, const T *, int, int, int, double *,         \
                                         cudaStream_t);                                         \
-    template void launch_psi_to_f64<T>(const T *, int, int, int, double *, cudaStream_t);      \
-    template void launch_psi_from_f64<T>(const double *, int, int, int, T *, int, cudaStream_t);
+    template void launch_psi_to_f64<T>(const MgCtl *, const T *, const T *, int, int, int,     \
+                                       double *, cudaStream_t);                                \
+    template void launch_psi_from_f64<T>(const double *, const MgCtl *, T *, T *, T *, int, int, \
+                                         int, int, cudaStream_t);
 FCD_INST(float)
 FCD_INST(double)
 
