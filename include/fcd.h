@@ -197,7 +197,8 @@ fcd_status fcd_solver_stats(fcd_ctx *ctx, long long *out5);
  * 32 nodes wide). FP32 contexts time 4 and 8 rows at create on their own grid
  * and keep the faster (both do the same arithmetic per node, so the results do
  * not depend on the choice); the environment variable FCD_COLLIDE_TILE_H=4 or 8,
- * set before create, fixes it. FP64 and tangent contexts use 8 and 4.
+ * set before create, fixes it. FP64 contexts use 4, or 2 on small lattices;
+ * tangent contexts 4.
  * FCD_EINVAL for a null argument. */
 fcd_status fcd_collide_tile_height(const fcd_ctx *ctx, int *rows);
 

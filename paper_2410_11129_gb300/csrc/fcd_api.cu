@@ -370,7 +370,19 @@ struct Engine : fcd_ctx {
     // buffers, which the first step overwrites, and record neither breakup nor
     // instability. FCD_COLLIDE_TILE_H=4 or 8 fixes the height instead.
     fcd_status tune_collide() {
-        if (sizeof(T) != 4) return FCD_OK;
+        if (sizeof(T) != 4) {
+            // FP64 arithmetic bounds the kernel (about 57 cycles per operation of a
+            // warp and quarter SM), so the tiles are small enough to spread the
+            // warps evenly: 4 rows, or 2 where 4-row tiles would be two per SM at
+            // most. Measured: 800 x 100 117 (8 rows), 106 (4), 108 us (2);
+            // 1600 x 200 359, 346, 352; 330 x 61 47, 47, 39; 200 x 40 47, 30, 28.
+            int dev = 0, sms = 0;
+            CK(cudaGetDevice(&dev));
+            CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+            const long long tiles = (long long)((prm.nx + TX - 1) / TX) * ((prm.ny + 3) / 4);
+            tile_h = tiles <= 2ll * sms ? 2 : 4;
+            return FCD_OK;
+        }
         const char *env = getenv("FCD_COLLIDE_TILE_H");
         if (env && (atoi(env) == 4 || atoi(env) == 8)) {
             tile_h = atoi(env);

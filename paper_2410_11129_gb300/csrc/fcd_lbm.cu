@@ -810,7 +810,18 @@ void launch_collide(int mode, int tile_h, const LbmArgs<T> &a, cudaStream_t s) {
             return;
         }
     }
-    (void)tile_h;
+    if constexpr (sizeof(T) == 8) {
+        if (tile_h == 2) {
+            dim3 b(TX, 2), gr = grid2(a.P.nx, a.P.ny, b);
+            if (a.open_x) collide_kernel<T, MODE_FP64, true, 2><<<gr, b, 0, s>>>(a);
+            else collide_kernel<T, MODE_FP64, false, 2><<<gr, b, 0, s>>>(a);
+        } else {
+            dim3 b(TX, 4), gr = grid2(a.P.nx, a.P.ny, b);
+            if (a.open_x) collide_kernel<T, MODE_FP64, true, 4><<<gr, b, 0, s>>>(a);
+            else collide_kernel<T, MODE_FP64, false, 4><<<gr, b, 0, s>>>(a);
+        }
+        return;
+    }
     dim3 b(TX, TY), gr = grid2(a.P.nx, a.P.ny, b);
     if (a.open_x) FCD_MODE_SWITCH(mode, T, (collide_kernel<T, M, true><<<gr, b, 0, s>>>(a)));
     else FCD_MODE_SWITCH(mode, T, (collide_kernel<T, M, false><<<gr, b, 0, s>>>(a)));

@@ -68,3 +68,23 @@ def test_share_of_the_gpu_does_not_change_bits(orc):
             assert np.array_equal(x, y)
         ch.close()
     b.close()
+
+
+@pytest.mark.parametrize("nx,ny,rows", [(130, 33, 2), (402, 123, 4)])
+def test_fp64_collide_tile_rows(orc, nx, ny, rows):
+    """Both tile heights of the FP64 collide-stream, ragged in both directions,
+    against the oracle after two steps (solves at 1e-12: 1e-11 in the populations)."""
+    from paper_2410_11129_gb300 import fcd
+    cfg = _cfg(nx, ny, mag_tol=1e-12)
+    ch = fcd.Channel(dict(cfg, precision="fp64"))
+    assert ch.collide_tile_height() == rows
+    ch.step(2)
+    orc.set_threads(orc.max_threads())
+    try:
+        sim = orc.Sim(dict(cfg, mag_max_iter=100000))
+        sim.step(2)
+    finally:
+        orc.set_threads(1)
+    f, g, _ = ch.populations()
+    assert np.abs(f - sim.f).max() <= 1e-11 and np.abs(g - sim.g).max() <= 1e-11
+    ch.close()
