@@ -204,8 +204,9 @@ fcd_status fcd_collide_tile_height(const fcd_ctx *ctx, int *rows);
 
 /* Timing of the stages of a step with CUDA events recorded on the context's
  * stream (inside the step graph): enable, run fcd_step, then read
- * ms4 = [phase recovery + coarse permeabilities, potential solve,
- * collide-stream, whole step] of the most recent step (synchronises). */
+ * ms4 = [phase recovery, potential solve, collide-stream, whole step] of the
+ * most recent step (synchronises). In FP32 contexts with a tolerance of 1e-4 or
+ * more the first also holds the opening sweep of the solve (one kernel). */
 fcd_status fcd_set_profiling(fcd_ctx *ctx, int enable);
 fcd_status fcd_last_step_profile(fcd_ctx *ctx, double *ms4);
 

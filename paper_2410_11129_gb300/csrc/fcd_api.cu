@@ -322,7 +322,7 @@ struct Engine : fcd_ctx {
         CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
         for (auto &e : ev) CK(cudaEventCreate(&e));
         mg = mg_create<T>(prm.nx, prm.ny, pitch, k, psiA, psiB, ctl, alloc, release, user, err,
-                          sizeof err, comp);
+                          sizeof err, comp, nullptr, psiP);
         if (!mg) return FCD_ENOMEM;
         cudaStream_t s = stream;
         CK(cudaMemsetAsync(ctl, 0, sizeof(MgCtl), s));
@@ -412,14 +412,35 @@ struct Engine : fcd_ctx {
     // The previous potential (for the extrapolated initial guess) := current.
     fcd_status keep_history() {
         if (sync_ctl() != FCD_OK) return FCD_ECUDA;
-        CK(cudaMemcpyAsync(psiP, h_ctl->cur ? psiB : psiA, psi_bytes(), cudaMemcpyDeviceToDevice, stream));
+        T *const now = psi_buffer(h_ctl->cur, psiA, psiB, psiP), *prev = psi_buffer(2 - h_ctl->back, psiA, psiB, psiP);
+        CK(cudaMemcpyAsync(prev, now, psi_bytes(), cudaMemcpyDeviceToDevice, stream));
         CK(cudaStreamSynchronize(stream));
         return FCD_OK;
     }
 
+    // Single-plane FP32 with a field: a step opens with one kernel, and the three
+    // psi' buffers take turns as current, previous step's and next; otherwise the
+    // first two alternate and psiP keeps the previous step's.
+    bool turns() const { return sizeof(T) == 4 && magnetic() && !mg_one_kernel<T>(mg); }
+
     // ---- one step as kernel launches on stream s (the MG loop by while node
     // when capturing, by host polling otherwise)
     fcd_status enqueue_pre(int c, cudaStream_t s) {
+        if constexpr (sizeof(T) == 4) {
+            if (turns()) {
+                OpenArgs A;
+                A.P = P;
+                A.g = static_cast<const float *>(static_cast<const void *>(g[c]));
+                A.phi1 = phi1;
+                A.phi2 = phi2;
+                mg_open_level(mg, &A);
+                A.tolH0 = prm.mag_tol * D.H0;
+                A.max_iter = prm.mag_max_iter;
+                A.step = d_step;
+                launch_phase_open(mode, A, s);
+                return FCD_OK;
+            }
+        }
         PhaseCtl pc{ctl, magnetic() ? 1 : 0, prm.mag_tol * D.H0, prm.mag_max_iter, d_step,
                     magnetic() ? 1 : 0, psiA, psiB, psiP, comp};
         launch_phase<T>(mode, P, g[c], phi1, phi2, k, pc, s);
@@ -436,6 +457,7 @@ struct Engine : fcd_ctx {
         a.phi2 = phi2;
         a.psi0 = psiA;
         a.psi1 = psiB;
+        a.psi2 = psiP;
         a.ctl = ctl;
         a.macro = store_macro ? macro : nullptr;
         a.brk = brk;
@@ -452,12 +474,16 @@ struct Engine : fcd_ctx {
             launch_open_bc<T>(mode, P, f[c], g[c], f[c ^ 1], g[c ^ 1], prm.u_max, D.u_avg, s, gate);
     }
     int post_kernels() const { return prm.open_x ? 2 : 1; }
-    // the phase kernel, and a one-kernel solve (the other form counts its cycles)
-    int pre_kernels() const { return 1 + (magnetic() && mg_one_kernel<T>(mg) ? 1 : 0); }
+    // the phase kernel, and a one-kernel solve (the other form counts its cycles,
+    // the one that a step's opening kernel holds among them)
+    int pre_kernels() const {
+        if (turns()) return prm.mag_max_iter > 0 ? 0 : 1;
+        return 1 + (magnetic() ? 1 : 0);
+    }
 
     // One solve with host checks between cycles (hierarchy m with control
-    // block c; default: the context's own).
-    fcd_status host_mg_loop(cudaStream_t s, MgHost<T> *m = nullptr, MgCtl *c = nullptr) {
+    // block c; default: the context's own). opened: its first sweep is done.
+    fcd_status host_mg_loop(cudaStream_t s, MgHost<T> *m = nullptr, MgCtl *c = nullptr, bool opened = false) {
         if (!m) {
             m = mg;
             c = ctl;
@@ -470,7 +496,7 @@ struct Engine : fcd_ctx {
             return FCD_OK;
         }
         if constexpr (sizeof(T) == 4) {
-            mg_presmooth(m, P.H0c, P.H0s, s);
+            if (!opened) mg_presmooth(m, P.H0c, P.H0s, s);
             for (int guard = 0; guard < 1000000; guard++) {
                 mg_cycle_head(m, P.H0c, P.H0s, 0, 0, 0, s);
                 CK(cudaGetLastError());
@@ -520,7 +546,6 @@ struct Engine : fcd_ctx {
     // per step (steps back to back): 1600 x 200 49.4 -> 45.1 us, 2400 x 300 87.6 ->
     // 80.4 us, 900 x 150 open 46.9 -> 42.0 us, the same bits.
     fcd_status capture_solve_and_collide(int c, int sm, cudaStream_t s) {
-        mg_presmooth(mg, P.H0c, P.H0s, s);
         cudaStreamCaptureStatus cs;
         cudaGraph_t gcap;
         const cudaGraphNode_t *deps = nullptr;
@@ -644,7 +669,7 @@ struct Engine : fcd_ctx {
             if (profiling) CK(cudaEventRecord(ev[1], s));
             if (magnetic()) {
                 NvtxScope r("fcd potential solve");
-                fcd_status st = host_mg_loop(s);
+                fcd_status st = host_mg_loop(s, nullptr, nullptr, turns());
                 if (st != FCD_OK) return st;
             }
             if (profiling) CK(cudaEventRecord(ev[2], s));
@@ -692,7 +717,7 @@ struct Engine : fcd_ctx {
         }
         launch_phase<T>(mode, P, g[cur], phi1, phi2, k,
                         PhaseCtl{ctl, 1, tol * D.H0, max_iter, nullptr, 0, nullptr, nullptr, nullptr}, s);
-        host_kernels += pre_kernels();  // the opening sweeps are counted with the sweep cycles
+        host_kernels += turns() ? 1 : pre_kernels();  // the opening sweep counts as a cycle
         CK(cudaGetLastError());
         fcd_status st = host_mg_loop(s);
         if (st != FCD_OK) return st;
@@ -805,7 +830,7 @@ struct Engine : fcd_ctx {
             launch_plane_to_f64<T>(macro + (which - FCD_FIELD_UX) * ps, prm.nx, prm.ny, pitch, st, s);
             host_kernels += 1;
         } else {
-            launch_psi_to_f64<T>(ctl, psiA, psiB, prm.nx, prm.ny, pitch, st, s);
+            launch_psi_to_f64<T>(ctl, psiA, psiB, psiP, prm.nx, prm.ny, pitch, st, s);
             host_kernels += 1;
         }
         cudaError_t e = cudaGetLastError();
@@ -832,7 +857,7 @@ struct Engine : fcd_ctx {
             dp = st + 27 * N;
         }
         launch_export<T>(mode, P, f[cur], g[cur], df, dg, s, unst, h_unst);
-        if (dp) launch_psi_to_f64<T>(ctl, psiA, psiB, prm.nx, prm.ny, pitch, dp, s);
+        if (dp) launch_psi_to_f64<T>(ctl, psiA, psiB, psiP, prm.nx, prm.ny, pitch, dp, s);
         host_kernels += dp ? 2 : 1;
         cudaError_t e = cudaGetLastError();
         if (!direct) {
@@ -888,7 +913,9 @@ struct Engine : fcd_ctx {
     // both level-0 potential buffers and the previous potential. Both potential
     // buffers travel, with the device's current-buffer index, so neither call
     // needs to read the control block on the host: each is one stream of
-    // asynchronous copies and a single synchronisation.
+    // asynchronous copies and a single synchronisation. Where the three buffers
+    // take turns they are stored by role (current, idle, previous step's), for
+    // which get_state reads the control block with its first synchronisation.
     size_t state_bytes() const override {
         return sizeof(SnapHeader) + 27 * (size_t)ps * sizeof(S) + 3 * psi_bytes();
     }
@@ -896,7 +923,16 @@ struct Engine : fcd_ctx {
     fcd_status get_state(void *dst, size_t bytes) override {
         if (!dst || bytes < state_bytes()) return fail(FCD_EINVAL, "snapshot buffer too small");
         cudaStream_t s = stream;
-        CK(cudaStreamSynchronize(s));  // the staging header may still be in flight
+        T *bufs[3] = {psiA, psiB, psiP};
+        if (turns()) {
+            if (sync_ctl() != FCD_OK) return FCD_ECUDA;
+            const int now = h_ctl->cur, prev = 2 - h_ctl->back;
+            bufs[0] = psi_buffer(now, psiA, psiB, psiP);
+            bufs[1] = psi_buffer(3 - now - prev, psiA, psiB, psiP);
+            bufs[2] = psi_buffer(prev, psiA, psiB, psiP);
+        } else {
+            CK(cudaStreamSynchronize(s));  // the staging header may still be in flight
+        }
         SnapHeader &h = *h_snap;
         std::memset(&h, 0, sizeof h);
         h.magic = SNAP_MAGIC;
@@ -910,13 +946,14 @@ struct Engine : fcd_ctx {
         CK(cudaMemcpyAsync(d, &h, sizeof h, cudaMemcpyDefault, s));
         CK(cudaMemcpyAsync(d + offsetof(SnapHeader, brk), brk, sizeof(unsigned long long),
                            cudaMemcpyDefault, s));
-        CK(cudaMemcpyAsync(d + offsetof(SnapHeader, cur), &ctl->cur, sizeof(int), cudaMemcpyDefault, s));
+        if (!turns())
+            CK(cudaMemcpyAsync(d + offsetof(SnapHeader, cur), &ctl->cur, sizeof(int), cudaMemcpyDefault, s));
         size_t off = sizeof h;
         CK(cudaMemcpyAsync(d + off, f[cur], 9 * ps * sizeof(S), cudaMemcpyDefault, s));
         off += 9 * ps * sizeof(S);
         CK(cudaMemcpyAsync(d + off, g[cur], 18 * ps * sizeof(S), cudaMemcpyDefault, s));
         off += 18 * ps * sizeof(S);
-        for (T *q : {psiA, psiB, psiP}) {
+        for (T *q : bufs) {
             CK(cudaMemcpyAsync(d + off, q, psi_bytes(), cudaMemcpyDefault, s));
             off += psi_bytes();
         }
@@ -953,6 +990,7 @@ struct Engine : fcd_ctx {
             off += psi_bytes();
         }
         CK(cudaMemcpyAsync(&ctl->cur, &h.cur, sizeof(int), cudaMemcpyHostToDevice, s));
+        CK(cudaMemsetAsync(&ctl->back, 0, sizeof(int), s));
         CK(cudaMemcpyAsync(brk, &h.brk, sizeof(unsigned long long), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(d_step, &h.step, sizeof(long long), cudaMemcpyHostToDevice, s));
         CK(cudaMemsetAsync(unst, 0xff, sizeof(unsigned long long), s));
@@ -1230,6 +1268,7 @@ struct TangentEngine : Engine<double> {
         a.phi2 = phi2;
         a.psi0 = psiT;
         a.psi1 = psiT;
+        a.psi2 = psiT;
         a.ctl = ctl;
         a.macro = store_macro ? macro : nullptr;
         a.brk = brk;
@@ -1746,6 +1785,7 @@ bool engine_view(fcd_ctx *c, EngineView *v) {
     v->psiA = e->psiA;
     v->psiB = e->psiB;
     v->psiP = e->psiP;
+    v->turns = e->turns() ? 1 : 0;
     v->macro = e->macro;
     v->ctl = e->ctl;
     v->mg = e->mg;

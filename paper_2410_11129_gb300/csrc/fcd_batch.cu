@@ -5,10 +5,12 @@
 // Periodic FP32 instances of one storage form and one level-0 form of the
 // potential make a group that one fixed set of batched kernels advances, one
 // CUDA graph per step:
-//   - the phase recovery of every instance in one launch over a work list of
-//     32 x 8 tiles spanning all instances;
+//   - the phase recovery and the opening sweep of every instance in one launch
+//     over a work list of 64 x 16 patches spanning all instances (instances of
+//     the pair form or without a field: the phase recovery alone, 32 x 8 tiles);
 //   - the potential solves of every instance in one loop of batched multigrid
-//     kernels (fcd_mg.cu), a single while node for the whole group;
+//     kernels (fcd_mg.cu), a single while node for the whole group (pair form:
+//     one-kernel solves, several side by side);
 //   - the fused collide-stream of every instance in one launch over a second
 //     work list, whose tile height (4, 8 or 16 rows) an autotuner picks at
 //     create by timing the three candidates on the group's own state.
@@ -36,8 +38,11 @@ struct Group {
     std::vector<int> idx;          // instances in the group
     std::vector<EngineView> v;
     int tile_h = 8;
-    int n_ptiles = 0, n_ctiles = 0;
-    BatchTile *d_ptiles = nullptr, *d_ctiles = nullptr;
+    // work lists: openings (single-plane solves), phase recoveries (the other
+    // instances), collide-streams
+    int n_otiles = 0, n_ptiles = 0, n_ctiles = 0;
+    BatchTile *d_otiles = nullptr, *d_ptiles = nullptr, *d_ctiles = nullptr;
+    OpenArgs *d_open[2] = {nullptr, nullptr};  // [parity]
     BatchLbm<float> *d_tab[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // [parity][macro]
     MgBatch *mg = nullptr;         // batched solves (single-plane form)
     // pair form: every instance's solve is one kernel, several side by side
@@ -118,6 +123,7 @@ std::vector<BatchLbm<float>> table(const Group &g, int c, bool macro, bool check
         a.phi2 = v.phi2;
         a.psi0 = v.psiA;
         a.psi1 = v.psiB;
+        a.psi2 = v.psiP;
         a.ctl = v.ctl;
         a.macro = macro ? v.macro : nullptr;
         a.brk = check ? v.brk : nullptr;
@@ -131,6 +137,32 @@ std::vector<BatchLbm<float>> table(const Group &g, int c, bool macro, bool check
         b.k = v.k;
     }
     return tab;
+}
+
+// The same for the openings (entries of the other instances are not used).
+std::vector<OpenArgs> open_table(const Group &g, int c) {
+    std::vector<OpenArgs> tab(g.v.size());
+    for (size_t i = 0; i < g.v.size(); i++) {
+        const EngineView &v = g.v[i];
+        OpenArgs &a = tab[i];
+        std::memset(&a, 0, sizeof a);
+        if (!v.turns) continue;
+        a.P = v.P;
+        a.g = static_cast<const float *>(v.g[c]);
+        a.phi1 = v.phi1;
+        a.phi2 = v.phi2;
+        mg_open_level(v.mg, &a);
+        a.tolH0 = v.tolH0;
+        a.max_iter = v.max_iter;
+        a.step = v.d_step;
+    }
+    return tab;
+}
+
+// The group's phase recoveries and openings.
+void launch_pre(const Group &g, int c, cudaStream_t s) {
+    launch_phase_batch<float>(g.mode, g.d_tab[c][0], g.d_ptiles, g.n_ptiles, s);
+    launch_phase_open_batch(g.mode, g.d_open[c], g.d_otiles, g.n_otiles, s);
 }
 
 // The tile height of the group's collide-stream: the fastest of the
@@ -179,15 +211,22 @@ fcd_status group_build(Group &g, const char **why) {
         *why = "stream/event creation";
         return FCD_ECUDA;
     }
-    std::vector<BatchTile> pt;
-    for (size_t i = 0; i < g.v.size(); i++)
-        for (int y = 0; y < g.v[i].P.ny; y += 8)
-            for (int x = 0; x < g.v[i].P.nx; x += 32) pt.push_back({(int)i, x, y, x == 0 && y == 0});
+    std::vector<BatchTile> pt, ot;
+    for (size_t i = 0; i < g.v.size(); i++) {
+        const int dx = g.v[i].turns ? OPEN_X : 32, dy = g.v[i].turns ? OPEN_Y : 8;
+        for (int y = 0; y < g.v[i].P.ny; y += dy)
+            for (int x = 0; x < g.v[i].P.nx; x += dx)
+                (g.v[i].turns ? ot : pt).push_back({(int)i, x, y, x == 0 && y == 0});
+    }
     g.n_ptiles = (int)pt.size();
     g.d_ptiles = upload(g.mem, pt);
-    for (int c = 0; c < 2; c++)
+    g.n_otiles = (int)ot.size();
+    g.d_otiles = upload(g.mem, ot);
+    for (int c = 0; c < 2; c++) {
         for (int m = 0; m < 2; m++) g.d_tab[c][m] = upload(g.mem, table(g, c, m != 0, true));
-    if (!g.d_ptiles || !g.d_tab[0][0] || !g.d_tab[0][1] || !g.d_tab[1][0] || !g.d_tab[1][1]) {
+        g.d_open[c] = upload(g.mem, open_table(g, c));
+    }
+    if (!g.d_ptiles || !g.d_otiles || !g.d_open[0] || !g.d_open[1] || !g.d_tab[0][0] || !g.d_tab[0][1] || !g.d_tab[1][0] || !g.d_tab[1][1]) {
         *why = "table allocation";
         return FCD_ENOMEM;
     }
@@ -307,13 +346,12 @@ cudaError_t capture_one_kernel_solves(Group &g, cudaStream_t s) {
 // loop condition after each pass of the body.
 cudaError_t group_host_step(Group &g, int c, int sm) {
     cudaStream_t s = g.stream;
-    launch_phase_batch<float>(g.mode, g.d_tab[c][0], g.d_ptiles, g.n_ptiles, s);
+    launch_pre(g, c, s);
     for (size_t i = 0; i < g.one.size(); i++) {
         const cudaError_t e = mg_solve<float>(g.one[i], g.one_c[i], g.one_s[i], s);
         if (e != cudaSuccess) return e;
     }
     if (g.mg) {
-        mg_batch_presmooth(g.mg, s);
         for (int guard = 0; guard < 1000000; guard++) {
             mg_batch_body(g.mg, s);
             const int any = mg_batch_any(g.mg, s);
@@ -343,10 +381,9 @@ cudaError_t group_graph_a(Group &g, int c) {
     cudaStream_t s = g.cap;
     cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    launch_phase_batch<float>(g.mode, g.d_tab[c][0], g.d_ptiles, g.n_ptiles, s);
+    launch_pre(g, c, s);
     if (!g.one.empty()) e = capture_one_kernel_solves(g, s);
     if (g.mg) {
-        mg_batch_presmooth(g.mg, s);
         e = capture_solve_loop(g, s);
     }
     return capture_end(s, e, &g.graphA[c], &g.execA[c]);

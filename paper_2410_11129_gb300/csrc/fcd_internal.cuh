@@ -118,6 +118,7 @@ struct Level {
     int nx, ny, pitch;
     T *e, *b, *k;             // correction (level 0: psi'), right-hand side, 1 + chi
     T *r;                     // scratch (level 0: second psi' buffer)
+    T *p3;                    // level 0: third psi' buffer (psi_buffer), nullptr where two rotate
     const int *cx0, *cy0;     // children of cell I: parent columns cx0[I] .. cx0[I+1]-1
     const T *xc, *yc, *wx, *wy;
     const T *ixe;             // 1 / (distance to the east centre), periodic
@@ -140,7 +141,9 @@ struct Level {
 // Device-side control block of one potential solve.
 struct MgCtl {
     unsigned long long norm_bits;  // max |r| of the current cycle (bits of a double >= 0)
-    int cur;                       // which level-0 buffer holds psi'
+    int cur;                       // which level-0 buffer holds psi' (psi_buffer)
+    int back;                      // 2 - the buffer that holds the previous step's psi': 0 where
+                                   // that is the third and only the first two take turns
     int iter;                      // V-cycles done in this solve
     int done;                      // 1 once converged or capped
     int converged;                 // 1 if the tolerance was met
@@ -170,6 +173,9 @@ struct MgCtl {
     unsigned bar;                     // arrivals at the kernel's grid barriers
     int stuck;                        // a barrier timed out: no solve runs any more
 };
+// Level-0 buffer 0, 1 or 2 of a, b, c.
+template <typename T>
+__host__ __device__ __forceinline__ T *psi_buffer(int i, T *a, T *b, T *c) { return i == 0 ? a : (i == 1 ? b : c); }
 // start of a potential solve (one thread)
 __device__ __forceinline__ void mg_reset_ctl(MgCtl *c, double tolH0, int max_iter) {
     c->norm_bits = 0ull;
@@ -250,7 +256,7 @@ struct LbmArgs {
     const void *f_src, *g_src;
     void *f_dst, *g_dst;
     const T *phi1, *phi2;
-    const T *psi0, *psi1;        // the two level-0 buffers; ctl->cur picks one
+    const T *psi0, *psi1, *psi2;  // the level-0 buffers; ctl->cur picks one
     const MgCtl *ctl;
     T *macro;                    // nullptr: do not store the macroscopic fields
     unsigned long long *brk;     // sticky breakup key (nullptr: no check)
@@ -320,14 +326,14 @@ void launch_plane_from_f64(const double *src, int nx, int ny, int pitch, T *dst,
 template <typename T>
 void launch_phi3_to_f64(const T *p1, const T *p2, int nx, int ny, int pitch, double *dst,
                         cudaStream_t s);
-// psi' of the current level-0 buffer (ctl->cur picks A or B; psi_planes<T>()
-// planes) to FP64, and from FP64 into it and into the newest previous potential
-// prev (comp: keep the low part, else the low plane is 0)
+// psi' of the current level-0 buffer (ctl->cur picks A, B or C;
+// psi_planes<T>() planes) to FP64, and from FP64 into it and into the previous
+// step's (comp: keep the low part, else the low plane is 0)
 template <typename T>
-void launch_psi_to_f64(const MgCtl *ctl, const T *A, const T *B, int nx, int ny, int pitch, double *dst,
+void launch_psi_to_f64(const MgCtl *ctl, const T *A, const T *B, const T *C, int nx, int ny, int pitch, double *dst,
                        cudaStream_t s);
 template <typename T>
-void launch_psi_from_f64(const double *src, const MgCtl *ctl, T *A, T *B, T *prev, int nx, int ny, int pitch,
+void launch_psi_from_f64(const double *src, const MgCtl *ctl, T *A, T *B, T *C, int nx, int ny, int pitch,
                          int comp, cudaStream_t s);
 
 // multigrid
@@ -337,7 +343,8 @@ template <typename T>
 MgHost<T> *mg_create(int nx, int ny, int pitch, T *k0, T *psiA, T *psiB, MgCtl *ctl,
                      void *(*alloc)(size_t, void *), void (*release)(void *, void *), void *user,
                      char *err, size_t errlen, int comp = 0,
-                     const MgHost<T> *share_coef = nullptr);  // FP64: use its coefficient planes
+                     const MgHost<T> *share_coef = nullptr,  // FP64: use its coefficient planes
+                     T *psiC = nullptr);                     // third buffer of psi' (single FP32 plane)
 template <typename T>
 void mg_destroy(MgHost<T> *m);
 // Solves of several kernels (the single FP32 plane). One V-cycle = head (lattice
@@ -348,7 +355,23 @@ void mg_cycle_head(MgHost<float> *m, float H0c, float H0s, cudaGraphConditionalH
 void mg_cycle_rest(MgHost<float> *m, float H0c, float H0s, cudaStream_t s);
 void mg_cycle_smooth(MgHost<float> *m, float H0c, float H0s, cudaStream_t s);
 void mg_cycle_twogrid(MgHost<float> *m, float H0c, float H0s, cudaStream_t s);
-void mg_presmooth(MgHost<float> *m, float H0c, float H0s, cudaStream_t s);  // opens every such solve
+void mg_presmooth(MgHost<float> *m, float H0c, float H0s, cudaStream_t s);  // opens such a solve outside a step
+// The phase recovery, the extrapolated guess and the opening sweep of a step's
+// solve in one kernel (such contexts, whose three psi' buffers take turns)
+struct OpenArgs {
+    Phys<float> P;
+    const float *g;
+    float *phi1, *phi2;
+    Level<float> L0;
+    MgCtl *ctl;
+    double tolH0;
+    int max_iter;
+    long long *step;
+};
+void mg_open_level(const MgHost<float> *m, OpenArgs *A);  // A->L0 and A->ctl
+void launch_phase_open(int mode, const OpenArgs &A, cudaStream_t s);
+constexpr int OPEN_X = 64, OPEN_Y = 16;  // patch of a block
+void launch_phase_open_batch(int mode, const OpenArgs *tab, const BatchTile *tiles, int ntiles, cudaStream_t s);
 int mg_kernels_per_cycle(const MgHost<float> *m);
 // Whole solve as one cooperative kernel (FP64 and the FP32 pair): whether the
 // hierarchy takes it, its launch, and the share of the GPU it may fill (1 /
@@ -377,8 +400,8 @@ void mg_psi_io(MgHost<double> *m, int op, double *plane, double *prev, cudaStrea
 template <typename T>
 int mg_levels(const MgHost<T> *m);
 // Batched solves of many FP32 hierarchies (one per instance; fields and
-// control blocks stay the instances' own): opening sweeps of every solve, and
-// the body of the loop that runs until every solve is done.
+// control blocks stay the instances' own): the body of the loop that runs until
+// every solve is done (launch_phase_open_batch opens them).
 // FP32 hierarchies of the single-plane form only (the pair's solves are one
 // kernel each).
 struct MgBatch;
@@ -386,7 +409,6 @@ MgBatch *mg_batch_create(const std::vector<MgHost<float> *> &ms, const std::vect
                          const std::vector<float> &H0s, void *(*alloc)(size_t, void *),
                          void (*release)(void *, void *), void *user, char *err, size_t errlen);
 void mg_batch_destroy(MgBatch *b);
-void mg_batch_presmooth(MgBatch *b, cudaStream_t s);
 // one pass of the loop body launched from the host (no graph conditions set)
 void mg_batch_body(MgBatch *b, cudaStream_t s);
 // the body in parts, for a graph whose while node (hw) holds them: the head
@@ -469,6 +491,7 @@ struct EngineView {
     Phys<float> P;
     void *f[2], *g[2];
     float *phi1, *phi2, *k, *psiA, *psiB, *psiP, *macro;
+    int turns;  // steps open with launch_phase_open
     MgCtl *ctl;
     MgHost<float> *mg;
     unsigned long long *brk, *unst;

@@ -1,6 +1,7 @@
 // fcd_lbm.cu -- lattice Boltzmann kernels of the coupled step (arXiv 2410.11129).
 //
 // phase_kernel   : Eq. 32 (phi_i = sum_a g^i_a), Eq. 24, Eq. 8 (k = 1 + chi)
+//                  (single-plane FP32 steps: phase_open of fcd_mg.cu)
 // collide_kernel : one fused pass per node: isotropic gradients and Laplacians
 //                  (Eqs. 34-35) from shared-memory tiles with a one-node halo,
 //                  chemical potentials and surface tension (Eqs. 25-28, 36),
@@ -286,7 +287,7 @@ __device__ __forceinline__ void collide_tile(const LbmArgs<T, typename Compute<T
             for (int a = 0; a < 18; a++) gpre[a] = __ldg(gs + (a * (int)ps + (int)n));
         }
     }
-    const T *psi = A.ctl->cur ? A.psi1 : A.psi0;
+    const T *psi = psi_buffer(A.ctl->cur, A.psi0, A.psi1, A.psi2);
     if (A.gate && *A.gate == 0) return;
 
     for (int i = threadIdx.y * TX + threadIdx.x; i < (TX + 2) * (TYM + 2); i += TX * TYM) {
@@ -741,11 +742,11 @@ __global__ void plane_from_f64(const double *src, int nx, int ny, int pitch, T *
 // psi' of a level-0 buffer in the FP64 exchange layout, and back (FP32: the
 // hi + lo pair of planes; FP64: one plane).
 template <typename T>
-__global__ void psi_to_f64(const MgCtl *ctl, const T *A, const T *B, int nx, int ny, int pitch, double *dst) {
+__global__ void psi_to_f64(const MgCtl *ctl, const T *A, const T *B, const T *C, int nx, int ny, int pitch, double *dst) {
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= nx || y >= ny) return;
-    const T *src = ctl->cur ? B : A;
+    const T *src = psi_buffer(ctl->cur, A, B, C);
     const long long n = (long long)y * pitch + x;
     double v = double(src[n]);
     if constexpr (psi_planes<T>() == 2) v += double(src[(long long)pitch * ny + n]);
@@ -753,12 +754,12 @@ __global__ void psi_to_f64(const MgCtl *ctl, const T *A, const T *B, int nx, int
 }
 
 template <typename T>
-__global__ void psi_from_f64(const double *src, const MgCtl *ctl, T *A, T *B, T *prev, int nx, int ny, int pitch,
+__global__ void psi_from_f64(const double *src, const MgCtl *ctl, T *A, T *B, T *C, int nx, int ny, int pitch,
                              int comp) {
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= nx || y >= ny) return;
-    T *dst = ctl->cur ? B : A;
+    T *dst = psi_buffer(ctl->cur, A, B, C), *prev = psi_buffer(2 - ctl->back, A, B, C);
     const long long n = (long long)y * pitch + x, lo = (long long)pitch * ny + n;
     const double v = src[(long long)y * nx + x];
     dst[n] = prev[n] = T(v);
@@ -905,17 +906,17 @@ void launch_plane_from_f64(const double *src, int nx, int ny, int pitch, T *dst,
 }
 
 template <typename T>
-void launch_psi_to_f64(const MgCtl *ctl, const T *A, const T *B, int nx, int ny, int pitch, double *dst,
+void launch_psi_to_f64(const MgCtl *ctl, const T *A, const T *B, const T *C, int nx, int ny, int pitch, double *dst,
                        cudaStream_t s) {
     dim3 b(32, 8);
-    psi_to_f64<T><<<grid2(nx, ny, b), b, 0, s>>>(ctl, A, B, nx, ny, pitch, dst);
+    psi_to_f64<T><<<grid2(nx, ny, b), b, 0, s>>>(ctl, A, B, C, nx, ny, pitch, dst);
 }
 
 template <typename T>
-void launch_psi_from_f64(const double *src, const MgCtl *ctl, T *A, T *B, T *prev, int nx, int ny, int pitch,
+void launch_psi_from_f64(const double *src, const MgCtl *ctl, T *A, T *B, T *C, int nx, int ny, int pitch,
                          int comp, cudaStream_t s) {
     dim3 b(32, 8);
-    psi_from_f64<T><<<grid2(nx, ny, b), b, 0, s>>>(src, ctl, A, B, prev, nx, ny, pitch, comp);
+    psi_from_f64<T><<<grid2(nx, ny, b), b, 0, s>>>(src, ctl, A, B, C, nx, ny, pitch, comp);
 }
 
 template <typename T>
@@ -946,7 +947,7 @@ void launch_phi3_to_f64(const T *p1, const T *p2, int nx, int ny, int pitch, dou
     template void launch_plane_from_f64<T>(const double *, int, int, int, T *, cudaStream_t);  \
     template void launch_phi3_to_f64<T>(const T *, const T *, int, int, int, double *,         \
                                         cudaStream_t);                                         \
-    template void launch_psi_to_f64<T>(const MgCtl *, const T *, const T *, int, int, int,     \
+    template void launch_psi_to_f64<T>(const MgCtl *, const T *, const T *, const T *, int, int, int, \
                                        double *, cudaStream_t);                                \
     template void launch_psi_from_f64<T>(const double *, const MgCtl *, T *, T *, T *, int, int, \
                                          int, int, cudaStream_t);

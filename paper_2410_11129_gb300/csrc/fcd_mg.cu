@@ -343,7 +343,7 @@ __device__ __forceinline__ void resid0_tile(const Level<T> &L0, const Level<TC> 
     const int I1 = min(I0 + 32, L1.nx), J1 = min(J0 + 8, L1.ny);
     const int fx0 = L1.cx0[I0], fx1 = L1.cx0[I1], fy0 = L1.cy0[J0], fy1 = L1.cy0[J1];
     const int wx = fx1 - fx0 + 2, wy = fy1 - fy0 + 2;
-    const T *psi = ctl->cur ? L0.r : L0.e;
+    const T *psi = psi_buffer(ctl->cur, L0.e, L0.r, L0.p3);
     {  // all loads issued before the shared-memory stores: warp w takes footprint
        // rows w, w + 8, w + 16, lane l columns l, l + 32, l + 64
         constexpr int NR = (RY + 7) / 8, NC = (RX + 31) / 32;
@@ -466,8 +466,9 @@ __device__ __forceinline__ void smooth0_tile(const Level<T> &L0, const Level<TC>
     __shared__ T sk[SY + 2][SX + 2];
     const int nx = L0.nx, ny = L0.ny, pitch = L0.pitch;
     const int x0 = bx * SX, y0 = by * SY;
-    const T *src = ctl->cur ? L0.r : L0.e;
-    T *dst = ctl->cur ? L0.e : L0.r;
+    const int cur = ctl->cur, prv = 2 - ctl->back;
+    const T *src = psi_buffer(cur, L0.e, L0.r, L0.p3);
+    T *dst = psi_buffer(3 - cur - prv, L0.e, L0.r, L0.p3);
     __shared__ ProlongTile<T, SX + 2, SY + 2> pt;
     if (add_coarse) prolong_tile_load(pt, L0, x0 - 1, y0 - 1);
     {  // tile with its frozen one-cell ring, all loads issued before the stores: warp w
@@ -929,15 +930,176 @@ __global__ void cycle_dispatch_kernel(MgCtl *ctl, cudaGraphConditionalHandle hs)
 
 
 
-// End of a full cycle (one thread): count it, flip the lattice buffer, clear
-// the norm for the next residual.
+// End of a full cycle (one thread): count it, turn the lattice buffers (the
+// result went to the one that is neither the current nor the previous step's),
+// clear the norm for the next residual.
 __device__ void cycle_close(MgCtl *ctl) {
     ctl->iter++;
     if (ctl->mode == 1) ctl->smooth_cycles++;
     else if (ctl->mode == 2) ctl->twogrid_cycles++;
     else ctl->total_cycles++;
-    ctl->cur ^= 1;
+    ctl->cur = 3 - ctl->cur - (2 - ctl->back);
     ctl->norm_bits = 0ull;
+}
+
+// ------------------------------------------- phase recovery and opening sweep
+// One kernel for what opens a step: phi_i = sum_a g^i_a and k of a 64 x 16 patch
+// and the ring around it, the guess 2 psi'(t) - psi'(t-1) there, and one
+// block-Gauss-Seidel sweep of the patch's four 32 x 8 tiles, each against its own
+// frozen ring (the arithmetic of the phase kernel and of smooth0, node by node).
+// As two kernels, a memory-bound pass (9600 x 1200: 176 us, its bytes at the copy
+// rate) was followed by one bound by its instructions (98 us), with k and psi'
+// written and read in between; the small lattices paid for the second kernel's
+// launch and first loads. The previous potential is not copied: the three buffers
+// turn. The ring's 18 populations are read twice, so the patch is four tiles (the
+// sectors loaded are 1.4 times the patch's; one tile alone 1.9 times). What bounds
+// it is the latency of the loads in flight: two nodes of a thread at a time, three
+// blocks of 256 per SM; one node and four blocks measured the same on 9600 x 1200
+// and 4% slower on 2400 x 300, patches of 64 x 8 290 us against 228, of 32 x 8
+// 590 us, of 128 x 8 and 128 x 16 no better. Measured per step, before and now:
+// 1600 x 200 43.5 -> 41.6 us, 2400 x 300 offset 80.9 -> 78.1, 900 x 150 open
+// 42.1 -> 40.2, 9600 x 1200 871 -> 825 (the two kernels 274 -> 228), 24 batched
+// channels 723 -> 699, the same bits.
+template <int MODE, int CX, int CY>
+__device__ __forceinline__ void phase_open_tile(const OpenArgs &A, int x0, int y0) {
+    constexpr int OX = CX * SX, OY = CY * SY, NT = CX * CY, WARPS = NT * QT / 32;
+    __shared__ float sk[NT][SY + 2][SX + 2], sp[NT][SY + 2][SX + 2];
+    const Phys<float> &P = A.P;
+    const Level<float> &L0 = A.L0;
+    MgCtl *const ctl = A.ctl;
+    const int nx = P.nx, ny = P.ny, pitch = P.pitch, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long ps = P.ps;
+    // the control block changes only after every block is done (below)
+    const int cur = ctl->cur, prv = 2 - ctl->back;
+    const float *now = psi_buffer(cur, L0.e, L0.r, L0.p3), *before = psi_buffer(prv, L0.e, L0.r, L0.p3);
+    float *dst = psi_buffer(3 - cur - prv, L0.e, L0.r, L0.p3);
+    // Nodes (px, py) of the patch and its ring, -1 .. OX by -1 .. OY, a warp at a
+    // time: item i < ROWS_W is 32 columns of one of the OY + 2 rows, the items
+    // after them are the two ring columns. FLIGHT nodes of a thread load at once.
+    static_assert(SX == 32, "a warp takes one tile's row");
+    constexpr int ROWS_W = CX * (OY + 2), ITEMS = ROWS_W + (2 * (OY + 2) + 31) / 32, FLIGHT = 2;
+    for (int i0 = warp; i0 < ITEMS; i0 += FLIGHT * WARPS) {
+        float gv[FLIGHT][18], pn[FLIGHT], pb[FLIGHT];
+        int px[FLIGHT], py[FLIGHT], n[FLIGHT];
+        bool act[FLIGHT];
+#pragma unroll
+        for (int q = 0; q < FLIGHT; q++) {
+            const int i = i0 + q * WARPS, e = (i - ROWS_W) * 32 + lane;
+            act[q] = i < ITEMS && e < 2 * (OY + 2);
+            if (!act[q]) continue;
+            px[q] = i < ROWS_W ? (i % CX) * 32 + lane : (e & 1 ? OX : -1);
+            py[q] = (i < ROWS_W ? i / CX : e >> 1) - 1;
+            int x = x0 + px[q];
+            if (x < 0) x += nx;
+            while (x >= nx) x -= nx;
+            const int y = y0 + py[q];
+            n[q] = (y < 0 ? 0 : (y >= ny ? ny - 1 : y)) * pitch + x;  // mirrored ghost rows
+            const float *g = A.g + n[q];
+#pragma unroll
+            for (int a = 0; a < 18; a++) gv[q][a] = __ldg(g + a * ps);
+            pn[q] = __ldg(now + n[q]);
+            pb[q] = __ldg(before + n[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < FLIGHT; q++) {
+            if (!act[q]) continue;
+            float p1 = 0.f, p2 = 0.f;
+#pragma unroll
+            for (int a = 0; a < 9; a++) {
+                p1 += gv[q][a] - g_off<MODE, float>(a);
+                p2 += gv[q][9 + a] - g_off<MODE, float>(a);
+            }
+            const float h1 = clamp01(p1), h2 = clamp01(p2), h3 = clamp01(1.f - p1 - p2);
+            const float k = 1.f / (P.ik[0] * h1 + P.ik[1] * h2 + P.ik[2] * h3);
+            if (px[q] >= 0 && px[q] < OX && py[q] >= 0 && py[q] < OY && x0 + px[q] < nx && y0 + py[q] < ny) {
+                A.phi1[n[q]] = p1;  // the patch's own node
+                A.phi2[n[q]] = p2;
+                L0.k[n[q]] = k;
+            }
+            const float guess = 2.f * pn[q] - pb[q];
+#pragma unroll
+            for (int w = 0; w < NT; w++) {
+                const int lx = px[q] - SX * (w % CX) + 1, ly = py[q] - SY * (w / CX) + 1;
+                if (lx >= 0 && lx < SX + 2 && ly >= 0 && ly < SY + 2) {
+                    sk[w][ly][lx] = k;
+                    sp[w][ly][lx] = guess;  // in ghost rows never read
+                }
+            }
+        }
+    }
+    __syncthreads();
+    const int w = tid / QT, t = tid % QT, tx0 = x0 + SX * (w % CX), ty0 = y0 + SY * (w / CX);
+    const int qx = 2 * (t % (SX / 2)), qy = 2 * (t / (SX / 2));
+    auto sweep = [&](auto wall) {
+        constexpr bool W = decltype(wall)::value;
+        Node9<float> nd[4];
+        float inv_diag[4];
+        bool own[4];
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            const int lx = qx + (c & 1) + 1, ly = qy + (c >> 1) + 1, y = ty0 + ly - 1;
+            own[c] = tx0 + lx - 1 < nx && y < ny;
+            inv_diag[c] = 0.f;
+            if (own[c]) {
+                auto kat = [&](int dx, int dy) { return sk[w][ly + dy][lx + dx]; };
+                nd[c] = node9<float, W>(kat, y, ny, P.H0c, P.H0s);
+                inv_diag[c] = 1.f / nd[c].diag;
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            const int lx = qx + (c & 1) + 1, ly = qy + (c >> 1) + 1, y = ty0 + ly - 1;
+            auto pat = [&](int dx, int dy) { return sp[w][ly + dy][lx + dx]; };
+            if (own[c]) {
+                float v = sp[w][ly][lx];
+                if (A.max_iter > 0) v = (off9<float, W>(nd[c], pat, y, ny) - nd[c].b) * inv_diag[c];
+                sp[w][ly][lx] = v;
+                dst[(long long)y * pitch + tx0 + lx - 1] = v;
+            }
+            if (c < 3)  // this tile's two warps; every thread of the tile passes
+                asm volatile("barrier.sync %0, %1;" ::"r"(w + 1), "n"(QT) : "memory");
+        }
+    };
+    if (ty0 == 0 || ty0 + SY >= ny) sweep(std::true_type{});
+    else sweep(std::false_type{});
+    __syncthreads();
+    const unsigned gx = (nx + OX - 1) / OX, gy = (ny + OY - 1) / OY;
+    if (tid == 0 && tile_done(ctl, L0.grp, (y0 / OY) * gx + x0 / OX, gx * gy, 0ull)) {
+        // the start of the solve and of the step, and the end of its opening cycle
+        mg_reset_ctl(ctl, A.tolH0, A.max_iter);
+        if (A.max_iter > 0) {
+            ctl->iter = 1;
+            ctl->smooth_cycles++;
+        }
+        ctl->back = 2 - cur;
+        ctl->cur = 3 - cur - prv;
+        ctl->step_cur = *A.step;
+        *A.step += 1;
+    }
+}
+
+constexpr int OPEN_CX = OPEN_X / SX, OPEN_CY = OPEN_Y / SY, OPEN_THREADS = OPEN_CX * OPEN_CY * QT;
+template <int MODE>
+__global__ void __launch_bounds__(OPEN_THREADS, 3) phase_open(const OpenArgs A) {
+    phase_open_tile<MODE, OPEN_CX, OPEN_CY>(A, blockIdx.x * OPEN_X, blockIdx.y * OPEN_Y);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(OPEN_THREADS, 3) phase_open_batch(const OpenArgs *tab, const BatchTile *tiles) {
+    const BatchTile t = tiles[blockIdx.x];
+    phase_open_tile<MODE, OPEN_CX, OPEN_CY>(tab[t.inst], t.x0, t.y0);
+}
+
+void launch_phase_open(int mode, const OpenArgs &A, cudaStream_t s) {
+    const dim3 g((A.P.nx + OPEN_X - 1) / OPEN_X, (A.P.ny + OPEN_Y - 1) / OPEN_Y);
+    if (mode == MODE_FP32) phase_open<MODE_FP32><<<g, OPEN_THREADS, 0, s>>>(A);
+    else phase_open<MODE_FP32_OFFSET><<<g, OPEN_THREADS, 0, s>>>(A);
+}
+
+void launch_phase_open_batch(int mode, const OpenArgs *tab, const BatchTile *tiles, int ntiles, cudaStream_t s) {
+    if (ntiles <= 0) return;
+    if (mode == MODE_FP32) phase_open_batch<MODE_FP32><<<ntiles, OPEN_THREADS, 0, s>>>(tab, tiles);
+    else phase_open_batch<MODE_FP32_OFFSET><<<ntiles, OPEN_THREADS, 0, s>>>(tab, tiles);
 }
 
 }  // namespace fcd
@@ -1084,7 +1246,7 @@ cudaError_t mg_solve(MgHost<T> *m, T H0c, T H0s, cudaStream_t s) {
 template <typename T>
 MgHost<T> *mg_create(int nx, int ny, int pitch, T *k0, T *psiA, T *psiB, MgCtl *ctl,
                      void *(*alloc)(size_t, void *), void (*release)(void *, void *), void *user,
-                     char *err, size_t errlen, int comp, const MgHost<T> *share_coef) {
+                     char *err, size_t errlen, int comp, const MgHost<T> *share_coef, T *psiC) {
     MgHost<T> *m = new MgHost<T>();
     m->alloc = alloc;
     m->release = release;
@@ -1204,6 +1366,7 @@ MgHost<T> *mg_create(int nx, int ny, int pitch, T *k0, T *psiA, T *psiB, MgCtl *
         L.k = k0;
         L.e = psiA;
         L.r = psiB;
+        L.p3 = psiC;
         L.comp = sizeof(T) == 4 && comp ? 1 : 0;
         {
             const std::vector<MgGroup> zero(MG_GROUPS, MgGroup{});
@@ -1289,6 +1452,11 @@ void mg_presmooth(MgHost<float> *m, float H0c, float H0s, cudaStream_t s) {
     launch_smooth0(m->L0, lv[1], 0, NU_SMOOTH_ONLY, H0c, H0s, m->ctl, 1, s);
 }
 
+void mg_open_level(const MgHost<float> *m, OpenArgs *A) {
+    A->L0 = m->L0;
+    A->ctl = m->ctl;
+}
+
 void mg_cycle_twogrid(MgHost<float> *m, float H0c, float H0s, cudaStream_t s) {
     dim3 bs(SX, SY);
     const std::vector<Level<TC>> &lv = m->lv;
@@ -1333,24 +1501,17 @@ struct MgBatchCtl {
     unsigned any_t; // ... some instance runs a two-grid cycle in this pass
 };
 
-constexpr int BS_FIRST = 0;  // the sweeps that open every solve
-constexpr int BS_CYCLE = 1;  // the lattice part that ends every cycle
-
-__global__ void __launch_bounds__(QT) smooth0_batch(const MgBatchInst *tab, const MgBatchTile *tiles,
-                                                    int kind) {
+// the lattice part that ends every cycle
+__global__ void __launch_bounds__(QT) smooth0_batch(const MgBatchInst *tab, const MgBatchTile *tiles) {
     const MgBatchTile t = tiles[blockIdx.x];
     const MgBatchInst &I = tab[t.inst];
-    int add = 0, sweeps = NU_SMOOTH_ONLY;
-    if (kind == BS_CYCLE) {  // V-cycle and two-grid cycle: coarse correction; else sweeps only
-        const int m = I.ctl->mode;
-        if (m == 3) return;  // this solve is over (uniform across the block)
-        add = m == 0 || m == 2;
-        sweeps = add ? NU_FINE : NU_SMOOTH_ONLY;
-    }
+    const int m = I.ctl->mode;
+    if (m == 3) return;  // this solve is over (uniform across the block)
+    const int add = m == 0 || m == 2;  // V-cycle and two-grid cycle: coarse correction; else sweeps only
+    const int sweeps = add ? NU_FINE : NU_SMOOTH_ONLY;
     const int q0 = t.by * I.gx0 + t.bx;
     for (int q = q0; q < q0 + t.cnt; q++) {
-        smooth0_tile<float>(I.L0, I.lv[1], add, sweeps, I.H0c, I.H0s, I.ctl, kind == BS_FIRST,
-                                  q % I.gx0, q / I.gx0, I.n0);
+        smooth0_tile<float>(I.L0, I.lv[1], add, sweeps, I.H0c, I.H0s, I.ctl, 0, q % I.gx0, q / I.gx0, I.n0);
         __syncthreads();  // the tile's shared arrays are reused by the next one
     }
 }
@@ -1529,10 +1690,6 @@ void mg_batch_destroy(MgBatch *b) {
     delete b;
 }
 
-void mg_batch_presmooth(MgBatch *b, cudaStream_t s) {
-    smooth0_batch<<<b->n_t0, QT, 0, s>>>(b->d_tab, b->d_t0, BS_FIRST);
-}
-
 // One pass of the loop body, in three parts: every instance's cycle head
 // (mg_batch_head); the coarse-level kernels of the V-cycle (mg_batch_vcycle)
 // and of the two-grid cycle (mg_batch_twogrid), each acting only for the
@@ -1560,7 +1717,7 @@ void mg_batch_twogrid(MgBatch *b, cudaStream_t s) {
 }
 
 void mg_batch_close(MgBatch *b, cudaStream_t s) {
-    smooth0_batch<<<b->n_t0, QT, 0, s>>>(b->d_tab, b->d_t0, BS_CYCLE);
+    smooth0_batch<<<b->n_t0, QT, 0, s>>>(b->d_tab, b->d_t0);
 }
 
 void mg_batch_body(MgBatch *b, cudaStream_t s) {
@@ -1669,7 +1826,7 @@ void mg_psi_io(MgHost<double> *m, int op, double *plane, double *prev, cudaStrea
 #define FCD_MG_INST(T)                                                                          \
     template MgHost<T> *mg_create<T>(int, int, int, T *, T *, T *, MgCtl *,                     \
                                      void *(*)(size_t, void *), void (*)(void *, void *), void *, \
-                                     char *, size_t, int, const MgHost<T> *);                   \
+                                     char *, size_t, int, const MgHost<T> *, T *);              \
     template void mg_destroy<T>(MgHost<T> *);                                                   \
     template int mg_levels<T>(const MgHost<T> *);                                               \
     template void mg_set_rhs<T>(MgHost<T> *, const T *);                                        \

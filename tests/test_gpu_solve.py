@@ -1,6 +1,6 @@
 """The one-kernel potential solve at the edges of its tiling (needs a GB300):
 32 x 8 lattice tiles, rows merged in pairs with three in the last cell of an odd
-count, lattices of two and three rows (rows not merged), coarse levels inside one
+32 x 8 lattice tiles, rows merged in pairs with three in the last cell of an odd
 block and (402 x 123, 800 x 100) across the grid."""
 import numpy as np
 import pytest
@@ -88,3 +88,57 @@ def test_fp64_collide_tile_rows(orc, nx, ny, rows):
     f, g, _ = ch.populations()
     assert np.abs(f - sim.f).max() <= 1e-11 and np.abs(g - sim.g).max() <= 1e-11
     ch.close()
+
+
+OPENINGS = [(n, p) for n in [(6, 3), (34, 9), (64, 16), (66, 17), (130, 33), (402, 123)] for p in ("fp32", "fp32_offset")]
+
+
+def _opening_pair(size, precision, max_iter):
+    """Two contexts of the single-plane FP32 solve at one state: populations as
+    initialised, the potential moved off its solution, for the last two steps."""
+    from paper_2410_11129_gb300 import fcd
+    cfg = dict(_cfg(*size, mag_tol=1e-4), mag_max_iter=max_iter, precision=precision)
+    a, b = fcd.Channel(cfg), fcd.Channel(cfg)
+    f, g, psi = a.populations()
+    rng = np.random.default_rng(7)
+    psi = (psi + 0.1 * a.derived()["H0"] * rng.standard_normal(psi.shape)).astype(np.float32).astype(np.float64)
+    for ch in (a, b):
+        ch.set_populations(f, g, psi)
+    return a, b, psi
+
+
+@pytest.mark.parametrize("size,precision", OPENINGS)
+def test_opening_of_a_step(size, precision):
+    """The kernel that opens a step against the phase recovery and the sweep of a
+    solve on its own, one cycle each, at the edges of its 64 x 16 patches: the same
+    sums in four dependent colours of about twenty roundings, 80 x 2^-24."""
+    a, b, psi = _opening_pair(size, precision, 1)
+    a.step(1)
+    b.solve_magnetic(1e-30, 1)
+    x, y = a.populations()[2], b.populations()[2]
+    assert np.abs(x - psi).max() > 0
+    assert np.abs(x - y).max() <= 80 * 2.0**-24 * (np.abs(psi).max() + a.derived()["H0"])
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("size,precision", OPENINGS[2:6])
+def test_potential_buffers_take_turns(size, precision):
+    """Without cycles a step leaves exactly 2 psi'(t) - psi'(t-1), through every
+    turn of the three buffers, and a snapshot continues with the same bits."""
+    a, b, prev = _opening_pair(size, precision, 0)
+    a.solve_magnetic(1e-30, 1)
+    cur = a.populations()[2].astype(np.float32)
+    prev = prev.astype(np.float32)
+    assert not np.array_equal(cur, prev)
+    buf = np.empty(a.state_bytes(), np.uint8)
+    for _ in range(4):
+        a.get_state(buf)
+        b.set_state(buf)
+        a.step(1)
+        b.step(1)
+        prev, cur = cur, np.float32(2) * cur - prev
+        for ch in (a, b):
+            assert np.array_equal(ch.populations()[2].astype(np.float32), cur)
+    a.close()
+    b.close()
