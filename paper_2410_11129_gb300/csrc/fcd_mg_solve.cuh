@@ -9,8 +9,8 @@
 // cycle are separated by grid barriers of about 1.5 us, every block takes the
 // same decisions from the same norm, and nothing returns to the host or to a
 // graph node until the solve ends. Measured per step at tolerance 1e-10: 200 x 40
-// 622 -> 245 us (12.0 -> 9.0 residuals), 800 x 100 827 -> 371 us (11.5 -> 8.5);
-// the FP32 pair on 402 x 123 at 1e-5: step 79 -> 48 us. Bound now by the chain of
+// 622 -> 207 us (12.0 -> 8.0 residuals), 800 x 100 827 -> 307 us (11.5 -> 7.7);
+// the FP32 pair on 402 x 123 at 1e-5: step 79 -> 42 us. Bound now by the chain of
 // phases: barriers a quarter, the FP64 residual a fifth (57 cycles per operation
 // of a warp), the single-block levels a fifth.
 //
@@ -42,6 +42,17 @@ constexpr int RT = 128;
 constexpr int SOLVE_WORKERS = SOLVE_THREADS / QT, RESID_WORKERS = SOLVE_THREADS / RT;
 constexpr int FVH = SOLVE_THREADS / 32;        // rows of a coarse-level tile (32 columns)
 static_assert(SOLVE_WORKERS <= 15, "one named barrier per worker, barrier 0 is the block's");
+// A cycle's correction falls short of the smooth errors by about a tenth, so it is
+// scaled. numpy prototype, rate per cycle at 1, 1.04, 1.08 and 1.1: 800 x 100 0.172,
+// 0.140, 0.126, 0.130; 200 x 40 0.163, 0.135, 0.126, 0.141; 400 x 122 0.209, 0.178,
+// 0.138, 0.125; chi = 5 0.316, 0.292, 0.267, 0.241. Not for an odd number of rows,
+// whose cells of three at the wall it overshoots (400 x 123: 0.210, at 1.05 0.295),
+// nor where rows are not merged. Measured, 1 -> 1.08: residuals per solve 8.5 ->
+// 7.6 on 800 x 100 at 1e-10 (485 -> 432 us per step) and 2.73 -> 2.44 at 1e-5 (180 ->
+// 170), 9.0 -> 8.0 on 200 x 40 (270 -> 241): no slower at any tolerance from 1e-4 to
+// 1e-12. Going straight to V-cycles (no two-grid cycles first) takes 457 us
+// per step on 800 x 100 and 251 on 200 x 40.
+constexpr TC OVER = TC(1.08);
 constexpr unsigned SPIN_LIMIT = 1u << 24;      // polls of a grid barrier (seconds)
 
 template <typename T>
@@ -135,7 +146,7 @@ __device__ __forceinline__ void ring_entries(int nx, int ny, int pitch, int x0, 
 // the coarse patch, a quarter or three quarters of the way.
 template <typename T>
 __device__ __forceinline__ void sweep_tile(SweepTile &S, const SolveArgs<T> &A, const Level<TC> &L1, const TC *from,
-                                           TC *to, int bx, int by, int w, int tid) {
+                                           TC *to, TC over, int bx, int by, int w, int tid) {
     const int nx = A.L0.nx, ny = A.L0.ny, pitch = A.L0.pitch, x0 = bx * SX, y0 = by * SY;
     const int qx = 2 * (tid % (SX / 2)), qy = 2 * (tid / (SX / 2));
     TC kv[ring_rows<QT>() + 1], ev[ring_rows<QT>() + 1], rr[4];
@@ -205,7 +216,7 @@ __device__ __forceinline__ void sweep_tile(SweepTile &S, const SolveArgs<T> &A, 
         if (own[c]) {
             const TC v = (off9<TC, true>(nd[c], pat, y, ny) - rr[c]) * inv[c];
             S.se[ly][lx] = v;
-            to[(long long)y * pitch + x0 + lx - 1] = v;
+            to[(long long)y * pitch + x0 + lx - 1] = over * v;
         }
         worker_sync<QT>(w);  // the last one: the tile's shared memory is reused
     }
@@ -780,6 +791,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
     const int max_iter = ctl->max_iter;
     int cur = ctl->cur, iter = 0, heads = 0, twogrid = 0, vcycles = 0;
     unsigned arrivals = 0;
+    const TC over = L[1].ny != A.L0.ny && A.L0.ny % 2 == 0 ? OVER : TC(1);
     auto psi = [&](int c) { return c ? A.L0.r : A.L0.e; };
     // tile t is worker (t / gridDim) % workers of block t % gridDim
     auto each_tile = [&](int w, int workers, auto f) {
@@ -827,9 +839,9 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
             }
         }
         if (!grid_barrier(ctl, arrivals)) return;
-        each_tile(sw, SOLVE_WORKERS, [&](int bx, int by) { sweep_tile<T>(wt[sw].s, A, L[1], nullptr, A.eA, bx, by, sw, st); });
+        each_tile(sw, SOLVE_WORKERS, [&](int bx, int by) { sweep_tile<T>(wt[sw].s, A, L[1], nullptr, A.eA, TC(1), bx, by, sw, st); });
         if (!grid_barrier(ctl, arrivals)) return;
-        each_tile(sw, SOLVE_WORKERS, [&](int bx, int by) { sweep_tile<T>(wt[sw].s, A, L[1], A.eA, A.eB, bx, by, sw, st); });
+        each_tile(sw, SOLVE_WORKERS, [&](int bx, int by) { sweep_tile<T>(wt[sw].s, A, L[1], A.eA, A.eB, over, bx, by, sw, st); });
         if (!grid_barrier(ctl, arrivals)) return;
         iter++;
     }
