@@ -185,12 +185,15 @@ fcd_status fcd_get_derived(const fcd_ctx *ctx, double *out15);
 fcd_status fcd_derive_params(const fcd_params *params, double *out15);
 
 /* Number of kernels launched by this context since create (for accounting;
- * synchronises to read the device-side cycle count). */
+ * synchronises to read the device-side cycle count; a solve in FP64, or in FP32
+ * below a tolerance of 1e-4, is one kernel). */
 long fcd_kernel_launches(const fcd_ctx *ctx);
 
 /* Cumulative potential-solver counters since create: [cycle heads (lattice
  * residual evaluations), V-cycles, two-grid cycles, lattice-sweep cycles,
- * solves stopped at the cycle cap] (synchronises). */
+ * solves stopped at the cycle cap] (synchronises). Lattice-sweep cycles, the
+ * opening of a solve among them, are those of FP32 contexts with a tolerance of
+ * 1e-4 or more; the other forms have none. */
 fcd_status fcd_solver_stats(fcd_ctx *ctx, long long *out5);
 
 /* Rows per tile of the fused collide-stream kernel (Sec. 2.2-2.4 update,
@@ -220,9 +223,10 @@ const char *fcd_last_error(const fcd_ctx *ctx);
  * fcd_batch_tuning): the periodic FP32 instances of one storage form and one
  * level-0 form of the potential (a tolerance below 1e-4 or not) advanced
  * together by one fixed set of kernels per step, each launched once over a
- * work list of tiles that spans them (phase recovery, a single loop of
- * batched multigrid kernels in which every instance runs the cycle its own
- * residual chose, and the fused collide-stream, whose tile height an
+ * work list of tiles that spans them (phase recovery with the opening sweep, a
+ * single loop of batched multigrid kernels in which every instance runs the
+ * cycle its own residual chose or, below 1e-4, every instance's one-kernel
+ * solve, up to eight side by side, and the fused collide-stream, whose tile height an
  * autotuner picks at create by timing), the other instances (FP64, open
  * channels) on their own streams beside them; or every instance's own step
  * graph on its own stream. The first steps time both and keep the faster.

@@ -205,7 +205,7 @@ struct SnapHeader {
     int nx, ny, precision, pitch;
     long long step;
     unsigned long long brk;
-    int cur, pad;  // which level-0 potential buffer is current
+    int cur, pad;  // which level-0 potential buffer is current; 0
 };
 static const unsigned SNAP_VERSION = 4;
 static const unsigned SNAP_MAGIC = 0x46434453u;  // "FCDS"
@@ -243,6 +243,7 @@ struct Engine : fcd_ctx {
     bool use_graph = true;
     bool profiling = false;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
+    cudaEvent_t snap_ev = nullptr;
     long host_kernels = 0;
     int reported_nonconv = 0;
     int copies = 1;  // plane sets per field: 1, or 1 + NT for the tangent context
@@ -281,6 +282,7 @@ struct Engine : fcd_ctx {
         if (cap) cudaStreamDestroy(cap);
         for (auto e : ev)
             if (e) cudaEventDestroy(e);
+        if (snap_ev) cudaEventDestroy(snap_ev);
     }
 
     bool magnetic() const { return D.H0 > 0.0; }
@@ -321,6 +323,7 @@ struct Engine : fcd_ctx {
         CK(cudaMallocHost(&h_unst, sizeof(unsigned long long)));
         CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
         for (auto &e : ev) CK(cudaEventCreate(&e));
+        CK(cudaEventCreateWithFlags(&snap_ev, cudaEventDisableTiming));
         mg = mg_create<T>(prm.nx, prm.ny, pitch, k, psiA, psiB, ctl, alloc, release, user, err,
                           sizeof err, comp, nullptr, psiP);
         if (!mg) return FCD_ENOMEM;
@@ -914,8 +917,8 @@ struct Engine : fcd_ctx {
     // buffers travel, with the device's current-buffer index, so neither call
     // needs to read the control block on the host: each is one stream of
     // asynchronous copies and a single synchronisation. Where the three buffers
-    // take turns they are stored by role (current, idle, previous step's), for
-    // which get_state reads the control block with its first synchronisation.
+    // take turns they are stored by role (current, idle, previous step's): get_state
+    // reads the control block first and waits for it while the populations travel.
     size_t state_bytes() const override {
         return sizeof(SnapHeader) + 27 * (size_t)ps * sizeof(S) + 3 * psi_bytes();
     }
@@ -923,15 +926,12 @@ struct Engine : fcd_ctx {
     fcd_status get_state(void *dst, size_t bytes) override {
         if (!dst || bytes < state_bytes()) return fail(FCD_EINVAL, "snapshot buffer too small");
         cudaStream_t s = stream;
+        char *d = static_cast<char *>(dst);
         T *bufs[3] = {psiA, psiB, psiP};
+        CK(cudaStreamSynchronize(s));  // the staging header may still be in flight
         if (turns()) {
-            if (sync_ctl() != FCD_OK) return FCD_ECUDA;
-            const int now = h_ctl->cur, prev = 2 - h_ctl->back;
-            bufs[0] = psi_buffer(now, psiA, psiB, psiP);
-            bufs[1] = psi_buffer(3 - now - prev, psiA, psiB, psiP);
-            bufs[2] = psi_buffer(prev, psiA, psiB, psiP);
-        } else {
-            CK(cudaStreamSynchronize(s));  // the staging header may still be in flight
+            CK(cudaMemcpyAsync(h_ctl, ctl, sizeof(MgCtl), cudaMemcpyDeviceToHost, s));
+            CK(cudaEventRecord(snap_ev, s));
         }
         SnapHeader &h = *h_snap;
         std::memset(&h, 0, sizeof h);
@@ -942,7 +942,6 @@ struct Engine : fcd_ctx {
         h.precision = prm.precision;
         h.pitch = pitch;
         h.step = step;
-        char *d = static_cast<char *>(dst);
         CK(cudaMemcpyAsync(d, &h, sizeof h, cudaMemcpyDefault, s));
         CK(cudaMemcpyAsync(d + offsetof(SnapHeader, brk), brk, sizeof(unsigned long long),
                            cudaMemcpyDefault, s));
@@ -953,6 +952,13 @@ struct Engine : fcd_ctx {
         off += 9 * ps * sizeof(S);
         CK(cudaMemcpyAsync(d + off, g[cur], 18 * ps * sizeof(S), cudaMemcpyDefault, s));
         off += 18 * ps * sizeof(S);
+        if (turns()) {
+            CK(cudaEventSynchronize(snap_ev));
+            const int now = h_ctl->cur, prev = 2 - h_ctl->back;
+            bufs[0] = psi_buffer(now, psiA, psiB, psiP);
+            bufs[1] = psi_buffer(3 - now - prev, psiA, psiB, psiP);
+            bufs[2] = psi_buffer(prev, psiA, psiB, psiP);
+        }
         for (T *q : bufs) {
             CK(cudaMemcpyAsync(d + off, q, psi_bytes(), cudaMemcpyDefault, s));
             off += psi_bytes();
@@ -989,8 +995,9 @@ struct Engine : fcd_ctx {
             CK(cudaMemcpyAsync(q, p + off, psi_bytes(), cudaMemcpyDefault, s));
             off += psi_bytes();
         }
-        CK(cudaMemcpyAsync(&ctl->cur, &h.cur, sizeof(int), cudaMemcpyHostToDevice, s));
-        CK(cudaMemsetAsync(&ctl->back, 0, sizeof(int), s));
+        static_assert(offsetof(MgCtl, back) == offsetof(MgCtl, cur) + sizeof(int), "cur and back in one copy");
+        h.pad = 0;  // back: the third buffer is the previous step's
+        CK(cudaMemcpyAsync(&ctl->cur, &h.cur, 2 * sizeof(int), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(brk, &h.brk, sizeof(unsigned long long), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(d_step, &h.step, sizeof(long long), cudaMemcpyHostToDevice, s));
         CK(cudaMemsetAsync(unst, 0xff, sizeof(unsigned long long), s));
