@@ -547,7 +547,10 @@ struct Engine : fcd_ctx {
     // sweeps, 2 a two-grid cycle) and ends with the next head, which sets the loop
     // condition, and then the collide-stream that the gate left out. Measured
     // per step (steps back to back): 1600 x 200 49.4 -> 45.1 us, 2400 x 300 87.6 ->
-    // 80.4 us, 900 x 150 open 46.9 -> 42.0 us, the same bits.
+    // 80.4 us, 900 x 150 open 46.9 -> 42.0 us, the same bits. The one use it slows:
+    // many contexts stepped in turn on the legacy default stream, which orders
+    // itself against every graph's branches (4 contexts 28.0 -> 28.5 us per step, 24
+    // 64 -> 69, 96 131 -> 181; on an own stream 96 go from 65 to 60).
     fcd_status capture_solve_and_collide(int c, int sm, cudaStream_t s) {
         cudaStreamCaptureStatus cs;
         cudaGraph_t gcap;
