@@ -43,7 +43,9 @@ typedef enum {
     FCD_OK = 0,
     FCD_EINVAL = 1,     /* bad argument or parameter set */
     FCD_ENOMEM = 2,     /* device allocation failed */
-    FCD_ECUDA = 3,      /* a CUDA call failed; the message names it */
+    FCD_ECUDA = 3,      /* a CUDA call failed, or a potential solve was given up at a
+                         * grid barrier after seconds (then until a new state is
+                         * set); the message names it */
     FCD_ENOCONV = 4,    /* potential solve hit its cycle cap before the tolerance */
     FCD_EUNSTABLE = 5,  /* non-finite values detected: a collision that produced a
                          * non-finite velocity or pressure marks its step on the

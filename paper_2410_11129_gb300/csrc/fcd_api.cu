@@ -185,6 +185,7 @@ struct fcd_ctx {
     virtual fcd_status set_profiling(int on) = 0;
     virtual fcd_status profile(double *ms) = 0;
     virtual int collide_tile_h() const = 0;
+    virtual fcd_status set_barrier_polls(unsigned polls) = 0;
     fcd_status fail(fcd_status s, const char *fmt, ...) {
         va_list ap;
         va_start(ap, fmt);
@@ -228,7 +229,8 @@ struct Engine : fcd_ctx {
     MgCtl *ctl = nullptr;
     MgHost<T> *mg = nullptr;
     unsigned long long *brk = nullptr;
-    unsigned long long *unst = nullptr;  // first step with a non-finite collision (~0: none)
+    Trouble *trouble = nullptr;          // what went wrong so far
+    unsigned long long *unst = nullptr;  // &trouble->unst
     long long *d_step = nullptr;
     double *obs_scratch = nullptr;
     ObsOut *obs_out = nullptr;
@@ -236,7 +238,7 @@ struct Engine : fcd_ctx {
     ObsPack *h_obs = nullptr;  // pinned; the last kernel of an observation writes it
     SnapHeader *h_snap = nullptr;  // pinned staging of snapshot headers
     unsigned long long *h_brk = nullptr;
-    unsigned long long *h_unst = nullptr;
+    Trouble *h_trouble = nullptr;
     cudaStream_t cap = nullptr;
     cudaGraph_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
     cudaGraphExec_t gexec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
@@ -278,7 +280,7 @@ struct Engine : fcd_ctx {
         if (h_obs) cudaFreeHost(h_obs);
         if (h_snap) cudaFreeHost(h_snap);
         if (h_brk) cudaFreeHost(h_brk);
-        if (h_unst) cudaFreeHost(h_unst);
+        if (h_trouble) cudaFreeHost(h_trouble);
         if (cap) cudaStreamDestroy(cap);
         for (auto e : ev)
             if (e) cudaEventDestroy(e);
@@ -308,24 +310,25 @@ struct Engine : fcd_ctx {
         macro = dalloc(3 * ps * sizeof(T));
         ctl = reinterpret_cast<MgCtl *>(dalloc(sizeof(MgCtl)));
         brk = reinterpret_cast<unsigned long long *>(dalloc(sizeof(unsigned long long)));
-        unst = reinterpret_cast<unsigned long long *>(dalloc(sizeof(unsigned long long)));
+        trouble = reinterpret_cast<Trouble *>(dalloc(sizeof(Trouble)));
         d_step = reinterpret_cast<long long *>(dalloc(sizeof(long long)));
         obs_scratch = reinterpret_cast<double *>(dalloc(observe_scratch_doubles(prm.nx, prm.ny) * sizeof(double)));
         obs_out = reinterpret_cast<ObsOut *>(dalloc(sizeof(ObsOut)));
         for (void *p : {f[0], f[1], g[0], g[1], (void *)phi1, (void *)phi2, (void *)k, (void *)psiA,
-                        (void *)psiB, (void *)psiP, (void *)macro, (void *)ctl, (void *)brk, (void *)unst, (void *)d_step,
+                        (void *)psiB, (void *)psiP, (void *)macro, (void *)ctl, (void *)brk, (void *)trouble, (void *)d_step,
                         (void *)obs_scratch, (void *)obs_out})
             if (!p) return fail(FCD_ENOMEM, "device allocation failed");
         CK(cudaMallocHost(&h_ctl, sizeof(MgCtl)));
         CK(cudaMallocHost(&h_obs, sizeof(ObsPack)));
         CK(cudaMallocHost(&h_snap, sizeof(SnapHeader)));
         CK(cudaMallocHost(&h_brk, sizeof(unsigned long long)));
-        CK(cudaMallocHost(&h_unst, sizeof(unsigned long long)));
+        CK(cudaMallocHost(&h_trouble, sizeof(Trouble)));
+        unst = &trouble->unst;
         CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
         for (auto &e : ev) CK(cudaEventCreate(&e));
         CK(cudaEventCreateWithFlags(&snap_ev, cudaEventDisableTiming));
         mg = mg_create<T>(prm.nx, prm.ny, pitch, k, psiA, psiB, ctl, alloc, release, user, err,
-                          sizeof err, comp, nullptr, psiP);
+                          sizeof err, trouble, comp, nullptr, psiP);
         if (!mg) return FCD_ENOMEM;
         cudaStream_t s = stream;
         CK(cudaMemsetAsync(ctl, 0, sizeof(MgCtl), s));
@@ -333,7 +336,8 @@ struct Engine : fcd_ctx {
         CK(cudaMemsetAsync(psiB, 0, psi_bytes(), s));
         CK(cudaMemsetAsync(psiP, 0, psi_bytes(), s));
         CK(cudaMemsetAsync(brk, 0xff, sizeof(unsigned long long), s));
-        CK(cudaMemsetAsync(unst, 0xff, sizeof(unsigned long long), s));
+        *h_trouble = Trouble{~0ull, 0, BARRIER_POLLS};
+        CK(cudaMemcpyAsync(trouble, h_trouble, sizeof(Trouble), cudaMemcpyHostToDevice, s));
         CK(cudaMemsetAsync(d_step, 0, sizeof(long long), s));
         // padding columns of every plane stay zero
         for (int b = 0; b < 2; b++) {
@@ -495,8 +499,7 @@ struct Engine : fcd_ctx {
             CK(mg_solve<T>(m, P.H0c, P.H0s, s));
             CK(cudaMemcpyAsync(h_ctl, c, sizeof(MgCtl), cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
-            if (h_ctl->stuck) return fail(FCD_ECUDA, "a grid barrier of the potential solve timed out");
-            return FCD_OK;
+            return h_ctl->stuck ? fail_stuck() : FCD_OK;
         }
         if constexpr (sizeof(T) == 4) {
             if (!opened) mg_presmooth(m, P.H0c, P.H0s, s);
@@ -739,13 +742,13 @@ struct Engine : fcd_ctx {
 
     fcd_status observe(fcd_obs *o) override {
         cudaStream_t s = stream;
-        launch_observe<T>(mode, P, g[cur], obs_scratch, obs_out, s, prm.open_x, ObsTail{h_obs, brk, unst, ctl});
+        launch_observe<T>(mode, P, g[cur], obs_scratch, obs_out, s, prm.open_x, ObsTail{h_obs, brk, trouble, ctl});
         host_kernels += 3;
         CK(cudaGetLastError());
         CK(cudaStreamSynchronize(s));
         const ObsOut &r = h_obs->o;
         *h_brk = h_obs->brk;
-        *h_unst = h_obs->unst;
+        *h_trouble = h_obs->trouble;
         *h_ctl = h_obs->ctl;
         std::memset(o, 0, sizeof *o);
         o->step = step;
@@ -775,8 +778,8 @@ struct Engine : fcd_ctx {
         }
         o->mag_iters = magnetic() ? h_ctl->last_iters : 0;
         o->mag_resid = magnetic() ? h_ctl->last_resid : 0.0;
-        if (h_ctl->stuck) return fail(FCD_ECUDA, "a grid barrier of the potential solve timed out");
-        if (unstable_status() != FCD_OK) return FCD_EUNSTABLE;
+        const fcd_status ts = trouble_status();
+        if (ts != FCD_OK) return ts;
         if (r.nonfinite) return fail(FCD_EUNSTABLE, "non-finite phase field at step %ld", step);
         if (h_ctl->nonconv_count > reported_nonconv) {
             reported_nonconv = h_ctl->nonconv_count;
@@ -786,12 +789,32 @@ struct Engine : fcd_ctx {
         return FCD_OK;
     }
 
-    // FCD_EUNSTABLE once a collision produced a non-finite velocity or
-    // pressure; h_unst must have been copied in the caller's synchronised batch.
-    fcd_status unstable_status() {
-        if (*h_unst == ~0ull) return FCD_OK;
+    // FCD_ECUDA once a solve was given up at a grid barrier, FCD_EUNSTABLE once a
+    // collision produced a non-finite velocity or pressure; h_trouble must have
+    // been copied in the caller's synchronised batch.
+    fcd_status fail_stuck() { return fail(FCD_ECUDA, "a grid barrier of a potential solve timed out"); }
+    fcd_status trouble_status() {
+        if (h_trouble->stuck) return fail_stuck();
+        if (h_trouble->unst == ~0ull) return FCD_OK;
         return fail(FCD_EUNSTABLE, "non-finite velocity or pressure, first in step %llu (now at step %ld)",
-                    *h_unst, step);
+                    h_trouble->unst, step);
+    }
+    // For tests of the bounded wait: later solves give up at a barrier after so
+    // many polls (0: the default).
+    fcd_status set_barrier_polls(unsigned polls) override {
+        const unsigned v = polls ? polls : BARRIER_POLLS;
+        CK(cudaDeviceSynchronize());  // a batch runs its instances' solves on other streams
+        CK(cudaMemcpy(&trouble->polls, &v, sizeof v, cudaMemcpyHostToDevice));
+        return FCD_OK;
+    }
+    // The record of a context that starts from a new state.
+    fcd_status clear_trouble(cudaStream_t s) {
+        CK(cudaMemsetAsync(unst, 0xff, sizeof(unsigned long long), s));
+        if (magnetic() && mg_one_kernel<T>(mg)) {
+            CK(cudaMemsetAsync(&trouble->stuck, 0, sizeof(int), s));
+            CK(cudaMemsetAsync(&ctl->stuck, 0, sizeof(int), s));
+        }
+        return FCD_OK;
     }
 
     double *staging(size_t doubles) {
@@ -842,11 +865,11 @@ struct Engine : fcd_ctx {
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess && !direct) e = cudaMemcpyAsync(dst, st, N * sizeof(double), cudaMemcpyDefault, s);
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(h_unst, unst, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
+            e = cudaMemcpyAsync(h_trouble, trouble, sizeof(Trouble), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) rc = fail(FCD_ECUDA, "get_field: %s", cudaGetErrorString(e));
         if (!direct) cudaFree(st);
-        if (rc == FCD_OK) rc = unstable_status();  // the field is delivered all the same
+        if (rc == FCD_OK) rc = trouble_status();  // the field is delivered all the same
         return rc;
     }
 
@@ -862,7 +885,7 @@ struct Engine : fcd_ctx {
             dg = st + 9 * N;
             dp = st + 27 * N;
         }
-        launch_export<T>(mode, P, f[cur], g[cur], df, dg, s, unst, h_unst);
+        launch_export<T>(mode, P, f[cur], g[cur], df, dg, s, trouble, h_trouble);
         if (dp) launch_psi_to_f64<T>(ctl, psiA, psiB, psiP, prm.nx, prm.ny, pitch, dp, s);
         host_kernels += dp ? 2 : 1;
         cudaError_t e = cudaGetLastError();
@@ -874,7 +897,7 @@ struct Engine : fcd_ctx {
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (st) cudaFree(st);
         if (e != cudaSuccess) return fail(FCD_ECUDA, "get_populations: %s", cudaGetErrorString(e));
-        return unstable_status();  // the populations are delivered all the same
+        return trouble_status();  // the populations are delivered all the same
     }
 
     fcd_status set_pops(const double *fi, const double *gi, const double *pi, long st_) override {
@@ -905,7 +928,7 @@ struct Engine : fcd_ctx {
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = cudaMemsetAsync(brk, 0xff, sizeof(unsigned long long), s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(unst, 0xff, sizeof(unsigned long long), s);
+        if (e == cudaSuccess && clear_trouble(s) != FCD_OK) e = cudaErrorUnknown;
         long long s64 = st_;
         if (e == cudaSuccess) e = cudaMemcpyAsync(d_step, &s64, sizeof(long long), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -966,8 +989,10 @@ struct Engine : fcd_ctx {
             CK(cudaMemcpyAsync(d + off, q, psi_bytes(), cudaMemcpyDefault, s));
             off += psi_bytes();
         }
+        const bool one = magnetic() && mg_one_kernel<T>(mg);
+        if (one) CK(cudaMemcpyAsync(h_trouble, trouble, sizeof(Trouble), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        return FCD_OK;
+        return one && h_trouble->stuck ? fail_stuck() : FCD_OK;
     }
 
     fcd_status set_state(const void *src, size_t bytes) override {
@@ -1003,7 +1028,8 @@ struct Engine : fcd_ctx {
         CK(cudaMemcpyAsync(&ctl->cur, &h.cur, 2 * sizeof(int), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(brk, &h.brk, sizeof(unsigned long long), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(d_step, &h.step, sizeof(long long), cudaMemcpyHostToDevice, s));
-        CK(cudaMemsetAsync(unst, 0xff, sizeof(unsigned long long), s));
+        const fcd_status ct = clear_trouble(s);
+        if (ct != FCD_OK) return ct;
         CK(cudaStreamSynchronize(s));
         step = (long)h.step;
         return FCD_OK;
@@ -1190,7 +1216,7 @@ struct TangentEngine : Engine<double> {
             // every tangent solve of a step has the primal solve's k, and the
             // primal solve forms the lattice coefficients first: share them
             mgt[c] = mg_create<double>(prm.nx, prm.ny, pitch, k, tA[c], tB[c], ctlt[c], alloc,
-                                       release, user, err, sizeof err, 0, mg);
+                                       release, user, err, sizeof err, trouble, 0, mg);
             if (!mgt[c]) return FCD_ENOMEM;
             mg_set_rhs<double>(mgt[c], rhst[c]);
             mg_set_share<double>(mgt[c], NT);  // the NT solves of a step run side by side
@@ -1324,6 +1350,7 @@ struct TangentEngine : Engine<double> {
         if (st != FCD_OK && st != FCD_ENOCONV) return st;
         cudaStream_t s = stream;
         TanCtls ctls;
+        ctls.trouble = trouble;
         for (int c = 0; c < NT; c++) ctls.c[c] = mgt[c] ? ctlt[c] : nullptr;
         launch_tangent_obs(P, static_cast<const double *>(g[cur]), obs_out, tobs, tan_out, ctls, s);
         host_kernels += 2;
@@ -1343,6 +1370,7 @@ struct TangentEngine : Engine<double> {
             o->dlx_o[c] = h_tan->dlx[c];
             o->dly_o[c] = h_tan->dly[c];
         }
+        if (h_tan->stuck) return fail_stuck();
         if (nonconv > reported_tangent_nonconv) {
             reported_tangent_nonconv = nonconv;
             return fail(FCD_ENOCONV, "a tangent potential solve stopped at the cycle cap");
@@ -1648,7 +1676,7 @@ struct AdjointEngine : Engine<double> {
         cudaStream_t s = stream;
         if (!mga && magnetic()) {
             mga = mg_create<double>(prm.nx, prm.ny, pitch, k, lamA, lamB, ctla, alloc, release, user, err,
-                                    sizeof err);
+                                    sizeof err, trouble);
             if (!mga) return FCD_ENOMEM;
             mg_set_rhs<double>(mga, rhs);
         }
@@ -1757,6 +1785,8 @@ struct AdjointEngine : Engine<double> {
             CK(cudaMemcpy(h_ctl, ctla, sizeof(MgCtl), cudaMemcpyDeviceToHost));
             o->solve_cycles = h_ctl->total_cycles + h_ctl->twogrid_cycles + h_ctl->smooth_cycles;
             o->capped_solves = h_ctl->nonconv_count;  // the control block is cleared per sweep
+            CK(cudaMemcpy(h_trouble, trouble, sizeof(Trouble), cudaMemcpyDeviceToHost));
+            if (h_trouble->stuck) return fail_stuck();
             if (o->capped_solves > 0)
                 return fail(FCD_ENOCONV, "%ld adjoint potential solves stopped at the cycle cap",
                             o->capped_solves);
@@ -2045,6 +2075,10 @@ fcd_status fcd_collide_tile_height(const fcd_ctx *c, int *rows) {
     *rows = c->collide_tile_h();
     return FCD_OK;
 }
+
+// Not part of the interface (fcd.h): tests make a grid barrier of this context's
+// solves run out.
+fcd_status fcd_set_barrier_polls(fcd_ctx *c, unsigned polls) { return c ? c->set_barrier_polls(polls) : FCD_EINVAL; }
 
 fcd_status fcd_set_profiling(fcd_ctx *c, int enable) { return c ? c->set_profiling(enable) : FCD_EINVAL; }
 

@@ -53,7 +53,6 @@ static_assert(SOLVE_WORKERS <= 15, "one named barrier per worker, barrier 0 is t
 // 1e-12. Going straight to V-cycles (no two-grid cycles first) takes 457 us
 // per step on 800 x 100 and 251 on 200 x 40.
 constexpr TC OVER = TC(1.08);
-constexpr unsigned SPIN_LIMIT = 1u << 24;      // polls of a grid barrier (seconds)
 
 template <typename T>
 struct SolveArgs {
@@ -62,13 +61,14 @@ struct SolveArgs {
     int nl, lc;
     T H0c, H0s;
     MgCtl *ctl;
+    Trouble *trouble;       // the context's: a barrier that gives up leaves its mark there
     int form_coef;          // FP64: form the node coefficients (else another solve of this k has)
     TC *r0, *eA, *eB, *k0;  // lattice planes of the correction: residual, e (two buffers), k
 };
 
 // Grid barrier of a cooperative launch; ctl->bar counts arrivals from the
-// solve's reset on. False once a barrier has timed out.
-__device__ __forceinline__ bool grid_barrier(MgCtl *c, unsigned &arrivals) {
+// solve's reset on. False once a barrier has timed out (tr: the context's record).
+__device__ __forceinline__ bool grid_barrier(MgCtl *c, Trouble *tr, unsigned polls, unsigned &arrivals) {
     __shared__ int ok;
     arrivals += gridDim.x;
     __syncthreads();
@@ -80,8 +80,9 @@ __device__ __forceinline__ bool grid_barrier(MgCtl *c, unsigned &arrivals) {
         while (true) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&c->bar) : "memory");
             if (seen >= arrivals) break;
-            if (++spin >= SPIN_LIMIT || ((spin & 1023u) == 0 && *(volatile int *)&c->stuck)) {
+            if (++spin >= polls || ((spin & 1023u) == 0 && *(volatile int *)&tr->stuck)) {
                 good = false;
+                atomicExch(&tr->stuck, 1);
                 atomicExch(&c->stuck, 1);
                 break;
             }
@@ -775,7 +776,11 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
     __shared__ double norm;
     MgCtl *const ctl = A.ctl;
     const int tid = threadIdx.x, nl = A.nl, lc = A.lc;
-    if (ctl->stuck) return;  // an earlier solve's barrier timed out
+    if (A.trouble->stuck) {  // an earlier solve's barrier timed out
+        if (blockIdx.x == 0 && tid == 0) ctl->stuck = 1;
+        return;
+    }
+    const unsigned polls = A.trouble->polls;
     if (tid < nl) L[tid] = A.lv[tid];
     __syncthreads();
     if (tid == 0) {
@@ -813,7 +818,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
             for (int q = 1; q < SOLVE_THREADS / 32; q++) mx = max(mx, wmax[q]);
             if (mx > 0) atomic_max_nonneg(&ctl->norm_slot[heads & 3], max_value(mx, T(0)));
         }
-        if (!grid_barrier(ctl, arrivals)) return;
+        if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
         if (tid == 0) {
             norm = __longlong_as_double((long long)__ldcg(&ctl->norm_slot[heads & 3]));
             if (blockIdx.x == 0) ctl->norm_slot[(heads + 2) & 3] = 0ull;  // two heads on, two barriers away
@@ -828,21 +833,21 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
             const bool setup = vcycles++ == 0;
             for (int l = 1; l < lc; l++) {
                 fv_phase<0>(fv, L[l], L[l + 1], NU_PRE);
-                if (!grid_barrier(ctl, arrivals)) return;
+                if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
                 restrict_phase(L[l], L[l + 1], setup);
-                if (!grid_barrier(ctl, arrivals)) return;
+                if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
             }
             if (blockIdx.x == 0) bottom_phase(bottom, B, L, lc, nl, setup);
             for (int l = lc - 1; l >= 1; l--) {
-                if (!grid_barrier(ctl, arrivals)) return;
+                if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
                 fv_phase<1>(fv, L[l], L[l + 1], NU_POST);
             }
         }
-        if (!grid_barrier(ctl, arrivals)) return;
+        if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
         each_tile(sw, SOLVE_WORKERS, [&](int bx, int by) { sweep_tile<T>(wt[sw].s, A, L[1], nullptr, A.eA, TC(1), bx, by, sw, st); });
-        if (!grid_barrier(ctl, arrivals)) return;
+        if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
         each_tile(sw, SOLVE_WORKERS, [&](int bx, int by) { sweep_tile<T>(wt[sw].s, A, L[1], A.eA, A.eB, over, bx, by, sw, st); });
-        if (!grid_barrier(ctl, arrivals)) return;
+        if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
         iter++;
     }
     if (blockIdx.x == 0 && tid == 0) {
