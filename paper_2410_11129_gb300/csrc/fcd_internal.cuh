@@ -171,6 +171,7 @@ struct MgCtl {
     // solves that run as one cooperative kernel (fcd_mg_solve.cuh); reset with the solve
     unsigned long long norm_slot[4];  // max |r| of the last heads (bits of doubles >= 0)
     unsigned bar;                     // arrivals at the kernel's grid barriers
+    double scale;                     // size of the right-hand side: H0, or max |rhs| where it is explicit
     int stuck;                        // this block's solve was given up (Trouble::stuck)
 };
 
@@ -186,7 +187,7 @@ constexpr unsigned BARRIER_POLLS = 1u << 24;  // seconds
 template <typename T>
 __host__ __device__ __forceinline__ T *psi_buffer(int i, T *a, T *b, T *c) { return i == 0 ? a : (i == 1 ? b : c); }
 // start of a potential solve (one thread)
-__device__ __forceinline__ void mg_reset_ctl(MgCtl *c, double tolH0, int max_iter) {
+__device__ __forceinline__ void mg_reset_ctl(MgCtl *c, double tolH0, int max_iter, double scale) {
     c->norm_bits = 0ull;
     c->iter = 0;
     c->done = 0;
@@ -201,6 +202,7 @@ __device__ __forceinline__ void mg_reset_ctl(MgCtl *c, double tolH0, int max_ite
     c->solve_heads = 0;
     for (int q = 0; q < 4; q++) c->norm_slot[q] = 0ull;
     c->bar = 0u;
+    c->scale = scale;
 }
 
 // What the phase kernel does besides Eq. 32: reset the solve's control block

@@ -54,6 +54,32 @@ static_assert(SOLVE_WORKERS <= 15, "one named barrier per worker, barrier 0 is t
 // per step on 800 x 100 and 251 on 200 x 40.
 constexpr TC OVER = TC(1.08);
 
+// The FP32 residual and correction are in units of a power of two near the
+// right-hand side's size (MgCtl::scale), which is the caller's: the seed of a
+// gradient may be 1e-60, far below the FP32 range. A power of two changes no
+// bits within that range. e: its exponent; 0 where there is no such size.
+template <typename T>
+struct Unit {
+    int e;
+    T value, inverse;
+    __device__ __forceinline__ explicit Unit(double scale) {
+        const int b = (__double2hiint(scale) >> 20) & 0x7ff;
+        e = b == 0 || b == 0x7ff ? 0 : b - 1023;
+        if (sizeof(T) == 4 && (e < -100 || e > 100)) e = 0;  // such a pair has left the FP32 range itself
+        e = e < -1000 ? -1000 : (e > 1000 ? 1000 : e);
+        value = T(__hiloint2double((1023 + e) << 20, 0));
+        inverse = T(__hiloint2double((1023 - e) << 20, 0));
+    }
+    // v in this unit
+    __device__ __forceinline__ TC of(float v) const { return v * (float)inverse; }
+    // by its exponent, on the integer pipe: FP64 arithmetic bounds the residual
+    // (a value that is not finite ends the solve at its norm)
+    __device__ __forceinline__ TC of(double v) const {
+        const int hi = __double2hiint(v), b = (hi >> 20) & 0x7ff, to = b == 0 ? 0 : min(max(b - e, 0), 0x7ff);
+        return TC(__hiloint2double((hi & 0x800fffff) | (to << 20), __double2loint(v)));
+    }
+};
+
 template <typename T>
 struct SolveArgs {
     Level<T> L0;
@@ -246,7 +272,7 @@ __device__ __forceinline__ T off9_two(const Node9<T> &n, PF pat, int y, int ny) 
     return s[0] + s[1];
 }
 
-// psi' of a tile (plus the correction e where there is one: written to psi_new),
+// psi' of a tile (plus the correction e, in units of `unit`, where there is one: written to psi_new),
 // its residual (to r0) and the residual summed onto the tile's level-1 cells;
 // returns the thread's max |r| (max_bits). A thread takes two neighbouring nodes
 // of a row, and the two rows of a cell sit 16 lanes apart. first: the solve's
@@ -256,8 +282,8 @@ __device__ __forceinline__ T off9_two(const Node9<T> &n, PF pat, int y, int ny) 
 // neighbours are ghosts.
 template <typename T, bool COMP>
 __device__ __forceinline__ long long resid_tile(ResidTile<T, COMP> &S, const SolveArgs<T> &A, const Level<TC> &L1,
-                                                const T *psi, T *psi_new, const TC *e, bool first, int bx, int by,
-                                                int w, int tid) {
+                                                const T *psi, T *psi_new, const TC *e, const Unit<T> &unit, bool first,
+                                                int bx, int by, int w, int tid) {
     const Level<T> &L0 = A.L0;
     const int nx = L0.nx, ny = L0.ny, pitch = L0.pitch, x0 = bx * SX, y0 = by * SY;
     const long long ps = (long long)pitch * ny;
@@ -296,8 +322,8 @@ __device__ __forceinline__ long long resid_tile(ResidTile<T, COMP> &S, const Sol
         });
         ring_entries<RT>(nx, ny, pitch, x0, y0, tid, [&](int q, int ly, int lx, long long n, bool inside) {
             if (e) {
-                if constexpr (COMP) comp_add(pv[q], lv[q], ev[q]);
-                else pv[q] += T(ev[q]);
+                if constexpr (COMP) comp_add(pv[q], lv[q], ev[q] * unit.value);
+                else pv[q] = fma(T(ev[q]), unit.value, pv[q]);
             }
             S.sp[ly][lx] = pv[q];
             if constexpr (COMP) S.sl[ly][lx] = lv[q];
@@ -342,7 +368,7 @@ __device__ __forceinline__ long long resid_tile(ResidTile<T, COMP> &S, const Sol
             }
             r = nd.b - (off9_two<T>(nd, pat, j, ny) - nd.diag * S.sp[ly][lx]);
         }
-        A.r0[n] = TC(r);
+        A.r0[n] = unit.of(r);
         sum += r;
         if (first) ks += S.sk[ly][lx];
         mx = max(mx, max_bits(r));
@@ -365,7 +391,7 @@ __device__ __forceinline__ long long resid_tile(ResidTile<T, COMP> &S, const Sol
     if (live && (!merged || (tid & (SX / 2)) == 0)) {
         const int I = ia / 2, J = merged ? j0 / 2 : j0;
         const long long q = (long long)J * L1.pitch + I;
-        L1.b[q] = TC(sum);
+        L1.b[q] = unit.of(sum);
         if (first) L1.k[q] = TC(ks / (T(L1.wx[I]) * T(L1.wy[J])));  // unit lattice cells
     }
     worker_sync<RT>(w);
@@ -793,6 +819,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
     __syncthreads();
     const int gx = (A.L0.nx + SX - 1) / SX, tiles = gx * ((A.L0.ny + SY - 1) / SY);
     const double tol = ctl->tolH0;
+    const Unit<T> unit(ctl->scale);
     const int max_iter = ctl->max_iter;
     int cur = ctl->cur, iter = 0, heads = 0, twogrid = 0, vcycles = 0;
     unsigned arrivals = 0;
@@ -806,7 +833,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
     while (true) {
         long long mx = 0;
         each_tile(rw, RESID_WORKERS, [&](int bx, int by) {
-            mx = max(mx, resid_tile<T, COMP>(wt[rw].r, A, L[1], psi(cur), psi(cur ^ 1), iter ? A.eB : nullptr,
+            mx = max(mx, resid_tile<T, COMP>(wt[rw].r, A, L[1], psi(cur), psi(cur ^ 1), iter ? A.eB : nullptr, unit,
                                              heads == 0, bx, by, rw, rt));
         });
         if (iter) cur ^= 1;
