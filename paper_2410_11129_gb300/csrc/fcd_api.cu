@@ -550,7 +550,10 @@ struct Engine : fcd_ctx {
     // sweeps, 2 a two-grid cycle) and ends with the next head, which sets the loop
     // condition, and then the collide-stream that the gate left out. Measured
     // per step (steps back to back): 1600 x 200 49.4 -> 45.1 us, 2400 x 300 87.6 ->
-    // 80.4 us, 900 x 150 open 46.9 -> 42.0 us, the same bits. The one use it slows:
+    // 80.4 us, 900 x 150 open 46.9 -> 42.0 us, the same bits. While profiling the
+    // collide-stream follows the IF node instead (no gate, no branch): an event
+    // between the two stages has no place beside the IF node, nor in its body.
+    // The one use it slows:
     // many contexts stepped in turn on the legacy default stream, which orders
     // itself against every graph's branches (4 contexts 28.0 -> 28.5 us per step, 24
     // 64 -> 69, 96 131 -> 181; on an own stream 96 go from 65 to 60).
@@ -621,7 +624,7 @@ struct Engine : fcd_ctx {
             e = cudaStreamEndCapture(bs, &out);
         }
         // after the loop: the collide-stream that the gate left out
-        if (e == cudaSuccess) {
+        if (e == cudaSuccess && !profiling) {
             e = cudaStreamBeginCaptureToGraph(bs, ifbody, &wnode, nullptr, 1, cudaStreamCaptureModeThreadLocal);
             if (e == cudaSuccess) {
                 enqueue_post(c, sm != 0, bs);
@@ -630,7 +633,12 @@ struct Engine : fcd_ctx {
         }
         cudaStreamDestroy(bs);
         CK(e);
-        if (profiling) CK(cudaEventRecordWithFlags(ev[2], s, cudaEventRecordExternal));
+        if (profiling) {
+            CK(cudaStreamUpdateCaptureDependencies(s, &ifnode, nullptr, 1, cudaStreamSetCaptureDependencies));
+            CK(cudaEventRecordWithFlags(ev[2], s, cudaEventRecordExternal));
+            enqueue_post(c, sm != 0, s);
+            return FCD_OK;
+        }
         enqueue_post(c, sm != 0, s, &ctl->first_done);
         CK(cudaStreamUpdateCaptureDependencies(s, &ifnode, nullptr, 1, cudaStreamAddCaptureDependencies));
         return FCD_OK;
