@@ -138,7 +138,9 @@ void fcd_set_allocator(fcd_alloc_fn alloc, fcd_free_fn release, void *user);
  * phase. *out is NULL on failure. */
 fcd_status fcd_create(const fcd_params *params, fcd_ctx **out);
 
-/* Queue later work on this cudaStream_t (passed as void*). */
+/* Queue later work on this cudaStream_t (passed as void*). On the legacy default
+ * stream steps may run on streams of the context that keep that stream's order
+ * with the caller's work; contexts stepped in turn there may then overlap. */
 fcd_status fcd_set_stream(fcd_ctx *ctx, void *cuda_stream);
 
 /* Advance n >= 0 coupled steps: phase recovery (Eq. 32), permeability (Eq. 8),

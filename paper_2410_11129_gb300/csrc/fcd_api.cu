@@ -246,6 +246,8 @@ struct Engine : fcd_ctx {
     bool profiling = false;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
     cudaEvent_t snap_ev = nullptr;
+    cudaStream_t beside = nullptr;  // see do_step
+    cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
     long host_kernels = 0;
     int reported_nonconv = 0;
     int copies = 1;  // plane sets per field: 1, or 1 + NT for the tangent context
@@ -281,10 +283,12 @@ struct Engine : fcd_ctx {
         if (h_snap) cudaFreeHost(h_snap);
         if (h_brk) cudaFreeHost(h_brk);
         if (h_trouble) cudaFreeHost(h_trouble);
-        if (cap) cudaStreamDestroy(cap);
+        for (auto t : {cap, beside})
+            if (t) cudaStreamDestroy(t);
         for (auto e : ev)
             if (e) cudaEventDestroy(e);
-        if (snap_ev) cudaEventDestroy(snap_ev);
+        for (auto e : {snap_ev, fork_ev, join_ev})
+            if (e) cudaEventDestroy(e);
     }
 
     bool magnetic() const { return D.H0 > 0.0; }
@@ -326,7 +330,7 @@ struct Engine : fcd_ctx {
         unst = &trouble->unst;
         CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
         for (auto &e : ev) CK(cudaEventCreate(&e));
-        CK(cudaEventCreateWithFlags(&snap_ev, cudaEventDisableTiming));
+        for (auto e : {&snap_ev, &fork_ev, &join_ev}) CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
         mg = mg_create<T>(prm.nx, prm.ny, pitch, k, psiA, psiB, ctl, alloc, release, user, err,
                           sizeof err, trouble, comp, nullptr, psiP);
         if (!mg) return FCD_ENOMEM;
@@ -552,11 +556,8 @@ struct Engine : fcd_ctx {
     // per step (steps back to back): 1600 x 200 49.4 -> 45.1 us, 2400 x 300 87.6 ->
     // 80.4 us, 900 x 150 open 46.9 -> 42.0 us, the same bits. While profiling the
     // collide-stream follows the IF node instead (no gate, no branch): an event
-    // between the two stages has no place beside the IF node, nor in its body.
-    // The one use it slows:
-    // many contexts stepped in turn on the legacy default stream, which orders
-    // itself against every graph's branches (4 contexts 28.0 -> 28.5 us per step, 24
-    // 64 -> 69, 96 131 -> 181; on an own stream 96 go from 65 to 60).
+    // between the two stages has no place beside the IF node, nor in its body. On
+    // the legacy default stream see do_step.
     fcd_status capture_solve_and_collide(int c, int sm, cudaStream_t s) {
         cudaStreamCaptureStatus cs;
         cudaGraph_t gcap;
@@ -667,9 +668,9 @@ struct Engine : fcd_ctx {
         return FCD_OK;
     }
 
-    // One step; sm != 0 also stores the macroscopic fields.
-    fcd_status one_step(int sm) {
-        cudaStream_t s = stream;
+    // One step on s; sm != 0 also stores the macroscopic fields.
+    fcd_status one_step(int sm) { return one_step(sm, stream); }
+    fcd_status one_step(int sm, cudaStream_t s) {
         if (use_graph) {
             if (!gexec[cur][sm]) {
                 fcd_status st = build_graph(cur, sm);
@@ -703,12 +704,38 @@ struct Engine : fcd_ctx {
         return FCD_OK;
     }
 
+    // The legacy default stream orders itself against the branches of every graph
+    // in the process, so that a branched step graph launched there costs more the
+    // more contexts there are (96 contexts in turn: 174 us per step, 129 without
+    // branches). Such graphs therefore run on streams of the context that keep
+    // that stream's order: one step on a blocking stream, which CUDA orders
+    // against it at no cost; several on a non-blocking one between two events,
+    // because many graphs in a row on a blocking stream cost about as much as on
+    // the legacy stream itself (96 contexts, 10 steps a call: 125 us, legacy 142, with
+    // events 56). us per step, contexts of 1600 x 200 in turn, unbranched -> branched
+    // on the legacy stream -> here: 1 context 56 -> 45 -> 45; 24 contexts, one step a
+    // call 82 -> 95 -> 25 (they overlap), 10 steps 81 -> 95 -> 47; 96 contexts
+    // 129 -> 174 -> 86 and 92 -> 142 -> 56.
     fcd_status do_step(long n) override {
         if (n < 0) return fail(FCD_EINVAL, "negative step count");
-        for (long i = 0; i < n; i++) {
-            const fcd_status st = one_step(i == n - 1 ? 1 : 0);
-            if (st != FCD_OK) return st;
+        const bool legacy = use_graph && turns() && (stream == nullptr || stream == cudaStreamLegacy);
+        const bool fork = legacy && n > 1;
+        cudaStream_t s = stream;
+        if (fork) {
+            s = cap;
+            CK(cudaEventRecord(fork_ev, stream));
+            CK(cudaStreamWaitEvent(s, fork_ev, 0));
+        } else if (legacy) {
+            if (!beside) CK(cudaStreamCreateWithFlags(&beside, cudaStreamDefault));
+            s = beside;
         }
+        fcd_status st = FCD_OK;
+        for (long i = 0; i < n && st == FCD_OK; i++) st = one_step(i == n - 1 ? 1 : 0, s);
+        if (fork) {
+            CK(cudaEventRecord(join_ev, s));
+            CK(cudaStreamWaitEvent(stream, join_ev, 0));
+        }
+        if (st != FCD_OK) return st;
         CK(cudaGetLastError());
         return FCD_OK;
     }
