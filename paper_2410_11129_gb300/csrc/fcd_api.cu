@@ -1873,6 +1873,12 @@ bool engine_view(fcd_ctx *c, EngineView *v) {
     return true;
 }
 
+bool engine_one_kernel(fcd_ctx *c) {
+    if (auto *e = dynamic_cast<Engine<float> *>(c)) return e->magnetic() && mg_one_kernel<float>(e->mg);
+    if (auto *d = dynamic_cast<Engine<double> *>(c)) return d->magnetic() && mg_one_kernel<double>(d->mg);
+    return false;
+}
+
 void engine_share(fcd_ctx *c, int share) {
     if (auto *e = dynamic_cast<Engine<float> *>(c)) mg_set_share<float>(e->mg, share);
     else if (auto *d = dynamic_cast<Engine<double> *>(c)) mg_set_share<double>(d->mg, share);

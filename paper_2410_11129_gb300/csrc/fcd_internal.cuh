@@ -517,6 +517,8 @@ struct EngineView {
 };
 // false (and v untouched) for any other context
 bool engine_view(fcd_ctx *c, EngineView *v);
+// whether the context's solves are one kernel each
+bool engine_one_kernel(fcd_ctx *c);
 // the context's solves run beside those of other contexts (1 / share of the SMs)
 void engine_share(fcd_ctx *c, int share);
 // the host-side record of a context after `steps` steps run by the batch
