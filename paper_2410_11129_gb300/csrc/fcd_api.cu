@@ -18,6 +18,7 @@
 #include <typeinfo>
 #include <vector>
 
+#include <cuda.h>
 #include <nvtx3/nvToolsExt.h>
 
 #include "fcd_adjoint.cuh"
@@ -859,27 +860,75 @@ struct Engine : fcd_ctx {
     }
 
     // Where the exchange kernels read or write directly: memory of the current
-    // device (nullptr too, which they skip). Anything else goes through a staging
-    // block: cudaMalloc and cudaFree of one, and the copy out of it, were most of
-    // an exchange with device memory (populations of 1600 x 200: 324 -> 75 us, of
-    // 9600 x 1200, 2.5 GB: 3.9 -> 1.7 ms, a conversion to FP32 included).
-    static bool on_device(const void *p) {
-        if (!p) return true;
+    // device (nullptr too, which they skip) that lies in one allocation. Anything
+    // else goes through a staging block: cudaMalloc and cudaFree of one, and the
+    // copy out of it, were most of an exchange with device memory (populations of
+    // 1600 x 200: 324 -> 75 us, of 9600 x 1200, 2.5 GB: 3.9 -> 1.7 ms, a conversion to
+    // FP32 included). A kernel does not notice the end of a buffer as that copy
+    // does, so a buffer that ends before its bytes do is refused here.
+    enum Reach { STAGED, DIRECT, SHORT };
+    static Reach reach(const void *p, size_t bytes) {
+        if (!p) return DIRECT;
         cudaPointerAttributes at;
         int dev = -1;
-        const bool ok = cudaPointerGetAttributes(&at, p) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
-                        at.type == cudaMemoryTypeDevice && at.device == dev &&
-                        reinterpret_cast<uintptr_t>(p) % alignof(double) == 0;
+        const bool here = cudaPointerGetAttributes(&at, p) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
+                          at.type == cudaMemoryTypeDevice && at.device == dev &&
+                          reinterpret_cast<uintptr_t>(p) % alignof(double) == 0;
         cudaGetLastError();  // clear the error of an unregistered pointer query
-        return ok;
+        if (!here) return STAGED;
+        const uintptr_t end = reinterpret_cast<uintptr_t>(p) + bytes;
+        uintptr_t q = reinterpret_cast<uintptr_t>(p);
+        if (!allocation_end(&q)) return STAGED;  // not known
+        if (q >= end) return DIRECT;
+        while (q < end)  // neighbouring allocations: one mapped piece by piece, or another's
+            if (!allocation_end(&q)) return SHORT;
+        return driver().mapped(p) ? DIRECT : STAGED;
     }
+    // The driver's records of an address.
+    struct Driver {
+        CUresult(CUDAAPI *range)(CUdeviceptr *, size_t *, CUdeviceptr) = nullptr;
+        CUresult(CUDAAPI *attribute)(void *, CUpointer_attribute, CUdeviceptr) = nullptr;
+        template <typename F>
+        static void get(const char *name, F *f) {
+            void *p = nullptr;
+            cudaDriverEntryPointQueryResult r;
+            if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &r) == cudaSuccess &&
+                r == cudaDriverEntryPointSuccess)
+                *f = reinterpret_cast<F>(p);
+        }
+        Driver() {
+            get("cuMemGetAddressRange", &range);
+            get("cuPointerGetAttribute", &attribute);
+        }
+        // memory of cuMemMap (torch's expandable segments: pieces of 20 MiB), not of cudaMalloc
+        bool mapped(const void *p) const {
+            int malloced = 1;
+            return attribute && attribute(&malloced, CU_POINTER_ATTRIBUTE_IS_LEGACY_CUDA_IPC_CAPABLE,
+                                          (CUdeviceptr)reinterpret_cast<uintptr_t>(p)) == CUDA_SUCCESS && !malloced;
+        }
+    };
+    static const Driver &driver() {
+        static const Driver d;
+        return d;
+    }
+    // *p := the end of the device allocation that it lies in; false: in none.
+    static bool allocation_end(uintptr_t *p) {
+        CUdeviceptr base = 0;
+        size_t size = 0;
+        if (!driver().range || driver().range(&base, &size, (CUdeviceptr)*p) != CUDA_SUCCESS) return false;
+        *p = (uintptr_t)base + size;
+        return true;
+    }
+    fcd_status fail_short() { return fail(FCD_ECUDA, "a device buffer ends before its values do"); }
 
     fcd_status field(int which, double *dst, size_t n) override {
         const size_t N = (size_t)prm.nx * prm.ny;
         if (!dst || n < N) return fail(FCD_EINVAL, "destination holds %zu of %zu values", n, N);
         if (which < FCD_FIELD_PHI1 || which > FCD_FIELD_PSI) return fail(FCD_EINVAL, "unknown field %d", which);
         cudaStream_t s = stream;
-        const bool direct = on_device(dst);
+        const Reach r = reach(dst, N * sizeof(double));
+        if (r == SHORT) return fail_short();
+        const bool direct = r == DIRECT;
         double *st = direct ? dst : staging(N);
         if (!st) return fail(FCD_ENOMEM, "staging allocation failed");
         fcd_status rc = FCD_OK;
@@ -911,7 +960,10 @@ struct Engine : fcd_ctx {
     fcd_status get_pops(double *fo, double *go, double *po) override {
         const size_t N = (size_t)prm.nx * prm.ny;
         cudaStream_t s = stream;
-        const bool direct = on_device(fo) && on_device(go) && on_device(po);
+        const Reach rf = reach(fo, 9 * N * sizeof(double)), rg = reach(go, 18 * N * sizeof(double)),
+                    rp = reach(po, N * sizeof(double));
+        if (rf == SHORT || rg == SHORT || rp == SHORT) return fail_short();
+        const bool direct = rf == DIRECT && rg == DIRECT && rp == DIRECT;
         double *st = nullptr, *df = fo, *dg = go, *dp = po;
         if (!direct) {
             st = staging(28 * N);
@@ -939,7 +991,10 @@ struct Engine : fcd_ctx {
         const size_t N = (size_t)prm.nx * prm.ny;
         if (st_ < 0) return fail(FCD_EINVAL, "negative step");
         cudaStream_t s = stream;
-        const bool direct = on_device(fi) && on_device(gi) && on_device(pi);
+        const Reach rf = reach(fi, 9 * N * sizeof(double)), rg = reach(gi, 18 * N * sizeof(double)),
+                    rp = reach(pi, N * sizeof(double));
+        if (rf == SHORT || rg == SHORT || rp == SHORT) return fail_short();
+        const bool direct = rf == DIRECT && rg == DIRECT && rp == DIRECT;
         double *st = nullptr;
         const double *sf = fi, *sg = gi, *sp = pi;
         cudaError_t e = cudaSuccess;
