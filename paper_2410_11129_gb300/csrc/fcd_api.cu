@@ -454,7 +454,7 @@ struct Engine : fcd_ctx {
             }
         }
         PhaseCtl pc{ctl, magnetic() ? 1 : 0, prm.mag_tol * D.H0, prm.mag_max_iter, d_step,
-                    magnetic() ? 1 : 0, psiA, psiB, psiP, comp};
+                    magnetic() ? 1 : 0, psiA, psiB, psiP, comp, stop_factor(prm.mag_tol, STOP_GUESSED)};
         launch_phase<T>(mode, P, g[c], phi1, phi2, k, pc, s);
         return FCD_OK;
     }
@@ -761,7 +761,7 @@ struct Engine : fcd_ctx {
             return FCD_OK;
         }
         launch_phase<T>(mode, P, g[cur], phi1, phi2, k,
-                        PhaseCtl{ctl, 1, tol * D.H0, max_iter, nullptr, 0, nullptr, nullptr, nullptr}, s);
+                        PhaseCtl{ctl, 1, tol * D.H0, max_iter, nullptr, 0, nullptr, nullptr, nullptr, 0, stop_factor(tol, STOP_ALONE)}, s);
         host_kernels += turns() ? 1 : pre_kernels();  // the opening sweep counts as a cycle
         CK(cudaGetLastError());
         fcd_status st = host_mg_loop(s);

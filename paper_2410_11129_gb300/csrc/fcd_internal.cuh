@@ -171,6 +171,7 @@ struct MgCtl {
     // solves that run as one cooperative kernel (fcd_mg_solve.cuh); reset with the solve
     unsigned long long norm_slot[4];  // max |r| of the last heads (bits of doubles >= 0)
     unsigned bar;                     // arrivals at the kernel's grid barriers
+    double stop;                      // max |r| that ends the solve in FP64 (tolH0 still decides convergence)
     double scale;                     // size of the right-hand side: H0, or max |rhs| where it is explicit
     int stuck;                        // this block's solve was given up (Trouble::stuck)
 };
@@ -186,8 +187,32 @@ constexpr unsigned BARRIER_POLLS = 1u << 24;  // seconds
 // Level-0 buffer 0, 1 or 2 of a, b, c.
 template <typename T>
 __host__ __device__ __forceinline__ T *psi_buffer(int i, T *a, T *b, T *c) { return i == 0 ? a : (i == 1 ? b : c); }
+// An FP64 solve goes on below its tolerance by this factor (at most to where its
+// residual is rounding). When the residual of its FP32-corrected cycles meets the
+// tolerance it is smooth, and a smooth residual stands for a larger error of psi'
+// than the rough one that cycles of FP64 sweeps, three to a digit, left at the same
+// tolerance: the more cycles, the larger the ratio, about 100 at 1e-10 from nothing,
+// 5 to 20 from a step's guess, 1 to 3 at 1e-5. Chosen so that the error against
+// 64-bit references is no larger than with FP64 sweeps (three seeds of the listed
+// FP64 cases, 16 drawn ones). Tolerance 1e-10, FP64 sweeps -> stopping at the
+// tolerance -> here, error and us per pass:
+//   populations after 16 steps, 800 x 100: 1.5e-15 -> 8e-15 -> 1e-15, 9300 -> 4250 -> 5010;
+//   200 x 40: 7e-15 -> 4e-14 -> 3e-15, 6740 -> 2320 -> 2760;
+//   psi' from nothing, 800 x 100: 3.6e-13 -> 3.1e-11 -> 8e-14, 2660 -> 777 -> 920;
+//   510 x 70: 2e-11 -> 5e-10 -> 1.4e-12;
+//   tangent derivatives, 800 x 100: 3e-12 -> 5e-11 -> 6e-13, 16400 -> 7150 -> 8020;
+//   gradient of the adjoint: 9e-14 -> 1.3e-12 -> 4e-14, 75500 -> 39100 -> 43700.
+// At 1e-3 the factor 1/2 keeps a guess that just passes from drifting to where the
+// whole cycle count is due at once (4800 x 600: 4173 us per step at 1, 3636 here, FP64
+// sweeps 3685; psi' 1.5e-2, 2.6e-3 and 1.1e-3 off).
+constexpr double STOP_GUESSED = 1.0 / 32;  // least: from a guess extrapolated in time (steps, tangents, adjoints)
+constexpr double STOP_ALONE = 1.0 / 256;   // least: a solve on its own, from any guess
+__host__ __device__ inline double stop_factor(double tol, double least) {
+    const double s = sqrt(1e5 * tol);
+    return s < least ? least : (s < 0.5 ? s : 0.5);
+}
 // start of a potential solve (one thread)
-__device__ __forceinline__ void mg_reset_ctl(MgCtl *c, double tolH0, int max_iter, double scale) {
+__device__ __forceinline__ void mg_reset_ctl(MgCtl *c, double tolH0, int max_iter, double scale, double stop) {
     c->norm_bits = 0ull;
     c->iter = 0;
     c->done = 0;
@@ -203,6 +228,7 @@ __device__ __forceinline__ void mg_reset_ctl(MgCtl *c, double tolH0, int max_ite
     for (int q = 0; q < 4; q++) c->norm_slot[q] = 0ull;
     c->bar = 0u;
     c->scale = scale;
+    c->stop = stop * tolH0;
 }
 
 // What the phase kernel does besides Eq. 32: reset the solve's control block
@@ -219,6 +245,7 @@ struct PhaseCtl {
     int extrap;
     void *psiA, *psiB, *psi_prev;
     int comp;  // FP32: psi' is the hi + lo pair (Level::comp)
+    double stop = 1.0;  // stop_factor
 };
 
 struct ObsOut {

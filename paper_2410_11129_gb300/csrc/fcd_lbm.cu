@@ -34,7 +34,7 @@ __device__ __forceinline__ void phase_tile(const Phys<T> &P, const void *gv, T *
     using S = typename StoreT<MODE>::type;
     if (pc.ctl && lead && threadIdx.x == 0 && threadIdx.y == 0) {
         MgCtl *c = pc.ctl;
-        if (pc.reset) mg_reset_ctl(c, pc.tolH0, pc.max_iter, c->H0);  // start of a potential solve
+        if (pc.reset) mg_reset_ctl(c, pc.tolH0, pc.max_iter, c->H0, pc.stop);  // start of a potential solve
         if (pc.step) {
             c->step_cur = *pc.step;
             *pc.step += 1;

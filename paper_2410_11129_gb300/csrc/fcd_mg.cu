@@ -1066,7 +1066,7 @@ __device__ __forceinline__ void phase_open_tile(const OpenArgs &A, int x0, int y
     const unsigned gx = (nx + OX - 1) / OX, gy = (ny + OY - 1) / OY;
     if (tid == 0 && tile_done(ctl, L0.grp, (y0 / OY) * gx + x0 / OX, gx * gy, 0ull)) {
         // the start of the solve and of the step, and the end of its opening cycle
-        mg_reset_ctl(ctl, A.tolH0, A.max_iter, ctl->H0);
+        mg_reset_ctl(ctl, A.tolH0, A.max_iter, ctl->H0, 1.0);
         if (A.max_iter > 0) {
             ctl->iter = 1;
             ctl->smooth_cycles++;
@@ -1751,7 +1751,7 @@ __global__ void mg_reset_kernel(MgCtl *c, const unsigned long long *scale_bits, 
                                 int max_iter) {
     // a zero right-hand side: the solution is zero and the guess is kept
     const double scale = __longlong_as_double((long long)*scale_bits);
-    mg_reset_ctl(c, scale > 0.0 ? tol * scale : INFINITY, max_iter, scale);
+    mg_reset_ctl(c, scale > 0.0 ? tol * scale : INFINITY, max_iter, scale, stop_factor(tol, STOP_GUESSED));
 }
 
 void mg_reset_scaled(MgCtl *ctl, const unsigned long long *scale_bits, double tol, int max_iter,

@@ -818,11 +818,13 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
     }
     __syncthreads();
     const int gx = (A.L0.nx + SX - 1) / SX, tiles = gx * ((A.L0.ny + SY - 1) / SY);
-    const double tol = ctl->tolH0;
+    const double tol = ctl->tolH0, stop = COMP ? tol : ctl->stop;
     const Unit<T> unit(ctl->scale);
     const int max_iter = ctl->max_iter;
     int cur = ctl->cur, iter = 0, heads = 0, twogrid = 0, vcycles = 0;
     unsigned arrivals = 0;
+    bool closing = false;          // the tolerance is met
+    double res = 0.0, last = 0.0;  // max |r| of psi(cur); of the closing head before
     const TC over = L[1].ny != A.L0.ny && A.L0.ny % 2 == 0 ? OVER : TC(1);
     auto psi = [&](int c) { return c ? A.L0.r : A.L0.e; };
     // tile t is worker (t / gridDim) % workers of block t % gridDim
@@ -852,7 +854,18 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
         }
         __syncthreads();
         heads++;
-        if (norm <= tol || iter >= max_iter || !(norm < INFINITY)) break;
+        res = norm;
+        if (closing && !(res < last)) {  // only rounding was left: the iterate before is the better one
+            cur ^= 1;
+            res = last;
+            break;
+        }
+        if (res <= stop || iter >= max_iter || !(res < INFINITY)) break;
+        if (res <= tol) {
+            if (closing && res > 0.5 * last) break;
+            closing = true;
+            last = res;
+        }
         if (twogrid < 2) {
             twogrid++;
             fv_phase<2>(fv, L[1], L[1], NU_TWOGRID);
@@ -883,9 +896,9 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
         ctl->mode = 3;
         ctl->iter = iter;
         ctl->cur = cur;
-        ctl->converged = norm <= tol;
-        if (!(norm <= tol)) ctl->nonconv_count++;
-        ctl->last_resid = ctl->H0 > 0.0 ? norm / ctl->H0 : 0.0;
+        ctl->converged = res <= tol;
+        if (!(res <= tol)) ctl->nonconv_count++;
+        ctl->last_resid = ctl->H0 > 0.0 ? res / ctl->H0 : 0.0;
         ctl->last_iters = iter;
         ctl->cycles_launched += heads;
         ctl->total_cycles += vcycles;
