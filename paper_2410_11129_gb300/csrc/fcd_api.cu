@@ -207,9 +207,10 @@ struct SnapHeader {
     int nx, ny, precision, pitch;
     long long step;
     unsigned long long brk;
-    int cur, pad;  // which level-0 potential buffer is current; 0
+    int cur, back;  // which level-0 potential buffer is current, 2 - the previous step's (MgCtl)
 };
-static const unsigned SNAP_VERSION = 4;
+// 5: the three buffers may stand in any order; 4: the third is the previous step's (back 0)
+static const unsigned SNAP_VERSION = 5, SNAP_VERSION_FIXED = 4;
 static const unsigned SNAP_MAGIC = 0x46434453u;  // "FCDS"
 
 template <typename T>
@@ -246,7 +247,6 @@ struct Engine : fcd_ctx {
     bool use_graph = true;
     bool profiling = false;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
-    cudaEvent_t snap_ev = nullptr;
     cudaStream_t beside = nullptr;  // see do_step
     cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
     long host_kernels = 0;
@@ -288,7 +288,7 @@ struct Engine : fcd_ctx {
             if (t) cudaStreamDestroy(t);
         for (auto e : ev)
             if (e) cudaEventDestroy(e);
-        for (auto e : {snap_ev, fork_ev, join_ev})
+        for (auto e : {fork_ev, join_ev})
             if (e) cudaEventDestroy(e);
     }
 
@@ -331,7 +331,7 @@ struct Engine : fcd_ctx {
         unst = &trouble->unst;
         CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
         for (auto &e : ev) CK(cudaEventCreate(&e));
-        for (auto e : {&snap_ev, &fork_ev, &join_ev}) CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+        for (auto e : {&fork_ev, &join_ev}) CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
         mg = mg_create<T>(prm.nx, prm.ny, pitch, k, psiA, psiB, ctl, alloc, release, user, err,
                           sizeof err, trouble, comp, nullptr, psiP);
         if (!mg) return FCD_ENOMEM;
@@ -1030,11 +1030,10 @@ struct Engine : fcd_ctx {
 
     // Snapshot: header, the 27 stored population planes of the current buffer,
     // both level-0 potential buffers and the previous potential. Both potential
-    // buffers travel, with the device's current-buffer index, so neither call
-    // needs to read the control block on the host: each is one stream of
-    // asynchronous copies and a single synchronisation. Where the three buffers
-    // take turns they are stored by role (current, idle, previous step's): get_state
-    // reads the control block first and waits for it while the populations travel.
+    // buffers travel, with the device's indices of the current and the previous one,
+    // so neither call needs to read the control block on the host: each is one stream
+    // of asynchronous copies and a single synchronisation. A context whose buffers do
+    // not take turns puts those of one whose do in its own order.
     size_t state_bytes() const override {
         return sizeof(SnapHeader) + 27 * (size_t)ps * sizeof(S) + 3 * psi_bytes();
     }
@@ -1043,16 +1042,11 @@ struct Engine : fcd_ctx {
         if (!dst || bytes < state_bytes()) return fail(FCD_EINVAL, "snapshot buffer too small");
         cudaStream_t s = stream;
         char *d = static_cast<char *>(dst);
-        T *bufs[3] = {psiA, psiB, psiP};
         CK(cudaStreamSynchronize(s));  // the staging header may still be in flight
-        if (turns()) {
-            CK(cudaMemcpyAsync(h_ctl, ctl, sizeof(MgCtl), cudaMemcpyDeviceToHost, s));
-            CK(cudaEventRecord(snap_ev, s));
-        }
         SnapHeader &h = *h_snap;
         std::memset(&h, 0, sizeof h);
         h.magic = SNAP_MAGIC;
-        h.version = SNAP_VERSION;
+        h.version = turns() ? SNAP_VERSION : SNAP_VERSION_FIXED;
         h.nx = prm.nx;
         h.ny = prm.ny;
         h.precision = prm.precision;
@@ -1061,21 +1055,15 @@ struct Engine : fcd_ctx {
         CK(cudaMemcpyAsync(d, &h, sizeof h, cudaMemcpyDefault, s));
         CK(cudaMemcpyAsync(d + offsetof(SnapHeader, brk), brk, sizeof(unsigned long long),
                            cudaMemcpyDefault, s));
-        if (!turns())
-            CK(cudaMemcpyAsync(d + offsetof(SnapHeader, cur), &ctl->cur, sizeof(int), cudaMemcpyDefault, s));
+        static_assert(offsetof(MgCtl, back) == offsetof(MgCtl, cur) + sizeof(int) &&
+                      offsetof(SnapHeader, back) == offsetof(SnapHeader, cur) + sizeof(int), "cur and back in one copy");
+        CK(cudaMemcpyAsync(d + offsetof(SnapHeader, cur), &ctl->cur, 2 * sizeof(int), cudaMemcpyDefault, s));
         size_t off = sizeof h;
         CK(cudaMemcpyAsync(d + off, f[cur], 9 * ps * sizeof(S), cudaMemcpyDefault, s));
         off += 9 * ps * sizeof(S);
         CK(cudaMemcpyAsync(d + off, g[cur], 18 * ps * sizeof(S), cudaMemcpyDefault, s));
         off += 18 * ps * sizeof(S);
-        if (turns()) {
-            CK(cudaEventSynchronize(snap_ev));
-            const int now = h_ctl->cur, prev = 2 - h_ctl->back;
-            bufs[0] = psi_buffer(now, psiA, psiB, psiP);
-            bufs[1] = psi_buffer(3 - now - prev, psiA, psiB, psiP);
-            bufs[2] = psi_buffer(prev, psiA, psiB, psiP);
-        }
-        for (T *q : bufs) {
+        for (T *q : {psiA, psiB, psiP}) {
             CK(cudaMemcpyAsync(d + off, q, psi_bytes(), cudaMemcpyDefault, s));
             off += psi_bytes();
         }
@@ -1100,8 +1088,11 @@ struct Engine : fcd_ctx {
             CK(cudaMemcpyAsync(&h, src, sizeof h, cudaMemcpyDefault, s));
             CK(cudaStreamSynchronize(s));
         }
-        if (h.magic != SNAP_MAGIC || h.version != SNAP_VERSION || h.nx != prm.nx || h.ny != prm.ny ||
-            h.precision != prm.precision || h.pitch != pitch || (h.cur != 0 && h.cur != 1))
+        if (h.version == SNAP_VERSION_FIXED) h.back = 0;
+        const int prev = 2 - h.back;
+        if (h.magic != SNAP_MAGIC || (h.version != SNAP_VERSION && h.version != SNAP_VERSION_FIXED) ||
+            h.nx != prm.nx || h.ny != prm.ny || h.precision != prm.precision || h.pitch != pitch || h.cur < 0 ||
+            h.cur > 2 || prev < 0 || prev > 2 || h.cur == prev)
             return fail(FCD_ESTATE, "snapshot does not match this context");
         const char *p = static_cast<const char *>(src);
         size_t off = sizeof h;
@@ -1109,12 +1100,17 @@ struct Engine : fcd_ctx {
         off += 9 * ps * sizeof(S);
         CK(cudaMemcpyAsync(g[cur], p + off, 18 * ps * sizeof(S), cudaMemcpyDefault, s));
         off += 18 * ps * sizeof(S);
-        for (T *q : {psiA, psiB, psiP}) {
+        T *bufs[3] = {psiA, psiB, psiP};
+        if (h.back != 0 && !turns()) {
+            bufs[h.cur] = psiA;
+            bufs[3 - h.cur - prev] = psiB;
+            bufs[prev] = psiP;
+            h.cur = h.back = 0;
+        }
+        for (T *q : bufs) {
             CK(cudaMemcpyAsync(q, p + off, psi_bytes(), cudaMemcpyDefault, s));
             off += psi_bytes();
         }
-        static_assert(offsetof(MgCtl, back) == offsetof(MgCtl, cur) + sizeof(int), "cur and back in one copy");
-        h.pad = 0;  // back: the third buffer is the previous step's
         CK(cudaMemcpyAsync(&ctl->cur, &h.cur, 2 * sizeof(int), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(brk, &h.brk, sizeof(unsigned long long), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(d_step, &h.step, sizeof(long long), cudaMemcpyHostToDevice, s));
