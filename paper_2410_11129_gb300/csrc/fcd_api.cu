@@ -231,8 +231,8 @@ struct Engine : fcd_ctx {
     MgCtl *ctl = nullptr;
     MgHost<T> *mg = nullptr;
     unsigned long long *brk = nullptr;
-    Trouble *trouble = nullptr;          // what went wrong so far
-    unsigned long long *unst = nullptr;  // &trouble->unst
+    unsigned long long *unst = nullptr;  // first step with a non-finite collision (~0: none)
+    Bound *bound = nullptr;
     long long *d_step = nullptr;
     double *obs_scratch = nullptr;
     ObsOut *obs_out = nullptr;
@@ -240,7 +240,8 @@ struct Engine : fcd_ctx {
     ObsPack *h_obs = nullptr;  // pinned; the last kernel of an observation writes it
     SnapHeader *h_snap = nullptr;  // pinned staging of snapshot headers
     unsigned long long *h_brk = nullptr;
-    Trouble *h_trouble = nullptr;
+    unsigned long long *h_unst = nullptr;
+    Bound *h_bound = nullptr;  // pinned; its stuck is the device's `told`
     cudaStream_t cap = nullptr;
     cudaGraph_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
     cudaGraphExec_t gexec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
@@ -283,7 +284,8 @@ struct Engine : fcd_ctx {
         if (h_obs) cudaFreeHost(h_obs);
         if (h_snap) cudaFreeHost(h_snap);
         if (h_brk) cudaFreeHost(h_brk);
-        if (h_trouble) cudaFreeHost(h_trouble);
+        if (h_unst) cudaFreeHost(h_unst);
+        if (h_bound) cudaFreeHost(h_bound);
         for (auto t : {cap, beside})
             if (t) cudaStreamDestroy(t);
         for (auto e : ev)
@@ -315,25 +317,26 @@ struct Engine : fcd_ctx {
         macro = dalloc(3 * ps * sizeof(T));
         ctl = reinterpret_cast<MgCtl *>(dalloc(sizeof(MgCtl)));
         brk = reinterpret_cast<unsigned long long *>(dalloc(sizeof(unsigned long long)));
-        trouble = reinterpret_cast<Trouble *>(dalloc(sizeof(Trouble)));
+        unst = reinterpret_cast<unsigned long long *>(dalloc(sizeof(unsigned long long)));
+        bound = reinterpret_cast<Bound *>(dalloc(sizeof(Bound)));
         d_step = reinterpret_cast<long long *>(dalloc(sizeof(long long)));
         obs_scratch = reinterpret_cast<double *>(dalloc(observe_scratch_doubles(prm.nx, prm.ny) * sizeof(double)));
         obs_out = reinterpret_cast<ObsOut *>(dalloc(sizeof(ObsOut)));
         for (void *p : {f[0], f[1], g[0], g[1], (void *)phi1, (void *)phi2, (void *)k, (void *)psiA,
-                        (void *)psiB, (void *)psiP, (void *)macro, (void *)ctl, (void *)brk, (void *)trouble, (void *)d_step,
+                        (void *)psiB, (void *)psiP, (void *)macro, (void *)ctl, (void *)brk, (void *)unst, (void *)d_step, (void *)bound,
                         (void *)obs_scratch, (void *)obs_out})
             if (!p) return fail(FCD_ENOMEM, "device allocation failed");
         CK(cudaMallocHost(&h_ctl, sizeof(MgCtl)));
         CK(cudaMallocHost(&h_obs, sizeof(ObsPack)));
         CK(cudaMallocHost(&h_snap, sizeof(SnapHeader)));
         CK(cudaMallocHost(&h_brk, sizeof(unsigned long long)));
-        CK(cudaMallocHost(&h_trouble, sizeof(Trouble)));
-        unst = &trouble->unst;
+        CK(cudaMallocHost(&h_unst, sizeof(unsigned long long)));
+        CK(cudaMallocHost(&h_bound, sizeof(Bound)));
         CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
         for (auto &e : ev) CK(cudaEventCreate(&e));
         for (auto e : {&fork_ev, &join_ev}) CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
         mg = mg_create<T>(prm.nx, prm.ny, pitch, k, psiA, psiB, ctl, alloc, release, user, err,
-                          sizeof err, trouble, comp, nullptr, psiP);
+                          sizeof err, bound, comp, nullptr, psiP);
         if (!mg) return FCD_ENOMEM;
         cudaStream_t s = stream;
         CK(cudaMemsetAsync(ctl, 0, sizeof(MgCtl), s));
@@ -341,8 +344,9 @@ struct Engine : fcd_ctx {
         CK(cudaMemsetAsync(psiB, 0, psi_bytes(), s));
         CK(cudaMemsetAsync(psiP, 0, psi_bytes(), s));
         CK(cudaMemsetAsync(brk, 0xff, sizeof(unsigned long long), s));
-        *h_trouble = Trouble{~0ull, 0, BARRIER_POLLS};
-        CK(cudaMemcpyAsync(trouble, h_trouble, sizeof(Trouble), cudaMemcpyHostToDevice, s));
+        CK(cudaMemsetAsync(unst, 0xff, sizeof(unsigned long long), s));
+        *h_bound = Bound{0, BARRIER_POLLS, &h_bound->stuck};
+        CK(cudaMemcpyAsync(bound, h_bound, sizeof(Bound), cudaMemcpyHostToDevice, s));
         CK(cudaMemsetAsync(d_step, 0, sizeof(long long), s));
         // padding columns of every plane stay zero
         for (int b = 0; b < 2; b++) {
@@ -504,7 +508,7 @@ struct Engine : fcd_ctx {
             CK(mg_solve<T>(m, P.H0c, P.H0s, s));
             CK(cudaMemcpyAsync(h_ctl, c, sizeof(MgCtl), cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
-            return h_ctl->stuck ? fail_stuck() : FCD_OK;
+            return stuck() ? fail_stuck() : FCD_OK;
         }
         if constexpr (sizeof(T) == 4) {
             if (!opened) mg_presmooth(m, P.H0c, P.H0s, s);
@@ -778,13 +782,13 @@ struct Engine : fcd_ctx {
 
     fcd_status observe(fcd_obs *o) override {
         cudaStream_t s = stream;
-        launch_observe<T>(mode, P, g[cur], obs_scratch, obs_out, s, prm.open_x, ObsTail{h_obs, brk, trouble, ctl});
+        launch_observe<T>(mode, P, g[cur], obs_scratch, obs_out, s, prm.open_x, ObsTail{h_obs, brk, unst, ctl});
         host_kernels += 3;
         CK(cudaGetLastError());
         CK(cudaStreamSynchronize(s));
         const ObsOut &r = h_obs->o;
         *h_brk = h_obs->brk;
-        *h_trouble = h_obs->trouble;
+        *h_unst = h_obs->unst;
         *h_ctl = h_obs->ctl;
         std::memset(o, 0, sizeof *o);
         o->step = step;
@@ -826,30 +830,30 @@ struct Engine : fcd_ctx {
     }
 
     // FCD_ECUDA once a solve was given up at a grid barrier, FCD_EUNSTABLE once a
-    // collision produced a non-finite velocity or pressure; h_trouble must have
-    // been copied in the caller's synchronised batch.
+    // collision produced a non-finite velocity or pressure; h_unst must have been
+    // copied in the caller's synchronised batch.
+    bool stuck() const { return *(volatile int *)&h_bound->stuck != 0; }
     fcd_status fail_stuck() { return fail(FCD_ECUDA, "a grid barrier of a potential solve timed out"); }
     fcd_status trouble_status() {
-        if (h_trouble->stuck) return fail_stuck();
-        if (h_trouble->unst == ~0ull) return FCD_OK;
+        if (stuck()) return fail_stuck();
+        if (*h_unst == ~0ull) return FCD_OK;
         return fail(FCD_EUNSTABLE, "non-finite velocity or pressure, first in step %llu (now at step %ld)",
-                    h_trouble->unst, step);
+                    *h_unst, step);
     }
     // For tests of the bounded wait: later solves give up at a barrier after so
     // many polls (0: the default).
     fcd_status set_barrier_polls(unsigned polls) override {
         const unsigned v = polls ? polls : BARRIER_POLLS;
         CK(cudaDeviceSynchronize());  // a batch runs its instances' solves on other streams
-        CK(cudaMemcpy(&trouble->polls, &v, sizeof v, cudaMemcpyHostToDevice));
+        CK(cudaMemcpy(&bound->polls, &v, sizeof v, cudaMemcpyHostToDevice));
         return FCD_OK;
     }
-    // The record of a context that starts from a new state.
-    fcd_status clear_trouble(cudaStream_t s) {
-        CK(cudaMemsetAsync(unst, 0xff, sizeof(unsigned long long), s));
-        if (magnetic() && mg_one_kernel<T>(mg)) {
-            CK(cudaMemsetAsync(&trouble->stuck, 0, sizeof(int), s));
-            CK(cudaMemsetAsync(&ctl->stuck, 0, sizeof(int), s));
-        }
+    // Solves run again once a new state is set (s has been synchronised).
+    fcd_status unstick(cudaStream_t s) {
+        if (!stuck()) return FCD_OK;
+        CK(cudaMemsetAsync(&bound->stuck, 0, sizeof(int), s));
+        CK(cudaStreamSynchronize(s));
+        h_bound->stuck = 0;
         return FCD_OK;
     }
 
@@ -949,7 +953,7 @@ struct Engine : fcd_ctx {
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess && !direct) e = cudaMemcpyAsync(dst, st, N * sizeof(double), cudaMemcpyDefault, s);
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(h_trouble, trouble, sizeof(Trouble), cudaMemcpyDeviceToHost, s);
+            e = cudaMemcpyAsync(h_unst, unst, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) rc = fail(FCD_ECUDA, "get_field: %s", cudaGetErrorString(e));
         if (!direct) cudaFree(st);
@@ -972,7 +976,7 @@ struct Engine : fcd_ctx {
             dg = st + 9 * N;
             dp = st + 27 * N;
         }
-        launch_export<T>(mode, P, f[cur], g[cur], df, dg, s, trouble, h_trouble);
+        launch_export<T>(mode, P, f[cur], g[cur], df, dg, s, unst, h_unst);
         if (dp) launch_psi_to_f64<T>(ctl, psiA, psiB, psiP, prm.nx, prm.ny, pitch, dp, s);
         host_kernels += dp ? 2 : 1;
         cudaError_t e = cudaGetLastError();
@@ -1018,14 +1022,14 @@ struct Engine : fcd_ctx {
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = cudaMemsetAsync(brk, 0xff, sizeof(unsigned long long), s);
-        if (e == cudaSuccess && clear_trouble(s) != FCD_OK) e = cudaErrorUnknown;
+        if (e == cudaSuccess) e = cudaMemsetAsync(unst, 0xff, sizeof(unsigned long long), s);
         long long s64 = st_;
         if (e == cudaSuccess) e = cudaMemcpyAsync(d_step, &s64, sizeof(long long), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (st) cudaFree(st);
         if (e != cudaSuccess) return fail(FCD_ECUDA, "set_populations: %s", cudaGetErrorString(e));
         step = st_;
-        return FCD_OK;
+        return unstick(s);
     }
 
     // Snapshot: header, the 27 stored population planes of the current buffer,
@@ -1067,10 +1071,8 @@ struct Engine : fcd_ctx {
             CK(cudaMemcpyAsync(d + off, q, psi_bytes(), cudaMemcpyDefault, s));
             off += psi_bytes();
         }
-        const bool one = magnetic() && mg_one_kernel<T>(mg);
-        if (one) CK(cudaMemcpyAsync(h_trouble, trouble, sizeof(Trouble), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        return one && h_trouble->stuck ? fail_stuck() : FCD_OK;
+        return stuck() ? fail_stuck() : FCD_OK;
     }
 
     fcd_status set_state(const void *src, size_t bytes) override {
@@ -1114,11 +1116,10 @@ struct Engine : fcd_ctx {
         CK(cudaMemcpyAsync(&ctl->cur, &h.cur, 2 * sizeof(int), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(brk, &h.brk, sizeof(unsigned long long), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(d_step, &h.step, sizeof(long long), cudaMemcpyHostToDevice, s));
-        const fcd_status ct = clear_trouble(s);
-        if (ct != FCD_OK) return ct;
+        CK(cudaMemsetAsync(unst, 0xff, sizeof(unsigned long long), s));
         CK(cudaStreamSynchronize(s));
         step = (long)h.step;
-        return FCD_OK;
+        return unstick(s);
     }
 
     fcd_status set_profiling(int on) override {
@@ -1302,7 +1303,7 @@ struct TangentEngine : Engine<double> {
             // every tangent solve of a step has the primal solve's k, and the
             // primal solve forms the lattice coefficients first: share them
             mgt[c] = mg_create<double>(prm.nx, prm.ny, pitch, k, tA[c], tB[c], ctlt[c], alloc,
-                                       release, user, err, sizeof err, trouble, 0, mg);
+                                       release, user, err, sizeof err, bound, 0, mg);
             if (!mgt[c]) return FCD_ENOMEM;
             mg_set_rhs<double>(mgt[c], rhst[c]);
             mg_set_share<double>(mgt[c], NT);  // the NT solves of a step run side by side
@@ -1436,7 +1437,6 @@ struct TangentEngine : Engine<double> {
         if (st != FCD_OK && st != FCD_ENOCONV) return st;
         cudaStream_t s = stream;
         TanCtls ctls;
-        ctls.trouble = trouble;
         for (int c = 0; c < NT; c++) ctls.c[c] = mgt[c] ? ctlt[c] : nullptr;
         launch_tangent_obs(P, static_cast<const double *>(g[cur]), obs_out, tobs, tan_out, ctls, s);
         host_kernels += 2;
@@ -1456,7 +1456,7 @@ struct TangentEngine : Engine<double> {
             o->dlx_o[c] = h_tan->dlx[c];
             o->dly_o[c] = h_tan->dly[c];
         }
-        if (h_tan->stuck) return fail_stuck();
+        if (stuck()) return fail_stuck();
         if (nonconv > reported_tangent_nonconv) {
             reported_tangent_nonconv = nonconv;
             return fail(FCD_ENOCONV, "a tangent potential solve stopped at the cycle cap");
@@ -1762,7 +1762,7 @@ struct AdjointEngine : Engine<double> {
         cudaStream_t s = stream;
         if (!mga && magnetic()) {
             mga = mg_create<double>(prm.nx, prm.ny, pitch, k, lamA, lamB, ctla, alloc, release, user, err,
-                                    sizeof err, trouble);
+                                    sizeof err, bound);
             if (!mga) return FCD_ENOMEM;
             mg_set_rhs<double>(mga, rhs);
         }
@@ -1871,8 +1871,7 @@ struct AdjointEngine : Engine<double> {
             CK(cudaMemcpy(h_ctl, ctla, sizeof(MgCtl), cudaMemcpyDeviceToHost));
             o->solve_cycles = h_ctl->total_cycles + h_ctl->twogrid_cycles + h_ctl->smooth_cycles;
             o->capped_solves = h_ctl->nonconv_count;  // the control block is cleared per sweep
-            CK(cudaMemcpy(h_trouble, trouble, sizeof(Trouble), cudaMemcpyDeviceToHost));
-            if (h_trouble->stuck) return fail_stuck();
+            if (stuck()) return fail_stuck();
             if (o->capped_solves > 0)
                 return fail(FCD_ENOCONV, "%ld adjoint potential solves stopped at the cycle cap",
                             o->capped_solves);

@@ -173,15 +173,13 @@ struct MgCtl {
     unsigned bar;                     // arrivals at the kernel's grid barriers
     double stop;                      // max |r| that ends the solve in FP64 (tolH0 still decides convergence)
     double scale;                     // size of the right-hand side: H0, or max |rhs| where it is explicit
-    int stuck;                        // this block's solve was given up (Trouble::stuck)
 };
 
-// What went wrong in a context, one record for all its solves and steps: every
-// call that delivers results reads it.
-struct Trouble {
-    unsigned long long unst;  // first step with a non-finite collision (~0: none)
-    int stuck;                // a grid barrier timed out: no solve runs until a new state is set
-    unsigned polls;           // polls after which a grid barrier gives up
+// The bounded wait of a context's one-kernel solves, one record for all of them.
+struct Bound {
+    int stuck;       // a grid barrier timed out: no solve runs until a new state is set
+    unsigned polls;  // polls after which a grid barrier gives up
+    int *told;       // the same as stuck in pinned host memory, for every call that delivers results
 };
 constexpr unsigned BARRIER_POLLS = 1u << 24;  // seconds
 // Level-0 buffer 0, 1 or 2 of a, b, c.
@@ -261,14 +259,12 @@ struct ObsOut {
 // block of pinned memory; tail.pack == nullptr: nothing is gathered.
 struct ObsPack {
     ObsOut o;
-    unsigned long long brk;
-    Trouble trouble;
+    unsigned long long brk, unst;
     MgCtl ctl;
 };
 struct ObsTail {
     ObsPack *pack = nullptr;
-    const unsigned long long *brk = nullptr;
-    const Trouble *trouble = nullptr;
+    const unsigned long long *brk = nullptr, *unst = nullptr;
     const MgCtl *ctl = nullptr;
 };
 
@@ -277,11 +273,9 @@ struct TanOut {
     double T_o, overlap, lx, ly;
     double dT_o[NT], doverlap[NT], dlx[NT], dly[NT];
     int nonconv;  // capped tangent solves so far, all directions
-    int stuck;    // a solve was given up
 };
 struct TanCtls {
     const MgCtl *c[NT];  // nullptr: that direction has not been solved
-    const Trouble *trouble;
 };
 
 }  // namespace fcd
@@ -353,11 +347,11 @@ template <typename T>
 void launch_init(int mode, const Phys<T> &P, double u_max, double r1, double r2, double xc,
                  double yc, double xi, void *f, void *g, T *macro, cudaStream_t s);
 // Populations (fo 9 planes, go 18; nullptr: skipped) in the FP64 exchange
-// layout; trouble: the context's record, copied to *trouble_out (pinned host memory).
+// layout; unst: the instability record, copied to *unst_out (pinned host memory).
 template <typename T>
 void launch_export(int mode, const Phys<T> &P, const void *f, const void *g, double *fo,
-                   double *go, cudaStream_t s, const Trouble *trouble = nullptr,
-                   Trouble *trouble_out = nullptr);
+                   double *go, cudaStream_t s, const unsigned long long *unst = nullptr,
+                   unsigned long long *unst_out = nullptr);
 template <typename T>
 void launch_import(int mode, const Phys<T> &P, const double *fi, const double *gi, void *f,
                    void *g, cudaStream_t s);
@@ -384,7 +378,7 @@ struct MgHost;  // defined in fcd_mg.cu
 template <typename T>
 MgHost<T> *mg_create(int nx, int ny, int pitch, T *k0, T *psiA, T *psiB, MgCtl *ctl,
                      void *(*alloc)(size_t, void *), void (*release)(void *, void *), void *user,
-                     char *err, size_t errlen, Trouble *trouble, int comp = 0,
+                     char *err, size_t errlen, Bound *bound, int comp = 0,
                      const MgHost<T> *share_coef = nullptr,  // FP64: use its coefficient planes
                      T *psiC = nullptr);                     // third buffer of psi' (single FP32 plane)
 template <typename T>

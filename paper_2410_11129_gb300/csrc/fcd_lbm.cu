@@ -682,11 +682,12 @@ __device__ __forceinline__ T weight_of(int a) {
 // One plane per blockIdx.z: 27 independent streams of loads and stores.
 template <typename T, int MODE>
 __global__ void __launch_bounds__(256) export_kernel(Phys<T> P, const void *fv, const void *gv, double *fo, double *go,
-                                                     const Trouble *trouble, Trouble *trouble_out) {
+                                                     const unsigned long long *unst,
+                                                     unsigned long long *unst_out) {
     using S = typename StoreT<MODE>::type;
     const int q = blockIdx.z;
-    if (trouble_out && blockIdx.x == 0 && blockIdx.y == 0 && q == 0 && threadIdx.x == 0 && threadIdx.y == 0)
-        *trouble_out = *trouble;
+    if (unst_out && blockIdx.x == 0 && blockIdx.y == 0 && q == 0 && threadIdx.x == 0 && threadIdx.y == 0)
+        *unst_out = *unst;
     double *out = q < 9 ? fo : go;
     if (!out) return;
     out += (long long)(q < 9 ? q : q - 9) * P.nx * P.ny;
@@ -880,9 +881,9 @@ void launch_init(int mode, const Phys<T> &P, double u_max, double r1, double r2,
 
 template <typename T>
 void launch_export(int mode, const Phys<T> &P, const void *f, const void *g, double *fo, double *go,
-                   cudaStream_t s, const Trouble *trouble, Trouble *trouble_out) {
+                   cudaStream_t s, const unsigned long long *unst, unsigned long long *unst_out) {
     const dim3 b(32, 8), gr((P.nx + 31) / 32, (P.ny + 31) / 32, 27);
-    FCD_MODE_SWITCH(mode, T, (export_kernel<T, M><<<gr, b, 0, s>>>(P, f, g, fo, go, trouble, trouble_out)));
+    FCD_MODE_SWITCH(mode, T, (export_kernel<T, M><<<gr, b, 0, s>>>(P, f, g, fo, go, unst, unst_out)));
 }
 
 template <typename T>
@@ -938,7 +939,8 @@ void launch_phi3_to_f64(const T *p1, const T *p2, int nx, int ny, int pitch, dou
     template void launch_init<T>(int, const Phys<T> &, double, double, double, double, double, \
                                  double, void *, void *, T *, cudaStream_t);                   \
     template void launch_export<T>(int, const Phys<T> &, const void *, const void *, double *, \
-                                   double *, cudaStream_t, const Trouble *, Trouble *);        \
+                                   double *, cudaStream_t, const unsigned long long *,         \
+                                   unsigned long long *);                                      \
     template void launch_import<T>(int, const Phys<T> &, const double *, const double *,       \
                                    void *, void *, cudaStream_t);                              \
     template void launch_plane_to_f64<T>(const T *, int, int, int, double *, cudaStream_t);    \

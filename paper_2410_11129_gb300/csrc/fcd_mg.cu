@@ -1125,7 +1125,7 @@ struct MgHost {
     // the one-kernel form: its first single-block level, shared memory, blocks
     int solve_lc = 0, solve_blocks = 0, sms = 0;
     TC *corr = nullptr;  // its lattice planes: residual, correction (two), k
-    Trouble *trouble = nullptr;
+    Bound *bound = nullptr;
     size_t solve_smem = 0;
 };
 
@@ -1233,7 +1233,7 @@ cudaError_t mg_solve(MgHost<T> *m, T H0c, T H0s, cudaStream_t s) {
     A.H0c = H0c;
     A.H0s = H0s;
     A.ctl = m->ctl;
-    A.trouble = m->trouble;
+    A.bound = m->bound;
     A.form_coef = m->coef_shared ? 0 : 1;
     const size_t ps = (size_t)m->L0.pitch * m->L0.ny;
     A.r0 = m->corr;
@@ -1248,9 +1248,9 @@ cudaError_t mg_solve(MgHost<T> *m, T H0c, T H0s, cudaStream_t s) {
 template <typename T>
 MgHost<T> *mg_create(int nx, int ny, int pitch, T *k0, T *psiA, T *psiB, MgCtl *ctl,
                      void *(*alloc)(size_t, void *), void (*release)(void *, void *), void *user,
-                     char *err, size_t errlen, Trouble *trouble, int comp, const MgHost<T> *share_coef, T *psiC) {
+                     char *err, size_t errlen, Bound *bound, int comp, const MgHost<T> *share_coef, T *psiC) {
     MgHost<T> *m = new MgHost<T>();
-    m->trouble = trouble;
+    m->bound = bound;
     m->alloc = alloc;
     m->release = release;
     m->user = user;
@@ -1829,7 +1829,7 @@ void mg_psi_io(MgHost<double> *m, int op, double *plane, double *prev, cudaStrea
 #define FCD_MG_INST(T)                                                                          \
     template MgHost<T> *mg_create<T>(int, int, int, T *, T *, T *, MgCtl *,                     \
                                      void *(*)(size_t, void *), void (*)(void *, void *), void *, \
-                                     char *, size_t, Trouble *, int, const MgHost<T> *, T *);   \
+                                     char *, size_t, Bound *, int, const MgHost<T> *, T *);     \
     template void mg_destroy<T>(MgHost<T> *);                                                   \
     template int mg_levels<T>(const MgHost<T> *);                                               \
     template void mg_set_rhs<T>(MgHost<T> *, const T *);                                        \

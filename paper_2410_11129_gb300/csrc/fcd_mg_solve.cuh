@@ -87,14 +87,14 @@ struct SolveArgs {
     int nl, lc;
     T H0c, H0s;
     MgCtl *ctl;
-    Trouble *trouble;       // the context's: a barrier that gives up leaves its mark there
+    Bound *bound;           // the context's: a barrier that gives up leaves its mark there
     int form_coef;          // FP64: form the node coefficients (else another solve of this k has)
     TC *r0, *eA, *eB, *k0;  // lattice planes of the correction: residual, e (two buffers), k
 };
 
 // Grid barrier of a cooperative launch; ctl->bar counts arrivals from the
-// solve's reset on. False once a barrier has timed out (tr: the context's record).
-__device__ __forceinline__ bool grid_barrier(MgCtl *c, Trouble *tr, unsigned polls, unsigned &arrivals) {
+// solve's reset on. False once a barrier has timed out.
+__device__ __forceinline__ bool grid_barrier(MgCtl *c, Bound *bound, unsigned polls, unsigned &arrivals) {
     __shared__ int ok;
     arrivals += gridDim.x;
     __syncthreads();
@@ -106,10 +106,10 @@ __device__ __forceinline__ bool grid_barrier(MgCtl *c, Trouble *tr, unsigned pol
         while (true) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&c->bar) : "memory");
             if (seen >= arrivals) break;
-            if (++spin >= polls || ((spin & 1023u) == 0 && *(volatile int *)&tr->stuck)) {
+            if (++spin >= polls || ((spin & 1023u) == 0 && *(volatile int *)&bound->stuck)) {
                 good = false;
-                atomicExch(&tr->stuck, 1);
-                atomicExch(&c->stuck, 1);
+                atomicExch(&bound->stuck, 1);
+                *(volatile int *)bound->told = 1;  // read after the stream has been synchronised
                 break;
             }
         }
@@ -802,11 +802,8 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
     __shared__ double norm;
     MgCtl *const ctl = A.ctl;
     const int tid = threadIdx.x, nl = A.nl, lc = A.lc;
-    if (A.trouble->stuck) {  // an earlier solve's barrier timed out
-        if (blockIdx.x == 0 && tid == 0) ctl->stuck = 1;
-        return;
-    }
-    const unsigned polls = A.trouble->polls;
+    if (A.bound->stuck) return;  // an earlier solve's barrier timed out
+    const unsigned polls = A.bound->polls;
     if (tid < nl) L[tid] = A.lv[tid];
     __syncthreads();
     if (tid == 0) {
@@ -847,7 +844,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
             for (int q = 1; q < SOLVE_THREADS / 32; q++) mx = max(mx, wmax[q]);
             if (mx > 0) atomic_max_nonneg(&ctl->norm_slot[heads & 3], max_value(mx, T(0)));
         }
-        if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
+        if (!grid_barrier(ctl, A.bound, polls, arrivals)) return;
         if (tid == 0) {
             norm = __longlong_as_double((long long)__ldcg(&ctl->norm_slot[heads & 3]));
             if (blockIdx.x == 0) ctl->norm_slot[(heads + 2) & 3] = 0ull;  // two heads on, two barriers away
@@ -873,21 +870,21 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
             const bool setup = vcycles++ == 0;
             for (int l = 1; l < lc; l++) {
                 fv_phase<0>(fv, L[l], L[l + 1], NU_PRE);
-                if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
+                if (!grid_barrier(ctl, A.bound, polls, arrivals)) return;
                 restrict_phase(L[l], L[l + 1], setup);
-                if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
+                if (!grid_barrier(ctl, A.bound, polls, arrivals)) return;
             }
             if (blockIdx.x == 0) bottom_phase(bottom, B, L, lc, nl, setup);
             for (int l = lc - 1; l >= 1; l--) {
-                if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
+                if (!grid_barrier(ctl, A.bound, polls, arrivals)) return;
                 fv_phase<1>(fv, L[l], L[l + 1], NU_POST);
             }
         }
-        if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
+        if (!grid_barrier(ctl, A.bound, polls, arrivals)) return;
         each_tile(sw, SOLVE_WORKERS, [&](int bx, int by) { sweep_tile<T>(wt[sw].s, A, L[1], nullptr, A.eA, TC(1), bx, by, sw, st); });
-        if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
+        if (!grid_barrier(ctl, A.bound, polls, arrivals)) return;
         each_tile(sw, SOLVE_WORKERS, [&](int bx, int by) { sweep_tile<T>(wt[sw].s, A, L[1], A.eA, A.eB, over, bx, by, sw, st); });
-        if (!grid_barrier(ctl, A.trouble, polls, arrivals)) return;
+        if (!grid_barrier(ctl, A.bound, polls, arrivals)) return;
         iter++;
     }
     if (blockIdx.x == 0 && tid == 0) {

@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(FIN) obs_final(int nx, const double *col, ObsO
     if (tail.pack) {
         tail.pack->o = r;
         tail.pack->brk = *tail.brk;
-        tail.pack->trouble = *tail.trouble;
+        tail.pack->unst = *tail.unst;
         tail.pack->ctl = *tail.ctl;
     }
 }

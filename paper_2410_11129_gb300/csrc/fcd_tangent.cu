@@ -164,7 +164,6 @@ __global__ void __launch_bounds__(TOB) tangent_obs_final(int nx, const DualT *ex
     out->lx = lx.v;
     out->ly = ly.v;
     out->nonconv = 0;
-    out->stuck = ctls.trouble->stuck;
     for (int q = 0; q < NT; q++) {
         out->dT_o[q] = To.d[q];
         out->doverlap[q] = tot[1 + q];
