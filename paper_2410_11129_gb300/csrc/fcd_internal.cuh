@@ -330,7 +330,7 @@ template <typename T>
 void launch_collide_batch(int mode, int tile_h, const BatchLbm<T> *tab, const BatchTile *tiles,
                           int ntiles, cudaStream_t s);
 // tile_h: rows per collide tile, 4 or 8 for the FP32 forms (the same
-// arithmetic per node; the faster one depends on the grid); FP64 uses 8.
+// arithmetic per node; the faster one depends on the grid); FP64 uses 4 or 2.
 template <typename T>
 void launch_collide(int mode, int tile_h, const LbmArgs<T> &a, cudaStream_t s);
 void launch_collide_tangent(const LbmArgs<double, DualT> &a, cudaStream_t s);
@@ -357,8 +357,6 @@ void launch_import(int mode, const Phys<T> &P, const double *fi, const double *g
                    void *g, cudaStream_t s);
 template <typename T>
 void launch_plane_to_f64(const T *src, int nx, int ny, int pitch, double *dst, cudaStream_t s);
-template <typename T>
-void launch_plane_from_f64(const double *src, int nx, int ny, int pitch, T *dst, cudaStream_t s);
 template <typename T>
 void launch_phi3_to_f64(const T *p1, const T *p2, int nx, int ny, int pitch, double *dst,
                         cudaStream_t s);
@@ -433,8 +431,6 @@ void mg_reset_scaled(MgCtl *ctl, const unsigned long long *scale_bits, double to
 void mg_tangent_rhs(MgHost<double> *m, const double *dk, double H0c, double H0s, double dH0c,
                     double dH0s, double *rhs, unsigned long long *rmax_bits, cudaStream_t s);
 void mg_psi_io(MgHost<double> *m, int op, double *plane, double *prev, cudaStream_t s);
-template <typename T>
-int mg_levels(const MgHost<T> *m);
 // Batched solves of many FP32 hierarchies (one per instance; fields and
 // control blocks stay the instances' own): the body of the loop that runs until
 // every solve is done (launch_phase_open_batch opens them).

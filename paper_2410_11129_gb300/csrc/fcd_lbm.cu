@@ -90,7 +90,7 @@ __device__ __forceinline__ void phase_tile(const Phys<T> &P, const void *gv, T *
                 two_sum(a, __fadd_rn(__fsub_rn(2.f * l, pl), e), hh, ll);
                 psi[m] = hh;
                 psi[L + m] = ll;
-            } else {
+            } else if constexpr (sizeof(T) == 8) {  // one FP32 plane: phase_open
                 const T now = ps_[r][0], before = pp_[r][0];
                 prev[m] = now;
                 psi[m] = T(2) * now - before;
@@ -731,14 +731,6 @@ __global__ void plane_to_f64(const T *src, int nx, int ny, int pitch, double *ds
     dst[(long long)y * nx + x] = double(src[(long long)y * pitch + x]);
 }
 
-template <typename T>
-__global__ void plane_from_f64(const double *src, int nx, int ny, int pitch, T *dst) {
-    int x = blockIdx.x * blockDim.x + threadIdx.x;
-    int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= nx || y >= ny) return;
-    dst[(long long)y * pitch + x] = T(src[(long long)y * nx + x]);
-}
-
 // psi' of a level-0 buffer in the FP64 exchange layout, and back (FP32: the
 // hi + lo pair of planes; FP64: one plane).
 template <typename T>
@@ -821,11 +813,11 @@ void launch_collide(int mode, int tile_h, const LbmArgs<T> &a, cudaStream_t s) {
             if (a.open_x) collide_kernel<T, MODE_FP64, true, 4><<<gr, b, 0, s>>>(a);
             else collide_kernel<T, MODE_FP64, false, 4><<<gr, b, 0, s>>>(a);
         }
-        return;
+    } else {
+        dim3 b(TX, TY), gr = grid2(a.P.nx, a.P.ny, b);
+        if (a.open_x) FCD_MODE_SWITCH(mode, T, (collide_kernel<T, M, true><<<gr, b, 0, s>>>(a)));
+        else FCD_MODE_SWITCH(mode, T, (collide_kernel<T, M, false><<<gr, b, 0, s>>>(a)));
     }
-    dim3 b(TX, TY), gr = grid2(a.P.nx, a.P.ny, b);
-    if (a.open_x) FCD_MODE_SWITCH(mode, T, (collide_kernel<T, M, true><<<gr, b, 0, s>>>(a)));
-    else FCD_MODE_SWITCH(mode, T, (collide_kernel<T, M, false><<<gr, b, 0, s>>>(a)));
 }
 
 template <typename T>
@@ -900,12 +892,6 @@ void launch_plane_to_f64(const T *src, int nx, int ny, int pitch, double *dst, c
 }
 
 template <typename T>
-void launch_plane_from_f64(const double *src, int nx, int ny, int pitch, T *dst, cudaStream_t s) {
-    dim3 b(32, 8);
-    plane_from_f64<T><<<grid2(nx, ny, b), b, 0, s>>>(src, nx, ny, pitch, dst);
-}
-
-template <typename T>
 void launch_psi_to_f64(const MgCtl *ctl, const T *A, const T *B, const T *C, int nx, int ny, int pitch, double *dst,
                        cudaStream_t s) {
     dim3 b(32, 8);
@@ -944,7 +930,6 @@ void launch_phi3_to_f64(const T *p1, const T *p2, int nx, int ny, int pitch, dou
     template void launch_import<T>(int, const Phys<T> &, const double *, const double *,       \
                                    void *, void *, cudaStream_t);                              \
     template void launch_plane_to_f64<T>(const T *, int, int, int, double *, cudaStream_t);    \
-    template void launch_plane_from_f64<T>(const double *, int, int, int, T *, cudaStream_t);  \
     template void launch_phi3_to_f64<T>(const T *, const T *, int, int, int, double *,         \
                                         cudaStream_t);                                         \
     template void launch_psi_to_f64<T>(const MgCtl *, const T *, const T *, const T *, int, int, int, \

@@ -1469,9 +1469,6 @@ void mg_cycle_twogrid(MgHost<float> *m, float H0c, float H0s, cudaStream_t s) {
 
 int mg_kernels_per_cycle(const MgHost<float> *m) { return 2 + 3 * (m->lc - 1); }  // after the head
 
-template <typename T>
-int mg_levels(const MgHost<T> *m) { return m->nl; }
-
 // ------------------------------------------------------------ batched solves
 // The potential solves of many FP32 channels driven by one fixed set of
 // kernels: each kernel runs over a work list of (instance, tile) entries that
@@ -1831,7 +1828,6 @@ void mg_psi_io(MgHost<double> *m, int op, double *plane, double *prev, cudaStrea
                                      void *(*)(size_t, void *), void (*)(void *, void *), void *, \
                                      char *, size_t, Bound *, int, const MgHost<T> *, T *);     \
     template void mg_destroy<T>(MgHost<T> *);                                                   \
-    template int mg_levels<T>(const MgHost<T> *);                                               \
     template void mg_set_rhs<T>(MgHost<T> *, const T *);                                        \
     template bool mg_one_kernel<T>(const MgHost<T> *);                                          \
     template cudaError_t mg_solve<T>(MgHost<T> *, T, T, cudaStream_t);                          \
