@@ -8,6 +8,7 @@
 // collide-stream. fcd_step(n)
 // launches n such graphs; nothing synchronises with the host in between.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstddef>
@@ -271,6 +272,7 @@ struct Engine : fcd_ctx {
     }
 
     ~Engine() override {
+        count_legacy(false);
         if (stream) cudaStreamSynchronize(stream);
         cudaDeviceSynchronize();
         for (int a = 0; a < 2; a++)
@@ -712,25 +714,36 @@ struct Engine : fcd_ctx {
     // The legacy default stream orders itself against the branches of every graph
     // in the process, so that a branched step graph launched there costs more the
     // more contexts there are (96 contexts in turn: 174 us per step, 129 without
-    // branches). Such graphs therefore run on streams of the context that keep
-    // that stream's order: one step on a blocking stream, which CUDA orders
-    // against it at no cost; several on a non-blocking one between two events,
-    // because many graphs in a row on a blocking stream cost about as much as on
-    // the legacy stream itself (96 contexts, 10 steps a call: 125 us, legacy 142, with
-    // events 56). us per step, contexts of 1600 x 200 in turn, unbranched -> branched
-    // on the legacy stream -> here: 1 context 56 -> 45 -> 45; 24 contexts, one step a
-    // call 82 -> 95 -> 25 (they overlap), 10 steps 81 -> 95 -> 47; 96 contexts
-    // 129 -> 174 -> 86 and 92 -> 142 -> 56.
+    // branches). Where other contexts step there too, such graphs therefore run on
+    // streams of the context that keep that stream's order: one step on a blocking
+    // stream, which CUDA orders against it; several, as for a context alone, on a
+    // non-blocking one between two events, because many graphs in a row on a blocking
+    // stream cost about as much as on the legacy stream itself (96 contexts, 10 steps
+    // a call: 125 us, legacy 142, with events 56). A context alone takes its single
+    // steps on the legacy stream itself: between the caller's own operations there a
+    // blocking stream costs 2 to 3 us (55.3 -> 58.4 us with a flush in front of every
+    // step). us per step, contexts of 1600 x 200 in turn, unbranched -> branched on
+    // the legacy stream -> here: 1 context 56 -> 45 -> 45; 24 contexts, one step a call
+    // 82 -> 95 -> 25 (they overlap), 10 steps 81 -> 95 -> 47; 96 contexts 129 -> 174 ->
+    // 86 and 92 -> 142 -> 56.
+    // legacy_users only counts: the routes give the same bits in the same order.
+    static inline std::atomic<int> legacy_users{0};
+    bool legacy_user = false;
+    void count_legacy(bool on) {
+        if (on != legacy_user) legacy_users += on ? 1 : -1;
+        legacy_user = on;
+    }
     fcd_status do_step(long n) override {
         if (n < 0) return fail(FCD_EINVAL, "negative step count");
         const bool legacy = use_graph && turns() && (stream == nullptr || stream == cudaStreamLegacy);
         const bool fork = legacy && n > 1;
+        count_legacy(legacy);
         cudaStream_t s = stream;
         if (fork) {
             s = cap;
             CK(cudaEventRecord(fork_ev, stream));
             CK(cudaStreamWaitEvent(s, fork_ev, 0));
-        } else if (legacy) {
+        } else if (legacy && legacy_users > 1) {
             if (!beside) CK(cudaStreamCreateWithFlags(&beside, cudaStreamDefault));
             s = beside;
         }

@@ -57,11 +57,16 @@ def test_legacy_stream_keeps_its_order(calls, open_x):
         ch.close()
 
 
-def test_a_synchronised_legacy_stream_has_no_step_left():
-    """A caller that moves a context to another stream after synchronising."""
+@pytest.mark.parametrize("others", [0, 1])
+def test_a_synchronised_legacy_stream_has_no_step_left(others):
+    """A caller that moves a context to another stream after synchronising, alone
+    on the default stream or not (its single steps take another route then)."""
     import torch
     from paper_2410_11129_gb300 import fcd
     a, b = fcd.Channel(_cfg(0)), fcd.Channel(_cfg(0))
+    more = [fcd.Channel(_cfg(1)) for _ in range(others)]
+    for ch in more:
+        ch.step(1)
     s = torch.cuda.Stream()
     for _ in range(20):
         a.step(1)
@@ -74,5 +79,5 @@ def test_a_synchronised_legacy_stream_has_no_step_left():
     b.step(80)
     for x, y in zip(a.populations(), b.populations()):
         assert np.array_equal(x, y)
-    a.close()
-    b.close()
+    for ch in [a, b] + more:
+        ch.close()
