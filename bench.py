@@ -41,10 +41,10 @@ COLLIDE_BYTES_PER_NODE_F32 = 240
 # rows (null once the source changes). On 1600x200 the 37 MB of output stays in
 # L2 when the launch ends, so only the reads reach DRAM inside the launch.
 NCU_TRAFFIC = {
-    ("b5b068562d18f977", "1600x200", 4): 38430464 + 242432,
-    ("b5b068562d18f977", "1600x200", 8): 38433536 + 257792,
-    ("b5b068562d18f977", "9600x1200", 4): 1383248896 + 1206289152,
-    ("b5b068562d18f977", "9600x1200", 8): 1383520256 + 1206574080,
+    ("a7d7f6085114d87d", "1600x200", 4): 38438400 + 276480,
+    ("a7d7f6085114d87d", "1600x200", 8): 38439680 + 279296,
+    ("a7d7f6085114d87d", "9600x1200", 4): 1383007232 + 1204817664,
+    ("a7d7f6085114d87d", "9600x1200", 8): 1383383808 + 1205111296,
 }
 
 
