@@ -32,6 +32,7 @@ using namespace fcd;
 namespace {
 
 constexpr int SIDE_SOLVES = 8;  // one-kernel solves of a batch that run side by side
+constexpr long long SHARE_NODES = 3000000;  // nodes of other instances per share (fcd_batch_create)
 
 struct Group {
     int mode = MODE_FP32;
@@ -487,12 +488,23 @@ fcd_status fcd_batch_create(const fcd_params *params, int n, fcd_batch **out) {
         b->inst.push_back(c);
         fcd_set_stream(c, s);
     }
-    // one-kernel solves of several instances run side by side; the other
-    // instances' kernels need no share kept for them (one 800 x 100 FP64 channel
-    // beside seven of one FP32 plane: 19 blocks before, 130 now)
-    const int solves = (int)std::count_if(b->inst.begin(), b->inst.end(), engine_one_kernel);
+    // One-kernel solves of several instances run side by side, each on its share of
+    // the SMs, whose blocks it fills for as long as it takes. The other instances
+    // need SMs in proportion to their work: about one share for every SHARE_NODES
+    // nodes, which take 0.3 ms per step, as long as such a solve. Measured, us per
+    // step at shares of 1, 2, 3, 4 and 8, this rule's one in brackets: one 800 x 100
+    // FP64 channel beside seven of one FP32 plane (2.1 M nodes) 700, [726], 778, 871,
+    // 1130; beside 23 (7 M) 1091, 927, [965], 1058, 1288; beside 60 (18 M) 2016, 1876,
+    // 1774, 1754, 1685 [7: 1690]; four beside 20 (6 M) 2656, 1912, 1612, 1503, 1510 [6: 1423].
+    int solves = 0;
+    long long others = 0;
+    for (size_t i = 0; i < b->inst.size(); i++) {
+        if (engine_one_kernel(b->inst[i])) solves++;
+        else others += (long long)params[i].nx * params[i].ny;
+    }
+    const int share = (int)std::min<long long>(SIDE_SOLVES, solves + (others + SHARE_NODES / 2) / SHARE_NODES);
     for (fcd_ctx *c : b->inst)
-        if (engine_one_kernel(c)) engine_share(c, std::min(solves, SIDE_SOLVES));
+        if (engine_one_kernel(c)) engine_share(c, share);
     // group the periodic FP32 instances by storage form and level-0 form of the
     // potential (one FP32 plane or the hi + lo pair), and split each such set
     // into about one group per GROUP_NODES lattice nodes (at most MAX_SPLIT),
