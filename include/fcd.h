@@ -87,7 +87,9 @@ typedef struct {
     double u_max;          /* centre-line speed of the body-force-driven channel flow */
     int ferro_phase;       /* 1 core, 2 shell, 0 none: selects the Eq. 41 branch */
     int precision;         /* fcd_precision: storage and arithmetic of the populations */
-    double mag_tol;        /* potential solve target ||L psi||_inf / H0 per step */
+    double mag_tol;        /* potential solve target ||L psi||_inf / H0 per step; an FP64 solve
+                            * goes on to a fraction of it (1/2 to 1/256), because the error
+                            * of psi' behind a residual that just meets it can be large */
     int mag_max_iter;      /* multigrid V-cycle cap per solve */
     double eps_n;          /* regulariser of n = grad phi / (|grad phi| + eps_n) */
     int open_x;            /* 0: periodic channel driven by a body force (u_max).

@@ -9,10 +9,15 @@
 // cycle are separated by grid barriers of about 1.5 us, every block takes the
 // same decisions from the same norm, and nothing returns to the host or to a
 // graph node until the solve ends. Measured per step at tolerance 1e-10: 200 x 40
-// 622 -> 207 us (12.0 -> 8.0 residuals), 800 x 100 827 -> 307 us (11.5 -> 7.7);
-// the FP32 pair on 402 x 123 at 1e-5: step 79 -> 42 us. Bound now by the chain of
-// phases: barriers a quarter, the FP64 residual a fifth (57 cycles per operation
-// of a warp), the single-block levels a fifth.
+// 622 -> 245 us (12.0 -> 9.4 residuals), 800 x 100 827 -> 390 us (11.5 -> 9.9), both to
+// errors no larger than before (stop_factor); the FP32 pair on 402 x 123 at 1e-5:
+// step 79 -> 42 us. Bound by the chain of phases. Clock stamps of one block on
+// 800 x 100: barriers with the wait for the slowest block a third, the grid-wide
+// coarse levels a quarter, the residual (FP64: 57 cycles per operation of a warp)
+// and the single-block levels a sixth each, the lattice sweeps a tenth; on 200 x 40:
+// single-block levels 43%, barriers 23%, residual 18%, sweeps 14%. 6% of the issue
+// slots are used. The FP64 form spills (128 registers of 512 threads: 192 bytes of
+// stack, the second node's coefficients in the residual).
 //
 // A cycle is a defect correction: the lattice residual in the context's type
 // (after which its norm decides) and its restriction; the coarse levels,
@@ -20,8 +25,7 @@
 // memory for the whole solve (their coefficients are formed once); then the
 // lattice's correction e = interpolated level-1 correction + two sweeps, in FP32
 // like every correction, which the next residual adds to psi'. FP64 arithmetic
-// (1/58 of FP32 here) is left in the residual alone, whose norm, against the
-// unchanged tolerance, is what defines the result. The two sweeps are separate
+// (1/58 of FP32 here) is left in the residual alone, whose norm decides. The two sweeps are separate
 // phases, so the second sees its neighbours' new values: a tile's second sweep
 // against the same frozen ring gains nothing (numpy prototype of the 800 x 100
 // channel: 0.27 per cycle with one sweep, 0.29 with two frozen, 0.165 with two
@@ -29,7 +33,7 @@
 //
 // Values that another block wrote in this kernel are read past the L1 cache
 // (__ldcg). Every wait is bounded: a barrier that does not complete marks the
-// control block and ends the kernel.
+// context (Bound) and ends the kernel.
 #pragma once
 
 namespace fcd {
@@ -47,7 +51,7 @@ static_assert(SOLVE_WORKERS <= 15, "one named barrier per worker, barrier 0 is t
 // 0.140, 0.126, 0.130; 200 x 40 0.163, 0.135, 0.126, 0.141; 400 x 122 0.209, 0.178,
 // 0.138, 0.125; chi = 5 0.316, 0.292, 0.267, 0.241. Not for an odd number of rows,
 // whose cells of three at the wall it overshoots (400 x 123: 0.210, at 1.05 0.295),
-// nor where rows are not merged. Measured, 1 -> 1.08: residuals per solve 8.5 ->
+// nor where rows are not merged. Measured with solves that stop at the tolerance, 1 -> 1.08: residuals per solve 8.5 ->
 // 7.6 on 800 x 100 at 1e-10 (485 -> 432 us per step) and 2.73 -> 2.44 at 1e-5 (180 ->
 // 170), 9.0 -> 8.0 on 200 x 40 (270 -> 241): no slower at any tolerance from 1e-4 to
 // 1e-12. Going straight to V-cycles (no two-grid cycles first) takes 457 us
