@@ -161,7 +161,8 @@ fcd_status fcd_solve_magnetic(fcd_ctx *ctx, double tol, int max_iter, int *iters
 /* Observables of the current state (Eqs. 38, 42; breakup of Sec. 2.5). Synchronous. */
 fcd_status fcd_observables(fcd_ctx *ctx, fcd_obs *out);
 
-/* Copy one field (fcd_field) into dst (nx*ny doubles, host or device). Synchronous. */
+/* Copy one field (fcd_field) into dst (nx*ny doubles, host or device; FCD_ECUDA for
+ * a device buffer that ends before them, here and below). Synchronous. */
 fcd_status fcd_get_field(fcd_ctx *ctx, int which, double *dst, size_t n);
 
 /* Populations and perturbation potential psi' in the FP64 exchange layout
