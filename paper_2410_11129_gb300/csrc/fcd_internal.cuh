@@ -182,6 +182,7 @@ struct Bound {
     int *told;       // the same as stuck in pinned host memory, for every call that delivers results
 };
 constexpr unsigned BARRIER_POLLS = 1u << 24;  // seconds
+
 // Level-0 buffer 0, 1 or 2 of a, b, c.
 template <typename T>
 __host__ __device__ __forceinline__ T *psi_buffer(int i, T *a, T *b, T *c) { return i == 0 ? a : (i == 1 ? b : c); }

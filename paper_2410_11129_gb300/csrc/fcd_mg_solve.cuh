@@ -25,11 +25,11 @@
 // memory for the whole solve (their coefficients are formed once); then the
 // lattice's correction e = interpolated level-1 correction + two sweeps, in FP32
 // like every correction, which the next residual adds to psi'. FP64 arithmetic
-// (1/58 of FP32 here) is left in the residual alone, whose norm decides. The two sweeps are separate
-// phases, so the second sees its neighbours' new values: a tile's second sweep
-// against the same frozen ring gains nothing (numpy prototype of the 800 x 100
-// channel: 0.27 per cycle with one sweep, 0.29 with two frozen, 0.165 with two
-// refreshed).
+// (1/58 of FP32 here) is left in the residual alone, whose norm decides. The two
+// sweeps are separate phases, so the second sees its neighbours' new values: a tile's
+// second sweep against the same frozen ring gains nothing (numpy prototype of the
+// 800 x 100 channel: 0.27 per cycle with one sweep, 0.29 with two frozen, 0.165 with
+// two refreshed).
 //
 // Values that another block wrote in this kernel are read past the L1 cache
 // (__ldcg). Every wait is bounded: a barrier that does not complete marks the
@@ -51,11 +51,11 @@ static_assert(SOLVE_WORKERS <= 15, "one named barrier per worker, barrier 0 is t
 // 0.140, 0.126, 0.130; 200 x 40 0.163, 0.135, 0.126, 0.141; 400 x 122 0.209, 0.178,
 // 0.138, 0.125; chi = 5 0.316, 0.292, 0.267, 0.241. Not for an odd number of rows,
 // whose cells of three at the wall it overshoots (400 x 123: 0.210, at 1.05 0.295),
-// nor where rows are not merged. Measured with solves that stop at the tolerance, 1 -> 1.08: residuals per solve 8.5 ->
-// 7.6 on 800 x 100 at 1e-10 (485 -> 432 us per step) and 2.73 -> 2.44 at 1e-5 (180 ->
-// 170), 9.0 -> 8.0 on 200 x 40 (270 -> 241): no slower at any tolerance from 1e-4 to
-// 1e-12. Going straight to V-cycles (no two-grid cycles first) takes 457 us
-// per step on 800 x 100 and 251 on 200 x 40.
+// nor where rows are not merged. Measured with solves that stop at the tolerance,
+// 1 -> 1.08: residuals per solve 8.5 -> 7.6 on 800 x 100 at 1e-10 (485 -> 432 us per
+// step) and 2.73 -> 2.44 at 1e-5 (180 -> 170), 9.0 -> 8.0 on 200 x 40 (270 -> 241): no
+// slower at any tolerance from 1e-4 to 1e-12. Going straight to V-cycles (no two-grid
+// cycles first) takes 457 us per step on 800 x 100 and 251 on 200 x 40.
 constexpr TC OVER = TC(1.08);
 
 // The FP32 residual and correction are in units of a power of two near the
@@ -806,10 +806,12 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) mg_solve_kernel(const SolveA
     __shared__ double norm;
     MgCtl *const ctl = A.ctl;
     const int tid = threadIdx.x, nl = A.nl, lc = A.lc;
-    if (A.bound->stuck) return;  // an earlier solve's barrier timed out
+    __shared__ int given_up;  // one answer for the block: a solve beside this one may give up right now
     const unsigned polls = A.bound->polls;
     if (tid < nl) L[tid] = A.lv[tid];
+    if (tid == 0) given_up = *(volatile int *)&A.bound->stuck;
     __syncthreads();
+    if (given_up) return;  // a barrier of this context timed out
     if (tid == 0) {
         int at = 0;
         for (int l = lc; l < nl; l++) {
